@@ -638,11 +638,25 @@ __global__ void __launch_bounds__(256) forward_affine_kernel(const float* __rest
 // maxdiff, ctrl[3] = number of active samples in the hp phase (the tail of idx); ctrl[CTRL_SWEEP] = sweeps finished in
 // this block, ctrl[CTRL_TAU] / ctrl[CTRL_SWITCH] = bits of tau and of the escalation threshold.
 // ------------------------------------------------------------------------------------------------
-constexpr int CTRL_WORDS = 16, CTRL_LABEL_FLAG = 5, CTRL_SWEEP = 8, CTRL_TAU = 9, CTRL_SWITCH = 10;
+constexpr int CTRL_WORDS = 16, CTRL_LABEL_FLAG = 5, CTRL_SWEEP = 8, CTRL_TAU = 9, CTRL_SWITCH = 10, CTRL_SEQ = 11;
+// Words of the pinned host array the last sweep-control kernel of a sweep fills (the device error word among them);
+// HOST_SEQ is stored after all others and counts the sweeps of this model, so the host can poll it.
+enum { HOST_ACTIVE, HOST_BAD, HOST_ERR, HOST_TOP, HOST_TWO_TERM, HOST_LABEL, HOST_SEQ, HOST_WORDS = 8 };
+__device__ __forceinline__ void report_to_host(int* ctrl, const int* err, int* host, int active, int bad, int top_bits, int two_term) {
+  volatile int* h = host;
+  h[HOST_ACTIVE] = active;
+  h[HOST_BAD] = bad;
+  h[HOST_ERR] = *reinterpret_cast<const volatile int*>(err);
+  h[HOST_TOP] = top_bits;
+  h[HOST_TWO_TERM] = two_term;
+  __threadfence_system();
+  h[HOST_SEQ] = ++ctrl[CTRL_SEQ];
+}
 // One CTA of 256 threads; the order of the surviving samples is kept (stable compaction), single-term samples first.
 __global__ void __launch_bounds__(256)
 jacobi_finalize_kernel(float* __restrict__ maxdiff, int* __restrict__ idx, int* __restrict__ idx_tmp,
-                       int* __restrict__ phase, int* __restrict__ ctrl, int* __restrict__ iters_sample) {
+                       int* __restrict__ phase, int* __restrict__ ctrl, int* __restrict__ iters_sample, const int* __restrict__ err,
+                       int* __restrict__ host) {
   __shared__ int s_cnt[2][8];
   __shared__ float s_top[8];
   __shared__ int s_flag[2][8];
@@ -709,6 +723,7 @@ jacobi_finalize_kernel(float* __restrict__ maxdiff, int* __restrict__ idx, int* 
     ctrl[2] = anynan ? 0x7fc00000 : __float_as_int(top);
     ctrl[3] = base1;
     ctrl[CTRL_SWEEP] = t;
+    report_to_host(ctrl, err, host, base0 + base1, anybad, ctrl[2], base1);
   }
 }
 
@@ -765,7 +780,7 @@ jacobi_finalize_count_kernel(float* __restrict__ maxdiff, const int* __restrict_
 
 __global__ void __launch_bounds__(256)
 jacobi_finalize_scan_kernel(int* __restrict__ blk_cnt, const float* __restrict__ blk_top, const int* __restrict__ blk_flag,
-                            int* __restrict__ ctrl, int nblk) {
+                            int* __restrict__ ctrl, int nblk, const int* __restrict__ err, int* __restrict__ host) {
   __shared__ int s_w[2][8];
   __shared__ float s_top[8];
   __shared__ int s_flag[8];
@@ -813,6 +828,7 @@ jacobi_finalize_scan_kernel(int* __restrict__ blk_cnt, const float* __restrict__
     ctrl[3] = base1;
     ctrl[7] = base0;                   // two-term survivors start here
     ctrl[CTRL_SWEEP] = ctrl[CTRL_SWEEP] + 1;
+    report_to_host(ctrl, err, host, base0 + base1, ctrl[1], ctrl[2], base1);
   }
 }
 
@@ -836,7 +852,7 @@ jacobi_finalize_scatter_kernel(const int* __restrict__ idx, int* __restrict__ id
 }
 
 __global__ void jacobi_begin_kernel(float* __restrict__ maxdiff, int* __restrict__ idx, int* __restrict__ phase,
-                                    int* __restrict__ ctrl, int B, int start_phase, float tau, float switch_thresh) {
+                                    int* __restrict__ ctrl, int B, int start_phase, float tau, float switch_thresh, int seq) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) {
     maxdiff[b] = 0.f;
     idx[b] = b;
@@ -847,6 +863,7 @@ __global__ void jacobi_begin_kernel(float* __restrict__ maxdiff, int* __restrict
     ctrl[CTRL_SWEEP] = 0;
     ctrl[CTRL_TAU] = __float_as_int(tau);
     ctrl[CTRL_SWITCH] = __float_as_int(switch_thresh);
+    ctrl[CTRL_SEQ] = seq;
   }
 }
 
