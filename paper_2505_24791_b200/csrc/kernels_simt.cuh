@@ -577,6 +577,52 @@ jacobi_update_split_kernel(const float* __restrict__ part, int ksplit, int part_
   if (lane == 0) atomic_max_nonneg(maxdiff + b, df);
 }
 
+// First sweep of a block whose samples all start from u^0 = 0 without class labels: every sample's causal pass sees the
+// same input, so the pass ran for one sample and this kernel applies its head output o [L, 2D] (interleaved, biases
+// included) to all of them:  u[b, l] <- v[b, l] exp(alpha) + mu,  maxdiff[b] = max |u[b] - 0|.  With shift != 0 position l
+// takes row l - 1 and position 0 is copied (TarFlow block), else row l (MLP-based flow: L values of token dimension 1).
+// A warp takes 512 consecutive values of one sample (16 coalesced loads in flight per lane): bound by reading v and
+// writing u once, o stays in L2.
+constexpr int FIRST_CHUNK = 512;
+__global__ void __launch_bounds__(256)
+jacobi_first_update_kernel(const float* __restrict__ o, const float* __restrict__ v, float* __restrict__ u,
+                           float* __restrict__ maxdiff, int B, int L, int D, int reversed, int shift) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int n = L * D, chunks = (n + FIRST_CHUNK - 1) / FIRST_CHUNK, lane = threadIdx.x & 31;
+  const long long unit = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int b = (int)(unit / chunks), e0 = (int)(unit - (long long)b * chunks) * FIRST_CHUNK;
+  if (b >= B) return;
+  const size_t base = (size_t)b * n;
+  float vv[FIRST_CHUNK / 32];
+#pragma unroll
+  for (int k = 0; k < FIRST_CHUNK / 32; ++k) {
+    const int e = e0 + k * 32 + lane;
+    vv[k] = e < n ? v[base + e] : 0.f;
+  }
+  float m = 0.f;
+#pragma unroll
+  for (int k = 0; k < FIRST_CHUNK / 32; ++k) {
+    const int e = e0 + k * 32 + lane;
+    if (e >= n) break;
+    const int tok = e / D, c = e - tok * D, l = tok_index(tok, L, reversed) - shift;
+    float nw = vv[k];
+    if (l >= 0) {
+      const float2 p = __ldg(reinterpret_cast<const float2*>(o + ((size_t)l * D + c) * 2));
+      nw = fmaf(nw, expf(p.y), p.x);
+    }
+    u[base + e] = nw;
+    const float df = fabsf(nw);
+    m = (df > m || df != df) ? df : m;
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {  // NaN-propagating max
+    const float other = __shfl_xor_sync(0xffffffffu, m, off);
+    m = (other > m || other != other) ? other : m;
+  }
+  if (lane == 0) atomic_max_nonneg(maxdiff + b, m);
+}
+
 // Sequential decoding: token t+1 of every sample from the head output of token t (Eq. 5).
 // o: [B, 2D] interleaved.
 __global__ void seq_update_kernel(const float* __restrict__ o, const float* __restrict__ v, float* __restrict__ u,

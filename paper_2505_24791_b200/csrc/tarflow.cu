@@ -1131,11 +1131,20 @@ static int sweep_pass(tf_model* m, int g, int n_slots, const float* u_src, const
   return run_pass<T>(m, g, n_slots, u_src, idx, labels, PASS_JACOBI, v, u_upd, hp);
 }
 
+// the pass over sample 0 alone, its head output (biases included) left in m->o
+template <class T>
+static int first_pass(tf_model* m, int g, const float* u_src, bool hp) {
+  if (m->is_maf) return maf_pass<T>(m, g, 1, u_src, nullptr, 1, nullptr, nullptr, hp, -1);
+  return run_pass<T>(m, g, 1, u_src, nullptr, nullptr, PASS_FORWARD, nullptr, nullptr, hp);
+}
+
 template <class T>
 static int run_jacobi_block(tf_model* m, int g, int B, const int* labels, const float* v, float* u, float tau,
                             int max_iters, const InvOpts& op, int* sweeps_out, int* iters_row) {
   const size_t n = (size_t)B * m->L * m->D, img = (size_t)B * m->cfg.C * m->cfg.H * m->cfg.W;
-  if (op.init_mode == 0) CU_OK(cudaMemsetAsync(u, 0, n * sizeof(float), m->stream));
+  // u^0 = 0 without class labels: the first sweep's pass is the same for every sample and runs for one of them only
+  const bool shared_first = op.init_mode == 0 && labels == nullptr && B > 1;
+  if (op.init_mode == 0) CU_OK(cudaMemsetAsync(u, 0, (shared_first ? n / B : n) * sizeof(float), m->stream));
   else if (op.init_mode == 1) CU_OK(cudaMemcpyAsync(u, v, n * sizeof(float), cudaMemcpyDeviceToDevice, m->stream));
   else TF_TRY(layout(m, const_cast<float*>(op.u0_img) + (size_t)g * img, u, B, 1));
   const bool l2 = m->trace_on && op.ref_img != nullptr && m->trace_l2 != nullptr;
@@ -1153,9 +1162,15 @@ static int run_jacobi_block(tf_model* m, int g, int B, const int* labels, const 
   const int cap = (op.fallback_sweeps > 0 && op.fallback_sweeps < max_iters) ? op.fallback_sweeps : max_iters;
   // everything one sweep launches: the pass over the single-term samples, the pass over the two-term samples, the
   // sweep control (which takes the sweep number and the thresholds from device memory)
-  auto enqueue_sweep = [&](int n_lp, int n_hpp) -> int {
-    if (n_lp > 0) TF_TRY(sweep_pass<T>(m, g, n_lp, u, m->idx, labels, v, u, false));
-    if (n_hpp > 0) TF_TRY(sweep_pass<T>(m, g, n_hpp, u, m->idx + n_lp, labels, v, u, true));
+  auto enqueue_sweep = [&](int n_lp, int n_hpp, bool first) -> int {
+    if (first) {
+      TF_TRY(first_pass<T>(m, g, u, n_hpp > 0));
+      const long long units = (long long)B * ((m->L * m->D + FIRST_CHUNK - 1) / FIRST_CHUNK);
+      LAUNCH_PDL(m, KC_AFFINE, jacobi_first_update_kernel, (unsigned)((units + 7) / 8), 256, 0, m->o, v, u, m->maxdiff, B, m->L, m->D,
+                 m->is_maf ? 0 : g & 1, m->is_maf ? 0 : 1);
+      TF_TRY(check_launch("jacobi_first_update_kernel"));
+    } else if (n_lp > 0) TF_TRY(sweep_pass<T>(m, g, n_lp, u, m->idx, labels, v, u, false));
+    if (!first && n_hpp > 0) TF_TRY(sweep_pass<T>(m, g, n_hpp, u, m->idx + n_lp, labels, v, u, true));
     const int na = n_lp + n_hpp;
     if (na <= FIN_CHUNK || m->fin_code == nullptr) {
       LAUNCH_PDL(m, KC_CTRL, jacobi_finalize_kernel, 1, 256, 0, m->maxdiff, m->idx, m->idx_tmp, m->phase, m->ctrl, iters_row,
@@ -1176,11 +1191,12 @@ static int run_jacobi_block(tf_model* m, int g, int B, const int* labels, const 
     ++t;
     ++m->sweep_seq;
     const int n_lp = n_active - n_hp;
+    const bool first = shared_first && t == 1;
     // Few rows: a sweep is a chain of short kernels whose launch cost exceeds their run time, so the whole sweep is
     // captured once per (block, single-term slots, two-term slots) and replayed as a graph afterwards.
-    const bool as_graph = m->use_graphs && m->cap_stream != nullptr && !m->prof_on && n_active <= FIN_CHUNK && (int64_t)n_active * m->L <= m->sweep_graph_rows;
+    const bool as_graph = m->use_graphs && m->cap_stream != nullptr && !m->prof_on && n_active <= FIN_CHUNK && (int64_t)(first ? 1 : n_active) * m->L <= m->sweep_graph_rows;
     if (as_graph) {
-      const auto key = std::make_tuple(g, n_lp, n_hp, (const void*)v, (const void*)u, (const void*)labels, (const void*)iters_row);
+      const auto key = std::make_tuple(g, first ? -1 - n_lp : n_lp, n_hp, (const void*)v, (const void*)u, (const void*)labels, (const void*)iters_row);
       auto it = m->sweep_graphs.find(key);
       if (it == m->sweep_graphs.end() && m->sweep_graphs.size() < 2048) {
         tf_model::SeqGraph sg;
@@ -1191,7 +1207,7 @@ static int run_jacobi_block(tf_model* m, int g, int B, const int* labels, const 
         cudaError_t e = cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeRelaxed);
         int r = TF_OK;
         if (e == cudaSuccess) {
-          r = enqueue_sweep(n_lp, n_hp);
+          r = enqueue_sweep(n_lp, n_hp, first);
           e = cudaStreamEndCapture(m->cap_stream, &graph);
         }
         m->stream = user;
@@ -1211,10 +1227,10 @@ static int run_jacobi_block(tf_model* m, int g, int B, const int* labels, const 
         CU_OK(cudaGraphLaunch(it->second.exec, m->stream));
         m->launches += it->second.nodes;
       } else {
-        TF_TRY(enqueue_sweep(n_lp, n_hp));
+        TF_TRY(enqueue_sweep(n_lp, n_hp, first));
       }
     } else {
-      TF_TRY(enqueue_sweep(n_lp, n_hp));
+      TF_TRY(enqueue_sweep(n_lp, n_hp, first));
     }
     if (l2 && t <= m->trace_l2_sweeps) {
       LAUNCH(m, KC_CTRL, l2_distance_kernel, B, 256, 0, u, m->ref_seq,
