@@ -22,6 +22,7 @@
 #include "attention_tc.cuh"
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "f32_engine.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_tc2.cuh"
 #include "kernels_simt.cuh"
@@ -216,6 +217,12 @@ struct tf_model {
   int part_cap_rows = 0;
   int part_head_npad = 0, part_head_rows = 0;  // the same buffer seen as [part_head_rows, part_head_npad] for the head's slices
   int64_t sweep_graph_rows = 4096;  // TARFLOW_SWEEP_GRAPH_ROWS: largest slots x tokens replayed from a graph (0 = never)
+  // fp32 engine: blocks that fit a cluster's shared memory are decoded by one launch (f32_engine.cuh)
+  f32::SeqPlan seq_plan;
+  std::vector<float*> seq_image;              // per block, the images of a cluster's CTAs
+  int seq_clusters = 0;                       // clusters that fit the GPU side by side (0: not eligible)
+  int seq_cluster_smem[3] = {0, 0, 0};        // dynamic shared memory with 1, 2, 4 samples per cluster (0: does not fit)
+  int seq_cluster_tail[3] = {0, 0, 0};        // how much of the head and embedding matrices is in shared memory too
   int seq_variant = 0;       // 0: the block's own token buffers, 1: the compact buffers of the sequential fall-back
   size_t seq_part_row_floats = 0;  // floats of partial tiles available per sample
   bool use_graphs = true;
@@ -434,8 +441,34 @@ static int launch_gemm_tc2(tf_model* m, int cls, const CUtensorMap& ma, const CU
   return TF_OK;
 }
 
+template <int BM, int BN, int TM, int KS, class Epi>
+static int launch_gemm_f32(tf_model* m, int cls, const float* A, const Matrix& W, int M, const Epi& epi) {
+  using C = f32::GemmCfg<BM, BN, TM, KS>;
+  auto kern = f32::gemm_kernel<BM, BN, TM, KS, Epi>;
+  static bool configured[kMaxDevices] = {false};  // per instantiation and device
+  const int dev = current_device();
+  if (dev < 0) return fail(TF_ECUDA, "no usable current device");
+  if (!configured[dev]) {
+    CU_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    configured[dev] = true;
+  }
+  LAUNCH_PDL(m, cls, kern, dim3((W.N + BN - 1) / BN, (M + BM - 1) / BM), C::THREADS, C::SMEM, A, reinterpret_cast<const float*>(W.w), M,
+             W.N, W.K, epi);
+  return check_launch("f32::gemm_kernel");
+}
+
+// fp32 product.  The tile shrinks until about every SM has one: the kernels are short and few, so spreading a product over
+// more SMs matters more than operand reuse.  K % 4 != 0 (an MLP flow of odd dimension) takes the scalar-load kernel.
 template <class T, class Epi>
 static int launch_gemm_simt(tf_model* m, int cls, const T* A, const Matrix& W, int M, const Epi& epi) {
+  if constexpr (sizeof(T) == 4) {
+    if (W.K % 4 == 0) {
+      auto tiles = [&](int bm, int bn) { return ((M + bm - 1) / bm) * ((W.N + bn - 1) / bn); };
+      if (tiles(64, 64) >= 2 * m->num_sms) return launch_gemm_f32<64, 64, 4, 2>(m, cls, A, W, M, epi);
+      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, 2, 4>(m, cls, A, W, M, epi);
+      return launch_gemm_f32<16, 32, 1, 4>(m, cls, A, W, M, epi);
+    }
+  }
   dim3 grid((W.N + 63) / 64, (M + 63) / 64);
   LAUNCH(m, cls, (gemm_simt_kernel<T, Epi>), grid, 256, 0, A, reinterpret_cast<const T*>(W.w), M, W.N, W.K, epi);
   return check_launch("gemm_simt_kernel");
@@ -578,6 +611,9 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
       else
         LAUNCH(m, KC_ATTN, attn::attention_mma_kernel<false>, grid, 128, attn::smem_bytes<false>(), qkv, qkv_lo, att,
                att_lo, L, d, sl2);
+    } else if (m->hd % 4 == 0 && m->hd <= 128) {
+      LAUNCH_PDL(m, KC_ATTN, f32::attention_kernel, dim3((L + f32::AT_Q - 1) / f32::AT_Q, m->cfg.n_heads, n_slots), 128,
+                 f32::attention_smem_floats(m->hd) * sizeof(float), qkv, att, L, d, m->hd, 1.0f / sqrtf((float)m->hd));
     } else {
       const int warps = 4;
       dim3 grid((L + warps - 1) / warps, m->cfg.n_heads, n_slots);
@@ -654,6 +690,39 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
 // ------------------------------------------------------------------------------------------------
 // sequential block with KV cache (Eq. 5): L-1 single-token passes
 // ------------------------------------------------------------------------------------------------
+// fp32 models whose block fits a cluster's shared memory: the whole block in one launch
+static int run_sequential_cluster(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
+  const BlockW& bw = m->blocks[g];
+  // one sample per cluster while the clusters fit the GPU side by side, then as many as shared memory allows
+  int S = 1;
+  while (S < 4 && B > S * m->seq_clusters && m->seq_cluster_smem[S == 1 ? 1 : 2] > 0) S *= 2;
+  const int si = S == 1 ? 0 : S == 2 ? 1 : 2;
+  static decltype(&f32::seq_cluster_kernel<1, 0>) const kernels[3][3] = {
+      {f32::seq_cluster_kernel<1, 0>, f32::seq_cluster_kernel<1, 1>, f32::seq_cluster_kernel<1, 2>},
+      {f32::seq_cluster_kernel<2, 0>, f32::seq_cluster_kernel<2, 1>, f32::seq_cluster_kernel<2, 2>},
+      {f32::seq_cluster_kernel<4, 0>, f32::seq_cluster_kernel<4, 1>, f32::seq_cluster_kernel<4, 2>}};
+  auto kern = kernels[si][m->seq_cluster_tail[si]];
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(f32::SC * ((B + S - 1) / S));
+  lc.blockDim = dim3(f32::ST);
+  lc.dynamicSmemBytes = m->seq_cluster_smem[si];
+  lc.stream = m->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = f32::SC;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  m->cur_rows = (int64_t)B * (m->L - 1);
+  m->pre(KC_SEQ_GEMM);
+  cudaError_t e = cudaLaunchKernelEx(&lc, kern, m->seq_plan, (const float*)m->seq_image[g], v, u, labels,
+                                     (const float*)bw.pos, (const float*)bw.cls, reinterpret_cast<float*>(m->kcache),
+                                     reinterpret_cast<float*>(m->vcache), m->cfg.max_batch, B, g & 1, m->err);
+  m->post(KC_SEQ_GEMM);
+  if (e != cudaSuccess) return fail(TF_ECUDA, "seq_cluster_kernel launch failed: %s", cudaGetErrorString(e));
+  return TF_OK;
+}
+
 template <class T>
 static int run_sequential_block(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
   const BlockW& bw = m->blocks[g];
@@ -665,6 +734,7 @@ static int run_sequential_block(tf_model* m, int g, int B, const int* labels, co
   const size_t layer_stride = (size_t)m->cfg.max_batch * L * d;
   const float scale = 1.0f / sqrtf((float)m->hd);
   int ethreads = d < 256 ? d : 256;
+  if (m->seq_clusters > 0) return run_sequential_cluster(m, g, B, labels, v, u);
   m->cur_rows = B;
   LAUNCH(m, KC_SEQ_UPDATE, copy_first_token_kernel, (B * D + 127) / 128, 128, 0, v, u, B, L, D, rev);
   for (int t = 0; t + 1 < L; ++t) {
@@ -1514,6 +1584,106 @@ static int upload_matrix(tf_model* m, Matrix* W, const float* src, int N, int K,
   return make_map_bf16(&W->map, w, (uint64_t)N, (uint64_t)K, (uint32_t)W->bn);
 }
 
+// Decides whether an fp32 model's blocks are decoded by f32::seq_cluster_kernel and cuts them into the CTAs' shares: whole
+// heads round robin, hidden units (multiples of four) so that the bytes come out even.
+static int plan_seq_cluster(tf_model* m) {
+  const int d = m->d, hid = m->hid, heads = m->cfg.n_heads, hd = m->hd, lpk = hd / 4;
+  if (d % 4 || hid % 4 || hd % 4 || hd > 128 || (lpk & (lpk - 1)) || d > 1024) return TF_OK;
+  f32::SeqPlan& P = m->seq_plan;
+  P.n_layers = m->cfg.n_layers; P.heads = heads; P.hd = hd; P.d = d; P.D = m->D; P.L = m->L;
+  P.owners = heads < f32::SC ? heads : f32::SC;
+  const int64_t share = ((int64_t)4 * d * d + (int64_t)2 * d * hid) / f32::SC;
+  int left = hid;
+  for (int r = f32::SC - 1; r >= 0; --r) {  // CTAs without heads come last and take the most hidden units
+    P.nown[r] = (heads - r + f32::SC - 1) / f32::SC;
+    if (P.nown[r] < 0) P.nown[r] = 0;
+    const int64_t room = share - (int64_t)4 * hd * d * P.nown[r];
+    int n = room <= 0 ? 0 : (int)(room / (2 * d)) / 4 * 4;
+    if (n > left || r == 0) n = left;
+    P.nu[r] = n;
+    left -= n;
+  }
+  int64_t most = 0, off = 0;
+  for (int r = 0; r < f32::SC; ++r) {
+    P.off[r] = (int)off;
+    if (P.fixed_floats(r) > most) most = P.fixed_floats(r);
+    off += P.fixed_floats(r) + P.tail_floats(2);
+    if (off > (1 << 28)) return TF_OK;
+  }
+  P.off[f32::SC] = (int)off;
+  const int limit = 226 * 1024;  // a block may have 227 KB, static shared memory and its padding included
+  for (int i = 0; i < 3; ++i) {
+    for (int level = 2; level >= 0 && m->seq_cluster_smem[i] == 0; --level) {
+      const int64_t need = (most + P.work_floats(1 << i) + P.tail_floats(level)) * (int64_t)sizeof(float);
+      if (need > limit) continue;
+      m->seq_cluster_tail[i] = level;
+      m->seq_cluster_smem[i] = (int)need;
+    }
+  }
+  if (m->seq_cluster_smem[0] == 0) return TF_OK;
+  for (auto kern : {f32::seq_cluster_kernel<1, 0>, f32::seq_cluster_kernel<1, 1>, f32::seq_cluster_kernel<1, 2>, f32::seq_cluster_kernel<2, 0>,
+                    f32::seq_cluster_kernel<2, 1>, f32::seq_cluster_kernel<2, 2>, f32::seq_cluster_kernel<4, 0>,
+                    f32::seq_cluster_kernel<4, 1>, f32::seq_cluster_kernel<4, 2>})
+    CU_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(f32::SC);
+  lc.blockDim = dim3(f32::ST);
+  lc.dynamicSmemBytes = m->seq_cluster_smem[0];
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = f32::SC;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, f32::seq_cluster_kernel<1, 0>, &lc) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  m->seq_clusters = n;
+  return TF_OK;
+}
+
+// the images of one block; `layers` is the first layer's tensors in the weight blob, w_out / b_out interleaved
+static int upload_seq_images(tf_model* m, const float* layers, const float* lnf, const float* b_in, const float* w_in_t,
+                             const float* w_out, const float* b_out) {
+  const f32::SeqPlan& P = m->seq_plan;
+  const int d = P.d, hid = m->hid, hd = P.hd, D = P.D, No = P.pad4(2 * D), Dp = P.pad4(D);
+  std::vector<float> img(P.off[f32::SC], 0.f);
+  int unit0 = 0;
+  for (int r = 0; r < f32::SC; ++r) {
+    const int nown = P.nown[r], nu = P.nu[r], nq = 3 * hd * nown;
+    float* o = img.data() + P.off[r];
+    const float* q = layers;
+    for (int i = 0; i < P.n_layers; ++i) {
+      const float *ln1 = q, *w_qkv = ln1 + 2 * d, *b_qkv = w_qkv + (size_t)3 * d * d, *w_o = b_qkv + 3 * d, *b_o = w_o + (size_t)d * d,
+                  *ln2 = b_o + d, *w_1 = ln2 + 2 * d, *b_1 = w_1 + (size_t)hid * d, *w_2 = b_1 + hid, *b_2 = w_2 + (size_t)d * hid;
+      q = b_2 + d;
+      auto row_of = [&](int n) { return (n / hd % 3) * d + (r + f32::SC * (n / (3 * hd))) * hd + n % hd; };  // row of w_qkv
+      auto put = [&](const float* p, int n) { memcpy(o, p, n * sizeof(float)); o += n; };
+      for (int n = 0; n < nq; ++n) put(w_qkv + (size_t)row_of(n) * d, d);
+      for (int n = 0; n < nq; ++n) *o++ = b_qkv[row_of(n)];
+      for (int n = 0; n < d; ++n)
+        for (int k = 0; k < nown; ++k) put(w_o + (size_t)n * d + (r + f32::SC * k) * hd, hd);
+      put(w_1 + (size_t)unit0 * d, nu * d);
+      put(b_1 + unit0, nu);
+      for (int n = 0; n < d; ++n) put(w_2 + (size_t)n * hid + unit0, nu);
+      put(ln1, 2 * d); put(b_o, d); put(ln2, 2 * d); put(b_2, d);
+    }
+    memcpy(o, lnf, 2 * d * sizeof(float)); o += 2 * d;
+    memcpy(o, b_in, d * sizeof(float)); o += d;
+    memcpy(o, w_out, (size_t)2 * D * d * sizeof(float)); o += (size_t)No * d;  // the image starts out as zeros
+    memcpy(o, b_out, 2 * D * sizeof(float)); o += No;
+    for (int j = 0; j < d; ++j)
+      for (int c = 0; c < Dp; ++c) *o++ = c < D ? w_in_t[(size_t)c * d + j] : 0.f;
+    unit0 += nu;
+  }
+  float* dev = nullptr;
+  TF_TRY(upload_f32(m, &dev, img.data(), img.size()));
+  m->seq_image.push_back(dev);
+  return TF_OK;
+}
+
 static size_t block_floats(const tf_config& c, int L, int D) {
   size_t d = c.width, hid = (size_t)c.mlp_ratio * d;
   size_t n = d * D + d + (size_t)L * d + (size_t)c.n_classes * d;
@@ -1545,19 +1715,22 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
 
   BlobReader rd{reinterpret_cast<const float*>(reinterpret_cast<const char*>(blob) + 64), nullptr};
   m->blocks.resize(c.n_blocks);
-  std::vector<float> tmp;
+  if (c.dtype == 0) TF_TRY(plan_seq_cluster(m));
+  std::vector<float> tmp, w_in_t;
   for (int g = 0; g < c.n_blocks; ++g) {
     BlockW& bw = m->blocks[g];
     const float* w_in = rd.take((size_t)d * D);
-    tmp.resize((size_t)d * D);
+    w_in_t.resize((size_t)d * D);
     for (int j = 0; j < d; ++j)
-      for (int cc = 0; cc < D; ++cc) tmp[(size_t)cc * d + j] = w_in[(size_t)j * D + cc];
-    TF_TRY(upload_f32(m, &bw.w_in_t, tmp.data(), tmp.size()));
-    TF_TRY(upload_f32(m, &bw.b_in, rd.take(d), d));
+      for (int cc = 0; cc < D; ++cc) w_in_t[(size_t)cc * d + j] = w_in[(size_t)j * D + cc];
+    TF_TRY(upload_f32(m, &bw.w_in_t, w_in_t.data(), w_in_t.size()));
+    const float* b_in = rd.take(d);
+    TF_TRY(upload_f32(m, &bw.b_in, b_in, d));
     TF_TRY(upload_f32(m, &bw.pos, rd.take((size_t)L * d), (size_t)L * d));
     bw.cls = nullptr;
     if (c.n_classes > 0) TF_TRY(upload_f32(m, &bw.cls, rd.take((size_t)c.n_classes * d), (size_t)c.n_classes * d));
     bw.layers.resize(c.n_layers);
+    const float* layers = rd.p;
     for (LayerW& lw : bw.layers) {
       TF_TRY(upload_f32(m, &lw.ln1_g, rd.take(d), d));
       TF_TRY(upload_f32(m, &lw.ln1_b, rd.take(d), d));
@@ -1572,6 +1745,7 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
       TF_TRY(upload_matrix(m, &lw.w_2, rd.take((size_t)d * hid), d, hid, staging));
       TF_TRY(upload_f32(m, &lw.b_2, rd.take(d), d));
     }
+    const float* lnf = rd.p;
     TF_TRY(upload_f32(m, &bw.lnf_g, rd.take(d), d));
     TF_TRY(upload_f32(m, &bw.lnf_b, rd.take(d), d));
     // head: interleave rows so that outputs (2c, 2c+1) = (mu~_c, alpha~_c)
@@ -1587,6 +1761,7 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
     }
     TF_TRY(upload_matrix(m, &bw.w_out, tmp.data(), 2 * D, d, staging));
     TF_TRY(upload_f32(m, &bw.b_out, btmp.data(), btmp.size()));
+    if (m->seq_clusters > 0) TF_TRY(upload_seq_images(m, layers, lnf, b_in, w_in_t.data(), tmp.data(), btmp.data()));
   }
 
   // workspace
@@ -1730,6 +1905,12 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
     TF_TRY(dev_alloc(m, &m->seq_stats, (size_t)tf_model::MAX_CHAINS * 16 * B));
     if (const char* e = getenv("TARFLOW_SWEEP_GRAPH_ROWS")) m->sweep_graph_rows = atoll(e);
     if (const char* e = getenv("TARFLOW_GRAPHS")) m->use_graphs = atoi(e) != 0;
+  }
+  if (c.dtype == 0) {
+    CU_OK(cudaFuncSetAttribute(f32::attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, f32::attention_smem_floats(128) * (int)sizeof(float)));
+    if (const char* e = getenv("TARFLOW_SWEEP_GRAPH_ROWS")) m->sweep_graph_rows = atoll(e);
+    if (const char* e = getenv("TARFLOW_GRAPHS")) m->use_graphs = atoi(e) != 0;
+    CU_OK(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
   }
   CU_OK(cudaDeviceSynchronize());
   return TF_OK;
