@@ -265,3 +265,694 @@ __device__ __forceinline__ void feed(const Job& job, Feed& f, uint32_t ring, uin
     }
   }
 }
+
+// grid: groups * HEADS clusters of CS CTAs (cooperative), 256 threads and a warp that moves the weights
+template <int D, int RT>
+__global__ void __launch_bounds__(NTHREADS + 32, 1)
+seq_block_kernel(const __grid_constant__ Job job) {
+  using C = Cfg<D, RT>;
+  constexpr int HEADS = C::HEADS, CS = C::CS, N1 = C::N1, CW = C::CW, QN = C::QN, SG = C::SG, NSL = C::NSL, UPC = C::UPC, NE = C::NE, NA = C::NA;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const uint32_t sb = smem_u32(smem), bars = sb + C::BARS;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int r = blockIdx.x % CS, cl = blockIdx.x / CS, c = cl % HEADS, group = cl / HEADS;  // r: rank in the cluster
+  const int row0 = group * job.rows, nb = job.B - row0 < job.rows ? job.B - row0 : job.rows;  // this group's samples
+  const int L = job.L, Dt = job.Dt, n_steps = L - 1, nl = job.n_layers;
+  int* err = job.err;
+  auto bar = [&](int i) { return bars + 8u * (2 * C::NSLOT + i); };
+  enum { B_IN0, B_IN1, B_RECV0, B_RECV1, B_ALL0, B_ALL1, B_OUT0, B_OUT1, B_STAT, B_HEAD };  // 0: attention half, 1: MLP half
+  uint8_t* tail_mem = smem + C::BARS + C::NBARS * 8;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail_mem);
+  volatile int* s_bad = reinterpret_cast<volatile int*>(tail_mem + 4);
+
+  if (tid == 0) {
+    for (int i = 0; i < C::NBARS; ++i) mbar_init(bars + 8u * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *s_bad = 0;
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tcgen05_fence_before();
+  __syncthreads();
+  cluster_sync();  // every CTA of the cluster has set up its barriers
+  tcgen05_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  // samples this CTA attends for: bl r .. bl r + mine - 1 of the group
+  const int bl = (nb + CS - 1) / CS, mine = nb - r * bl < bl ? (nb - r * bl > 0 ? nb - r * bl : 0) : bl;
+  auto rows_of = [&](int p) { return ((size_t)(row0 + r * bl + p) * HEADS + c) * L * HD; };  // cache rows of (sample, head)
+
+  if (warp == NWARPS) {
+    // ==================================================================== weights
+    if (lane == 0) {
+      Feed fd;
+      feed<D, RT>(job, fd, sb + C::RING, bars, r, c, job.prefetch_w && group == 0, mine, rows_of(0));
+    }
+  } else {
+    constexpr uint32_t idesc = make_idesc(RT);
+    // attention roles: the eight warps share every sample's keys (the same split whatever the batch), eight lanes share a key, four
+    // keys per lane group in flight
+    constexpr int KR = NWARPS * 4;  // keys apart in a lane group
+    const int sub = lane & 7, kgrp = warp * 4 + (lane >> 3);
+    // hidden units this thread finishes: eight of them, samples fb, fb + FB, ...
+    constexpr int FB = NTHREADS / (UPC / 8);
+    const int u8 = (tid % (UPC / 8)) * 8, fb = tid / (UPC / 8);
+    // rows of the residual stream: the cluster owns rows own0 .. own0 + own - 1 of the group, this CTA their columns r CW ..;
+    // thread = (column quad q, row, group g of slices); the warps of g == 0 hold the residual stream itself in h
+    const int rpc = (nb + HEADS - 1) / HEADS, own0 = c * rpc, own = nb - own0 < rpc ? (nb - own0 > 0 ? nb - own0 : 0) : rpc;
+    const int q = tid % QN, lrow = (tid / QN) % C::RPC, g = tid / (QN * C::RPC), col = r * CW + 4 * q;
+    const bool my_row = lrow < own, holder = warp < C::GW;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 h = zero4;
+    float4* s_sum = reinterpret_cast<float4*>(smem + C::SUM);
+    float* s_xn = reinterpret_cast<float*>(smem + C::XN);
+    float* s_tok = reinterpret_cast<float*>(smem + C::TOK);
+    float* s_bias = reinterpret_cast<float*>(smem + C::BIAS);
+    float* s_merge = reinterpret_cast<float*>(smem + C::MERGE);
+    unsigned long long* xrow = job.xrow + (size_t)group * RT * (D / 2);
+    unsigned long long* xpart = job.xpart + (size_t)group * RT * HEADS * D;
+    int slot = 0;  // position in the weight ring
+    uint32_t ring_parity = 0, stat_parity = 0, seq = job.seq0;
+    bool alive = true;  // no wait of this thread has failed: after a failure no barrier is armed any more
+
+    auto cbar = [&]() { named_bar_sync(1, NTHREADS); };
+    auto await = [&](int b, uint32_t parity, int code) {
+      if (!wait_bar(bar(b), parity, err, code)) alive = false;
+      __syncwarp();
+    };
+    // unit u of the phase has arrived: its address (warp 0); the products of unit u have been issued; next phase
+    auto take = [&](int u) {
+      const int s = slot + u, wrap = s >= C::NSLOT;
+      if (!wait_bar(bars + 8u * (s - (wrap ? C::NSLOT : 0)), ring_parity ^ (uint32_t)wrap, err, TFERR_WAIT_FULL)) alive = false;
+      __syncwarp();
+      return sb + C::RING + (s - (wrap ? C::NSLOT : 0)) * C::UNIT;
+    };
+    auto release = [&](int u) {
+      const int s = slot + u;
+      umma_commit(bars + 8u * (C::NSLOT + (s >= C::NSLOT ? s - C::NSLOT : s)));
+    };
+    auto advance = [&](int n) {
+      slot += n;
+      if (slot >= C::NSLOT) { slot -= C::NSLOT; ring_parity ^= 1u; }
+    };
+    auto mma = [&](uint32_t d, uint32_t w, uint32_t x, bool add) {
+      const uint64_t wd = make_smem_desc(w), xd = make_smem_desc(x);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) umma_f16(d, wd + 2u * k, xd + 2u * k, idesc, k > 0 || add);
+    };
+    // one warp polls, everybody else waits at the compute warps' barrier
+    auto meet = [&](int b, uint32_t parity) {
+      if (warp == 0) await(b, parity, TFERR_WAIT_FULL);
+      cbar();
+    };
+    auto ld4 = [&](const float* p) { return __ldg(reinterpret_cast<const float4*>(p + col)); };
+    auto token_at = [&](int row, int l) { return ((size_t)(row0 + own0 + row) * L + tok_index(l, L, job.reversed)) * Dt; };
+
+#pragma unroll 1
+    for (int row = 0; row < own; ++row) {  // the first token is copied (Eq. 5, first row)
+      const size_t e = token_at(row, 0);
+#pragma unroll 1
+      for (int cc = tid; cc < Dt; cc += NTHREADS) {
+        const float x = job.v[e + cc];
+        s_tok[row * Dt + cc] = x;
+        if (r == 0) job.u[e + cc] = x;
+      }
+    }
+
+    for (int t = 0; t < n_steps; ++t) {
+      cbar();
+      if (__shfl_sync(0xffffffffu, *s_bad, 0) != 0) break;
+#pragma unroll 1
+      for (int half = 0; half <= 2 * nl; ++half) {
+        const Layer* ly = job.layers + (half >> 1);
+        const int mlp = half & 1;                                   // which half of the layer follows
+        const uint32_t lp = (uint32_t)(t * nl + (half >> 1)) & 1u;  // parity of its barriers
+        // ================================================================== residual rows of this cluster
+        if (own > 0) {
+          float4 gg = zero4, bb = zero4, add = zero4, sum[NA];
+#pragma unroll
+          for (int i = 0; i < NA; ++i) sum[i] = zero4;
+          if (holder && my_row) {
+            gg = ld4(half == 2 * nl ? job.lnf_g : mlp ? ly->ln2_g : ly->ln1_g);
+            bb = ld4(half == 2 * nl ? job.lnf_b : mlp ? ly->ln2_b : ly->ln1_b);
+            add = ld4(half == 0 ? job.b_in : mlp ? ly->b_o : ly[-1].b_2);
+          }
+          if (half == 0) {  // embedding of token t
+            if (my_row) {
+              if (holder) {
+                const float4 p = ld4(job.pos + (size_t)t * D);
+                add.x += p.x; add.y += p.y; add.z += p.z; add.w += p.w;
+                if (job.cls != nullptr) {
+                  const float4 y = ld4(job.cls + (size_t)job.labels[row0 + own0 + lrow] * D);
+                  add.x += y.x; add.y += y.y; add.z += y.z; add.w += y.w;
+                }
+                h = zero4;
+              }
+#pragma unroll
+              for (int i = 0; i < NA; ++i)
+#pragma unroll 4
+                for (int cc = g + i * SG; cc < Dt; cc += C::SGC) {
+                  const float4 w = ld4(job.w_in_t + (size_t)cc * D);
+                  const float tv = s_tok[lrow * Dt + cc];
+                  sum[i].x = fmaf(tv, w.x, sum[i].x); sum[i].y = fmaf(tv, w.y, sum[i].y);
+                  sum[i].z = fmaf(tv, w.z, sum[i].z); sum[i].w = fmaf(tv, w.w, sum[i].w);
+                }
+            }
+          } else if (my_row) {  // the slices of this thread's groups, added in index order
+            unsigned long long w[NSL][4];
+            Spin spin;
+            bool ok = true, all;
+            const unsigned long long* at = xpart + ((size_t)(own0 + lrow) * HEADS + g) * D + col;
+            do {  // one slice is polled; when it is there, so are, nearly always, the others
+              ll_load2(at, w[0][0], w[0][1]);
+              ll_load2(at + 2, w[0][2], w[0][3]);
+            } while (!(ll_here(w[0][0], w[0][1], seq) && ll_here(w[0][2], w[0][3], seq)) && (ok = spin.more(err)));
+            if (NSL > 1) do {
+                all = true;
+#pragma unroll
+                for (int k = 1; k < NSL; ++k) {
+                  ll_load2(at + (size_t)k * SG * D, w[k][0], w[k][1]);
+                  ll_load2(at + (size_t)k * SG * D + 2, w[k][2], w[k][3]);
+                }
+#pragma unroll
+                for (int k = 1; k < NSL; ++k) all = all && ll_here(w[k][0], w[k][1], seq) && ll_here(w[k][2], w[k][3], seq);
+              } while (!all && ok && (ok = spin.more(err)));
+            alive = alive && ok;
+#pragma unroll
+            for (int k = 0; k < NSL; ++k) {
+              float4& a = sum[k % NA];
+              a.x += __uint_as_float((uint32_t)w[k][0]); a.y += __uint_as_float((uint32_t)w[k][1]);
+              a.z += __uint_as_float((uint32_t)w[k][2]); a.w += __uint_as_float((uint32_t)w[k][3]);
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < NA; ++i)
+            if (i > 0 || !holder) s_sum[((g + i * SG - 1) * C::RPC + lrow) * QN + q] = sum[i];
+          cbar();
+          if (holder) {
+            if (tid == 0 && alive) mbar_arrive_expect_tx(bar(B_STAT), (uint32_t)(own * NE * 8));
+            __syncwarp();
+            h.x += add.x + sum[0].x; h.y += add.y + sum[0].y; h.z += add.z + sum[0].z; h.w += add.w + sum[0].w;
+#pragma unroll
+            for (int k = 0; k < C::SGC - 1; ++k) {
+              const float4 y = s_sum[(k * C::RPC + lrow) * QN + q];
+              h.x += y.x; h.y += y.y; h.z += y.z; h.w += y.w;
+            }
+            // LayerNorm: (mean, squared deviations) of CE columns by shuffles, exchanged over the cluster and combined
+            // (Chan et al.), as accurate as two passes over the row
+            float s = (h.x + h.y) + (h.z + h.w);
+#pragma unroll
+            for (int o = (QN > 32 ? 32 : QN) / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            const float wmean = s * (1.f / C::CE);
+            float a0 = h.x - wmean, a1 = h.y - wmean, a2 = h.z - wmean, a3 = h.w - wmean;
+            float m2 = (a0 * a0 + a1 * a1) + (a2 * a2 + a3 * a3);
+#pragma unroll
+            for (int o = (QN > 32 ? 32 : QN) / 2; o > 0; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+            const int ql = QN > 32 ? q & 31 : q;
+            if (my_row && ql < CS)
+              st_async2(peer_addr(sb + C::STAT + (lrow * NE + r * C::SPR + (QN > 32 ? q >> 5 : 0)) * 8, ql), __float_as_uint(wmean),
+                        __float_as_uint(m2), peer_addr(bar(B_STAT), ql));
+            __syncwarp();
+            await(B_STAT, stat_parity, TFERR_WAIT_FULL);
+            const float2* st = reinterpret_cast<const float2*>(smem + C::STAT) + lrow * NE;
+            float mean = 0.f;
+#pragma unroll
+            for (int k = 0; k < NE; ++k) mean += st[k].x;
+            mean *= 1.f / NE;
+            m2 = 0.f;
+#pragma unroll
+            for (int k = 0; k < NE; ++k) {
+              const float2 e = st[k];
+              m2 += fmaf((float)C::CE * (e.x - mean), e.x - mean, e.y);
+            }
+            const float rstd = rsqrtf(m2 * (1.f / D) + 1e-5f);
+            const uint32_t lo = pack_bf16(fmaf((h.x - mean) * rstd, gg.x, bb.x), fmaf((h.y - mean) * rstd, gg.y, bb.y));
+            const uint32_t hi = pack_bf16(fmaf((h.z - mean) * rstd, gg.z, bb.z), fmaf((h.w - mean) * rstd, gg.w, bb.w));
+            if (my_row) {
+              if (half < 2 * nl) {  // this thread's columns of the next projection's input
+                ll_store2(xrow + ((size_t)(own0 + lrow) * CS + r) * (CW / 2) + 2 * q, lo, hi, seq + 1);
+              } else {  // the head's input
+                const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&lo));
+                const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hi));
+                *reinterpret_cast<float4*>(s_xn + lrow * CW + 4 * q) = make_float4(f0.x, f0.y, f1.x, f1.y);
+              }
+            }
+          }
+          stat_parity ^= 1u;
+          cbar();  // the other warps have waited here instead of polling for the next rows
+        }
+        ++seq;
+        if (half == 2 * nl) break;
+        // ================================================================== half a layer
+        if (tid == 0 && alive) {
+          if (mlp) {
+            mbar_arrive_expect_tx(bar(B_RECV1), (uint32_t)(CS * nb * UPC * 4));
+            mbar_arrive_expect_tx(bar(B_ALL1), (uint32_t)(nb * UNITS * 2));
+          } else {
+            if (mine > 0) mbar_arrive_expect_tx(bar(B_RECV0), (uint32_t)(CS * mine * 192 * 4));
+            mbar_arrive_expect_tx(bar(B_ALL0), (uint32_t)(nb * 128));
+          }
+        }
+        __syncwarp();
+        bf16 *kc = job.kc + (half >> 1) * job.layer_stride, *vc = job.vc + (half >> 1) * job.layer_stride;
+        uint4 kv[4], vv[4];  // rows of the cache in flight
+        auto fetch = [&](int p, int j0) {
+          const size_t base = rows_of(p) + sub * 8;
+          const bf16 *kr = kc + base, *vr = vc + base;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int j = j0 + k * KR + kgrp;
+            kv[k] = vv[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (j < t) {
+              kv[k] = __ldcg(reinterpret_cast<const uint4*>(kr + j * HD));
+              vv[k] = __ldcg(reinterpret_cast<const uint4*>(vr + j * HD));
+            }
+          }
+        };
+        if (half == 1 && own > 0 && t + 1 < n_steps) {  // what the end of the step will read from memory: on its way to L2
+          if (holder && my_row) prefetch_line(job.pos + (size_t)(t + 1) * D + col);
+          const int per = (Dt + 31) / 32;
+          if (tid < own * per) prefetch_line(job.v + token_at(tid / per, t + 1) + (tid % per) * 32);
+        }
+        if (!mlp) {
+          if (tid < 192) s_bias[tid] = __ldg(ly->b_qkv + (tid >> 6) * D + c * HD + (tid & 63));
+          if (mine > 0) fetch(0, 0);  // rows of earlier tokens: on their way while q is computed
+        }
+        {  // rows of the projection's input (this rank's columns) into swizzled [RT][64] operand tiles
+          constexpr int IT = RT * QN / NTHREADS;
+          unsigned long long w[IT][2];
+          Spin spin;
+          bool ok = true, all;
+          const int first = tid / QN;
+          const unsigned long long* at = xrow + ((size_t)first * CS + r) * (CW / 2) + 2 * q;
+          if (first < nb) {
+            do ll_load2(at, w[0][0], w[0][1]);
+            while (!ll_here(w[0][0], w[0][1], seq) && (ok = spin.more(err)));
+          }
+          if (IT > 1) do {
+              all = true;
+#pragma unroll
+              for (int k = 1; k < IT; ++k)
+                if (first + k * (NTHREADS / QN) < nb) ll_load2(at + (size_t)k * (NTHREADS / QN) * (D / 2), w[k][0], w[k][1]);
+#pragma unroll
+              for (int k = 1; k < IT; ++k)
+                if (first + k * (NTHREADS / QN) < nb) all = all && ll_here(w[k][0], w[k][1], seq);
+            } while (!all && ok && (ok = spin.more(err)));
+          alive = alive && ok;
+#pragma unroll
+          for (int k = 0; k < IT; ++k) {
+            const int row = first + k * (NTHREADS / QN);
+            if (row < nb)
+              *reinterpret_cast<uint2*>(smem + C::ACT + (q >> 4) * (RT * 128) + swz128(row, (q & 15) >> 1) + (q & 1) * 8) =
+                  make_uint2((uint32_t)w[k][0], (uint32_t)w[k][1]);
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+        }
+        cbar();
+        if (warp == 0) {
+#pragma unroll 1
+          for (int u = 0; u < (mlp ? 4 : 3); ++u) {
+            const uint32_t w = take(u);
+            tcgen05_fence_after();
+            if (elect_one()) {
+              const uint32_t act = sb + C::ACT;
+              if (mlp) {  // per slab the cluster's 256 units; with 64-row tiles a pair of units is one operand
+                if (N1 == 4) {
+                  mma(tmem, w, act + u * (RT * 128), u > 0);
+                  mma(tmem + RT, w + 16384, act + u * (RT * 128), u > 0);
+                } else if (N1 == 2) {
+                  mma(tmem + (u & 1) * RT, w, act + (u >> 1) * (RT * 128), u > 1);
+                } else if (u & 1) {
+                  mma(tmem + (u >> 1) * RT, w - C::UNIT, act, false);
+                }
+              } else if (u < 2) {  // q | k per slab
+                if (N1 == 1) {
+                  if (u == 1) mma(tmem, w - C::UNIT, act, false);
+                } else {
+#pragma unroll 1
+                  for (int z = 0; z < N1 / 2; ++z) mma(tmem, w + z * 16384, act + (u * (N1 / 2) + z) * (RT * 128), u + z > 0);
+                }
+              } else {  // v of every slab
+#pragma unroll 1
+                for (int z = 0; z < N1; ++z) mma(tmem + RT, w + z * 8192, act + z * (RT * 128), z > 0);
+              }
+              if (N1 == 1 && (mlp || u < 2)) {
+                if (u & 1) { release(u - 1); release(u); }
+              } else {
+                release(u);
+              }
+              if (u == (mlp ? 3 : 2)) umma_commit(bar(B_IN0 + mlp));
+            }
+            __syncwarp();
+          }
+          await(B_IN0 + mlp, lp, TFERR_WAIT_TMEM_FULL);
+          tcgen05_fence_before();
+        }
+        advance(mlp ? 4 : 3);
+        cbar();
+        tcgen05_fence_after();
+        const uint32_t t_lane = tmem + (warp >> 2) * RT + ((uint32_t)((warp & 3) * 32) << 16);
+        if (!mlp) {
+          // ---------------------------------------------------------------- attention
+          if (warp < 6) {  // reduce-scatter: warp w holds channels 32 w .. of q | k | v, one sample per column
+            float* stg = reinterpret_cast<float*>(smem + C::STG) + warp * 32 + lane;
+#pragma unroll 1
+            for (int b0 = 0; b0 < nb; b0 += 8) {
+              float v[8];
+              tmem_cols8(t_lane + b0, v);
+#pragma unroll
+              for (int b = 0; b < 8; ++b)
+                if (b0 + b < nb) stg[(b0 + b) * 192] = v[b];
+            }
+            tcgen05_fence_before();
+          }
+          fence_proxy_async_smem();
+          cbar();
+          if (tid < CS) {  // samples bl p .. go to CTA p
+            const int n = nb - tid * bl < bl ? nb - tid * bl : bl;
+            if (n > 0)
+              copy_to_peer(peer_addr(sb + C::RECV + r * C::BL * 768, tid), sb + C::STG + tid * bl * 768, (uint32_t)n * 768,
+                           peer_addr(bar(B_RECV0), tid));
+          }
+          __syncwarp();
+          if (mine > 0) {
+            meet(B_RECV0, lp);
+            for (int i = tid; i < mine * 48; i += NTHREADS) {  // four channels of q, k or v of one sample
+              const int p = i / 48, c4 = i - p * 48;
+              float4 x = *reinterpret_cast<const float4*>(s_bias + 4 * c4);
+              const float* src = reinterpret_cast<const float*>(smem + C::RECV) + p * 192 + 4 * c4;
+#pragma unroll
+              for (int k = 0; k < CS; ++k) {
+                const float4 y = *reinterpret_cast<const float4*>(src + k * C::BL * 192);
+                x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+              }
+              uint8_t* mem = smem + C::QKV + p * 512;
+              if (c4 < 16) {  // scores in base-2 units: softmax via exp2
+                *reinterpret_cast<float4*>(mem + 16 * c4) =
+                    make_float4(x.x * job.scale_log2e, x.y * job.scale_log2e, x.z * job.scale_log2e, x.w * job.scale_log2e);
+              } else {
+                const uint2 w2 = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+                *reinterpret_cast<uint2*>(mem + 256 + (c4 - 16) * 8) = w2;
+                *reinterpret_cast<uint2*>((c4 < 32 ? kc : vc) + rows_of(p) + (size_t)t * HD + (c4 & 15) * 4) = w2;
+              }
+            }
+            cbar();
+#pragma unroll 1
+            for (int p = 0; p < mine; ++p) {
+              const uint8_t* mem = smem + C::QKV + p * 512;
+              float2 q2[4], o2[4];
+#pragma unroll
+              for (int i = 0; i < 4; i += 2) {
+                const float4 q4 = *reinterpret_cast<const float4*>(mem + sub * 32 + i * 8);
+                q2[i] = make_float2(q4.x, q4.y);
+                q2[i + 1] = make_float2(q4.z, q4.w);
+                o2[i] = o2[i + 1] = make_float2(0.f, 0.f);
+              }
+              float m_run = -INFINITY, l_run = 0.f;
+#pragma unroll 1
+              for (int j0 = 0; j0 <= t; j0 += 4 * KR) {
+                uint4 kn[4], vn[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  kn[k] = kv[k];
+                  vn[k] = vv[k];
+                }
+                // the next round's rows (of the next sample after the last one) travel while this round is worked on
+                const bool on = j0 + 4 * KR <= t;
+                if (on || p + 1 < mine) fetch(on ? p : p + 1, on ? j0 + 4 * KR : 0);
+                float sc[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  if (j0 + k * KR + kgrp == t) {  // the new row
+                    kn[k] = *reinterpret_cast<const uint4*>(mem + 256 + sub * 16);
+                    vn[k] = *reinterpret_cast<const uint4*>(mem + 384 + sub * 16);
+                  }
+                  const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kn[k]);
+                  float2 s2 = fmul2(q2[0], __bfloat1622float2(k2[0]));
+#pragma unroll
+                  for (int i = 1; i < 4; ++i) s2 = ffma2(q2[i], __bfloat1622float2(k2[i]), s2);
+                  sc[k] = s2.x + s2.y;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int off = 1; off < 8; off <<= 1)
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], off);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  if (j0 + k * KR + kgrp > t) sc[k] = -INFINITY;
+                const float m_new = fmaxf(fmaxf(m_run, fmaxf(sc[0], sc[1])), fmaxf(sc[2], sc[3]));
+                const float m_ref = m_new > -INFINITY ? m_new : 0.f;  // a group that has seen no key yet keeps its zeros
+                const float corr = ex2_approx(m_run - m_ref);         // 0 when m_run = -inf
+                l_run *= corr;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) o2[i] = fmul2(o2[i], make_float2(corr, corr));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  const float pj = ex2_approx(sc[k] - m_ref);  // 0 for a masked key
+                  l_run += pj;
+                  const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&vn[k]);
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) o2[i] = ffma2(make_float2(pj, pj), __bfloat1622float2(v2[i]), o2[i]);
+                }
+                m_run = m_new;
+                __syncwarp();
+              }
+              float o[8];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                o[2 * i] = o2[i].x;
+                o[2 * i + 1] = o2[i].y;
+              }
+              // the warp's four groups, then (through shared memory) the sample's warps
+              const float mw = fmaxf(fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 8)),
+                                     fmaxf(__shfl_xor_sync(0xffffffffu, m_run, 16), __shfl_xor_sync(0xffffffffu, m_run, 24)));
+              const float f = mw > -INFINITY ? ex2_approx(m_run - mw) : 0.f;
+              l_run *= f;
+              l_run += __shfl_xor_sync(0xffffffffu, l_run, 8);
+              l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) o[i] *= f;
+#pragma unroll
+              for (int off = 8; off < 32; off <<= 1)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[i] += __shfl_xor_sync(0xffffffffu, o[i], off);
+              float* mg = s_merge + (p * NWARPS + warp) * 72;
+              if (lane < 8) {
+                *reinterpret_cast<float4*>(mg + 8 * lane) = make_float4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<float4*>(mg + 8 * lane + 4) = make_float4(o[4], o[5], o[6], o[7]);
+                if (lane == 0) { mg[64] = mw; mg[65] = l_run; }
+              }
+              __syncwarp();
+            }
+            cbar();
+#pragma unroll 1
+            for (int i = tid; i < mine * 8 * CS; i += NTHREADS) {  // all-gather: (receiving CTA, eight channels, sample)
+              const int peer = i & (CS - 1), c8 = (i / CS) & 7, p = i / (8 * CS);
+              const float* mg = s_merge + p * NWARPS * 72;
+              float mx = mg[64];
+#pragma unroll
+              for (int k = 1; k < NWARPS; ++k) mx = fmaxf(mx, mg[k * 72 + 64]);
+              float den = 0.f, num[8];
+#pragma unroll
+              for (int z = 0; z < 8; ++z) num[z] = 0.f;
+#pragma unroll 4
+              for (int k = 0; k < NWARPS; ++k) {
+                const float e = ex2_approx(mg[k * 72 + 64] - mx);  // 0 for a warp without keys
+                den = fmaf(e, mg[k * 72 + 65], den);
+                const float4 a = *reinterpret_cast<const float4*>(mg + k * 72 + 8 * c8);
+                const float4 b = *reinterpret_cast<const float4*>(mg + k * 72 + 8 * c8 + 4);
+                num[0] = fmaf(e, a.x, num[0]); num[1] = fmaf(e, a.y, num[1]); num[2] = fmaf(e, a.z, num[2]); num[3] = fmaf(e, a.w, num[3]);
+                num[4] = fmaf(e, b.x, num[4]); num[5] = fmaf(e, b.y, num[5]); num[6] = fmaf(e, b.z, num[6]); num[7] = fmaf(e, b.w, num[7]);
+              }
+              const float inv = 1.f / den;
+              st_async4(peer_addr(sb + C::ACT + swz128(r * bl + p, c8), peer), pack_bf16(num[0] * inv, num[1] * inv),
+                        pack_bf16(num[2] * inv, num[3] * inv), pack_bf16(num[4] * inv, num[5] * inv), pack_bf16(num[6] * inv, num[7] * inv),
+                        peer_addr(bar(B_ALL0), peer));
+            }
+          }
+        } else {
+          // ---------------------------------------------------------------- bias + GELU
+          {  // reduce-scatter: warp w holds units 32 w .. of the cluster's 256, one sample per column
+            const int unit = warp * 32 + lane;
+            float* stg = reinterpret_cast<float*>(smem + C::STG) + (unit / UPC) * nb * UPC + unit % UPC;
+#pragma unroll 1
+            for (int b0 = 0; b0 < nb; b0 += 8) {
+              float v[8];
+              tmem_cols8(t_lane + b0, v);
+#pragma unroll
+              for (int b = 0; b < 8; ++b)
+                if (b0 + b < nb) stg[(b0 + b) * UPC] = v[b];
+            }
+            tcgen05_fence_before();
+          }
+          const float4 bias0 = __ldg(reinterpret_cast<const float4*>(ly->b_1 + c * UNITS + r * UPC + u8));
+          const float4 bias1 = __ldg(reinterpret_cast<const float4*>(ly->b_1 + c * UNITS + r * UPC + u8 + 4));
+          fence_proxy_async_smem();
+          cbar();
+          if (tid < CS)
+            copy_to_peer(peer_addr(sb + C::RECV + r * RT * UPC * 4, tid), sb + C::STG + tid * nb * UPC * 4, (uint32_t)(nb * UPC * 4),
+                         peer_addr(bar(B_RECV1), tid));
+          __syncwarp();
+          meet(B_RECV1, lp);
+#pragma unroll 1
+          for (int b = fb; b < nb; b += FB) {
+            const float* src = reinterpret_cast<const float*>(smem + C::RECV) + b * UPC + u8;
+            float4 x = bias0, y = bias1;
+#pragma unroll
+            for (int k = 0; k < CS; ++k) {
+              const float4 e = *reinterpret_cast<const float4*>(src + k * RT * UPC), f = *reinterpret_cast<const float4*>(src + k * RT * UPC + 4);
+              x.x += e.x; x.y += e.y; x.z += e.z; x.w += e.w;
+              y.x += f.x; y.y += f.y; y.z += f.z; y.w += f.w;
+            }
+            const float2 g0 = gelu_erf_fast2(make_float2(x.x, x.y)), g1 = gelu_erf_fast2(make_float2(x.z, x.w));
+            const float2 g2 = gelu_erf_fast2(make_float2(y.x, y.y)), g3 = gelu_erf_fast2(make_float2(y.z, y.w));
+            const uint32_t w0 = pack_bf16(g0.x, g0.y), w1 = pack_bf16(g1.x, g1.y), w2 = pack_bf16(g2.x, g2.y), w3 = pack_bf16(g3.x, g3.y);
+            const int unit = r * UPC + u8;  // operand tile unit / 64, 16-byte piece (unit % 64) / 8
+            const uint32_t off = sb + C::ACT + (unit >> 6) * (RT * 128) + swz128(b, (unit & 63) >> 3);
+#pragma unroll
+            for (int k = 0; k < CS; ++k) st_async4(peer_addr(off, k), w0, w1, w2, w3, peer_addr(bar(B_ALL1), k));
+          }
+        }
+        // ------------------------------------------------------------------ output projection and this cluster's partial rows
+        __syncwarp();
+        if (warp == 0) {
+          await(B_ALL0 + mlp, lp, TFERR_WAIT_FULL);
+          fence_proxy_async_smem();  // the tiles were written through the generic proxy
+#pragma unroll 1
+          for (int u = 0; u < (mlp ? 4 : 1); ++u) {
+            const uint32_t w = take(u);
+            tcgen05_fence_after();
+            if (elect_one()) {
+#pragma unroll
+              for (int z = 0; z < C::MT; ++z) mma(tmem + (2 + z) * RT, w + z * 16384, sb + C::ACT + u * (RT * 128), u > 0);
+              release(u);
+              if (u == (mlp ? 3 : 0)) umma_commit(bar(B_OUT0 + mlp));
+            }
+            __syncwarp();
+          }
+          await(B_OUT0 + mlp, lp, TFERR_WAIT_TMEM_FULL);
+          tcgen05_fence_before();
+        }
+        advance(mlp ? 4 : 1);
+        cbar();
+        tcgen05_fence_after();
+        if ((warp & 3) * 32 < CW) {  // accumulator lane = column, column = sample; warps 4-7: the second output tile or half of the samples
+          constexpr int NB = C::MT == 2 ? RT : RT / 2;
+          const int c0 = C::MT == 2 ? 0 : (warp >> 2) * NB, m = C::MT == 2 ? warp >> 2 : 0;
+          unsigned long long* out = xpart + ((size_t)c0 * HEADS + c) * D + r * CW + m * 128 + (warp & 3) * 32 + lane;
+#pragma unroll 1
+          for (int b0 = 0; b0 < NB && c0 + b0 < nb; b0 += 8) {
+            float v[8];
+            tmem_cols8(tmem + (2 + m) * RT + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(c0 + b0), v);
+#pragma unroll
+            for (int b = 0; b < 8; ++b)
+              if (c0 + b0 + b < nb) ll_store(out + (size_t)(b0 + b) * HEADS * D, __float_as_uint(v[b]), seq);
+          }
+          tcgen05_fence_before();
+        }
+        __syncwarp();
+      }
+      // ==================================================================== head and update of the own rows
+      const int bad = *reinterpret_cast<volatile int*>(err);  // looked at when the next step begins
+      if (own > 0) {
+        constexpr int KO = N1 == 4 ? 2 : 4;
+        const int n2 = 2 * Dt, hs = tid & 7, og = tid >> 3;
+        if (tid == 0 && alive) mbar_arrive_expect_tx(bar(B_HEAD), (uint32_t)(CS * own * n2 * 4));
+        __syncwarp();
+        float v_first = 0.f;  // operands of this thread's value of the first row: requested before the head is done
+        float2 b_first = make_float2(0.f, 0.f);
+        if (tid < Dt) {
+          v_first = job.v[token_at(0, t + 1) + tid];
+          b_first = __ldg(reinterpret_cast<const float2*>(job.b_out + 2 * tid));
+        }
+#pragma unroll 1
+        for (int n0 = 0; n0 < n2; n0 += 32 * KO) {  // eight lanes share an output, KO outputs per lane group
+          uint4 w[KO][N1];
+#pragma unroll
+          for (int k = 0; k < KO; ++k)
+#pragma unroll
+            for (int z = 0; z < N1; ++z) {
+              const int n = n0 + k * 32 + og;
+              w[k][z] = make_uint4(0u, 0u, 0u, 0u);
+              if (n < n2) w[k][z] = __ldg(reinterpret_cast<const uint4*>(job.w_out + (size_t)n * D + r * CW + z * 64 + hs * 8));
+            }
+#pragma unroll 1
+          for (int row = 0; row < own; ++row) {
+            float acc[KO];
+#pragma unroll
+            for (int k = 0; k < KO; ++k) acc[k] = 0.f;
+#pragma unroll
+            for (int z = 0; z < N1; ++z) {
+              const float4 x0 = *reinterpret_cast<const float4*>(s_xn + row * CW + z * 64 + hs * 8);
+              const float4 x1 = *reinterpret_cast<const float4*>(s_xn + row * CW + z * 64 + hs * 8 + 4);
+#pragma unroll
+              for (int k = 0; k < KO; ++k) {
+                const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&w[k][z]);
+                const float2 c0 = __bfloat1622float2(w2[0]), c1 = __bfloat1622float2(w2[1]);
+                const float2 c2 = __bfloat1622float2(w2[2]), c3 = __bfloat1622float2(w2[3]);
+                acc[k] = fmaf(x0.x, c0.x, acc[k]); acc[k] = fmaf(x0.y, c0.y, acc[k]);
+                acc[k] = fmaf(x0.z, c1.x, acc[k]); acc[k] = fmaf(x0.w, c1.y, acc[k]);
+                acc[k] = fmaf(x1.x, c2.x, acc[k]); acc[k] = fmaf(x1.y, c2.y, acc[k]);
+                acc[k] = fmaf(x1.z, c3.x, acc[k]); acc[k] = fmaf(x1.w, c3.y, acc[k]);
+              }
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+              for (int k = 0; k < KO; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+            if (hs < CS) {
+              const uint32_t dst = peer_addr(sb + C::RECV + ((r * C::RPC + row) * n2 + n0 + og) * 4, hs), pbar = peer_addr(bar(B_HEAD), hs);
+#pragma unroll
+              for (int k = 0; k < KO; ++k)
+                if (n0 + k * 32 + og < n2) st_async1(dst + k * 128, acc[k], pbar);
+            }
+            __syncwarp();
+          }
+        }
+        meet(B_HEAD, (uint32_t)(t & 1));
+#pragma unroll 1
+        for (int row = 0; row < own; ++row) {
+          const size_t e = token_at(row, t + 1);
+#pragma unroll 1
+          for (int cc = tid; cc < Dt; cc += NTHREADS) {
+            const bool pre = cc == tid;
+            const float vv = pre && row == 0 ? v_first : job.v[e + cc];
+            float2 o = pre ? b_first : __ldg(reinterpret_cast<const float2*>(job.b_out + 2 * cc));  // (mu~, alpha~) of value cc
+#pragma unroll
+            for (int k = 0; k < CS; ++k) {
+              const float2 y = *reinterpret_cast<const float2*>(smem + C::RECV + ((k * C::RPC + row) * n2 + 2 * cc) * 4);
+              o.x += y.x;
+              o.y += y.y;
+            }
+            const float x = fmaf(vv, expf(o.y), o.x);  // Eq. 5
+            s_tok[row * Dt + cc] = x;
+            if (r == 0) job.u[e + cc] = x;
+          }
+        }
+      }
+      if (tid == 0) *s_bad = bad;
+    }
+  }
+
+  // every copy into this CTA has been waited for; the cluster meets before anyone leaves
+  tcgen05_fence_before();
+  __syncthreads();
+  if (warp == 1 && *reinterpret_cast<volatile int*>(err) != 0) {  // a wait gave up: let copies and MMAs in flight drain
+    unsigned long long t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
+  }
+  cluster_sync();
+  if (warp == 1) {
+    tcgen05_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM) : "memory");
+  }
+}
+
+}  // namespace seqp
