@@ -27,6 +27,7 @@
 #include "gemm_tc2.cuh"
 #include "kernels_simt.cuh"
 #include "seq_decode.cuh"
+#include "seq_persist.cuh"
 
 // ------------------------------------------------------------------------------------------------
 // errors
@@ -206,6 +207,12 @@ struct tf_model {
   // fence + ticket + fence of the last arriver and its one-CTA reduction cost more than the kernel boundary and the
   // many-CTA consumer kernel they replace.
   bool seq_fin = false;
+  // bf16 engine: blocks decoded by one cooperative launch (seq_persist.cuh)
+  std::vector<seqp::Layer*> seqp_layers;       // per block, device memory
+  int seqp_groups[2] = {0, 0};                 // groups of 16 / 32 samples that fit the GPU side by side (0: not eligible)
+  uint32_t seqp_seq = 1;                       // sequence number of the next exchange
+  unsigned long long *seqp_part = nullptr, *seqp_row = nullptr;
+  bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
   int seq_attn_threads = 0;  // TARFLOW_SEQ_ATTN_THREADS=128|256: CTA size of the step attention (0 = by the number of CTAs)
   int seq_kbn_force = 0;     // TARFLOW_SEQ_KBN
   // Jacobi sweeps over few rows are replayed from graphs: one per (block, single-term slots, two-term slots, buffers)
@@ -1078,7 +1085,129 @@ static int run_sequential_chain(tf_model* m, const SeqCtx& cx, int g, const int*
   return TF_OK;
 }
 
+// ---- blocks decoded by one cooperative launch
+using SeqpKernel = void (*)(seqp::Job);
+struct SeqpShape { SeqpKernel kern; int smem, cs, heads; size_t part, row; };  // exchange words per group
+template <int D, int RT>
+static SeqpShape seqp_shape() {
+  using C = seqp::Cfg<D, RT>;
+  return {seqp::seq_block_kernel<D, RT>, C::TOTAL, C::CS, C::HEADS, (size_t)RT * C::HEADS * D, (size_t)RT * D / 2};
+}
+static SeqpShape seqp_shape_of(int d, int rt) {
+  if (rt == 16) return d == 1024 ? seqp_shape<1024, 16>() : d == 512 ? seqp_shape<512, 16>() : d == 256 ? seqp_shape<256, 16>() : seqp_shape<128, 16>();
+  return d == 1024 ? seqp_shape<1024, 32>() : d == 512 ? seqp_shape<512, 32>() : d == 256 ? seqp_shape<256, 32>() : seqp_shape<128, 32>();
+}
+
+// launches (max_clusters == nullptr), or asks how many clusters fit the GPU side by side
+static int seqp_launch(tf_model* m, const SeqpShape& sh, int groups, const seqp::Job* job, int* max_clusters) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(groups * sh.heads * sh.cs);
+  lc.blockDim = dim3(seqp::NTHREADS + 32);
+  lc.dynamicSmemBytes = sh.smem;
+  lc.stream = m->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = sh.cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;  // the clusters wait on one another
+  at[1].val.cooperative = 1;
+  lc.attrs = at;
+  lc.numAttrs = max_clusters ? 1 : 2;
+  if (max_clusters) {
+    if (cudaOccupancyMaxActiveClusters(max_clusters, sh.kern, &lc) != cudaSuccess) {
+      cudaGetLastError();
+      *max_clusters = 0;
+    }
+    return TF_OK;
+  }
+  const cudaError_t e = cudaLaunchKernelEx(&lc, sh.kern, *job);
+  if (e != cudaSuccess) return fail(TF_ECUDA, "seq_block_kernel launch failed: %s", cudaGetErrorString(e));
+  return TF_OK;
+}
+
+// at load: whether the shape fits, the layers' tables, the exchange buffers
+static int seqp_setup(tf_model* m) {
+  const int d = m->d;
+  if ((d != 128 && d != 256 && d != 512 && d != 1024) || m->hid != 4 * d || m->hd != 64 || m->D > (d == 1024 ? 256 : 128)) return TF_OK;
+  size_t part = 0, row = 0;
+  for (int i = 0; i < 2; ++i) {
+    const SeqpShape sh = seqp_shape_of(d, 16 << i);
+    CU_OK(cudaFuncSetAttribute(sh.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem));
+    int n = 0;
+    TF_TRY(seqp_launch(m, sh, 1, nullptr, &n));
+    int groups = n / sh.heads;
+    if (groups > m->cfg.max_batch) groups = m->cfg.max_batch;
+    m->seqp_groups[i] = groups;
+    if (groups * sh.part > part) part = groups * sh.part;
+    if (groups * sh.row > row) row = groups * sh.row;
+  }
+  if (m->seqp_groups[0] == 0 || m->seqp_groups[1] == 0) return TF_OK;
+  TF_TRY(dev_alloc(m, &m->seqp_part, part));
+  TF_TRY(dev_alloc(m, &m->seqp_row, row));
+  CU_OK(cudaMemset(m->seqp_part, 0, part * sizeof(*m->seqp_part)));
+  CU_OK(cudaMemset(m->seqp_row, 0, row * sizeof(*m->seqp_row)));
+  for (BlockW& bw : m->blocks) {
+    std::vector<seqp::Layer> table;
+    for (LayerW& lw : bw.layers) {
+      seqp::Layer ly;
+      TF_TRY(make_map_bf16(&ly.qkv, lw.w_qkv.w, lw.w_qkv.N, lw.w_qkv.K, 64));
+      TF_TRY(make_map_bf16(&ly.wo, lw.w_o.w, lw.w_o.N, lw.w_o.K, 64));
+      TF_TRY(make_map_bf16(&ly.w1, lw.w_1.w, lw.w_1.N, lw.w_1.K, 64));
+      TF_TRY(make_map_bf16(&ly.w2, lw.w_2.w, lw.w_2.N, lw.w_2.K, 64));
+      ly.ln1_g = lw.ln1_g; ly.ln1_b = lw.ln1_b; ly.b_qkv = lw.b_qkv; ly.b_o = lw.b_o;
+      ly.ln2_g = lw.ln2_g; ly.ln2_b = lw.ln2_b; ly.b_1 = lw.b_1; ly.b_2 = lw.b_2;
+      table.push_back(ly);
+    }
+    seqp::Layer* dev = nullptr;
+    TF_TRY(dev_alloc(m, &dev, table.size()));
+    CU_OK(cudaMemcpy(dev, table.data(), table.size() * sizeof(seqp::Layer), cudaMemcpyHostToDevice));
+    m->seqp_layers.push_back(dev);
+  }
+  return TF_OK;
+}
+
+// Batches that need more than one launch go to the chain of kernels, whose cost hardly grows with the batch (width 1024,
+// 96 samples: 135 ms in two launches).
+static bool seqp_on(const tf_model* m, int B) {
+  return !m->seqp_layers.empty() && m->seq_use_persist && m->seq_use_tc && !m->seq_fin && !m->seq_fuse_gelu && m->seq_fuse_tail < 0 &&
+         B <= 32 * m->seqp_groups[1];
+}
+
+static int run_sequential_persistent(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
+  const BlockW& bw = m->blocks[g];
+  const int L = m->L, D = m->D, nl = m->cfg.n_layers, n_steps = L - 1;
+  constexpr size_t kL2Half = 64u << 20;  // what may be expected to stay in L2 from one step to the next
+  const size_t weights = (size_t)nl * 12 * m->d * m->d * sizeof(bf16);
+  // All groups that fit, however few samples each (16 samples at width 512: 12.4 ms with four groups, 16.9 with one); the
+  // 16-sample kernel (shorter exchanges) where that is enough.
+  const int i = B <= 16 * m->seqp_groups[0] ? 0 : 1;
+  const SeqpShape sh = seqp_shape_of(m->d, 16 << i);
+  const int want = B < m->seqp_groups[i] ? B : m->seqp_groups[i];
+  seqp::Job job = {};
+  job.rows = (B + want - 1) / want;
+  job.layers = m->seqp_layers[g];
+  job.lnf_g = bw.lnf_g; job.lnf_b = bw.lnf_b; job.w_in_t = bw.w_in_t; job.b_in = bw.b_in; job.pos = bw.pos; job.cls = bw.cls;
+  job.b_out = bw.b_out; job.w_out = reinterpret_cast<const bf16*>(bw.w_out.w);
+  job.v = v; job.u = u; job.labels = labels;
+  job.kc = reinterpret_cast<bf16*>(m->kcache); job.vc = reinterpret_cast<bf16*>(m->vcache);
+  job.layer_stride = (size_t)m->cfg.max_batch * L * m->d;
+  job.xpart = m->seqp_part; job.xrow = m->seqp_row;
+  job.n_layers = nl; job.B = B; job.L = L; job.Dt = D; job.reversed = g & 1;
+  job.seq0 = m->seqp_seq;
+  m->seqp_seq += (uint32_t)((2 * nl + 1) * n_steps + 1);
+  job.prefetch_w = weights > kL2Half;
+  job.prefetch_kv = (size_t)nl * B * L * m->d * 2 * sizeof(bf16) > kL2Half;
+  job.scale_log2e = 1.4426950408889634f / sqrtf((float)m->hd);
+  job.err = m->err;
+  m->cur_rows = (int64_t)B * n_steps;
+  m->pre(KC_SEQ_BLOCK);
+  TF_TRY(seqp_launch(m, sh, (B + job.rows - 1) / job.rows, &job, nullptr));
+  m->post(KC_SEQ_BLOCK);
+  return TF_OK;
+}
+
 static int run_sequential_block_bf16(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
+  if (seqp_on(m, B)) return run_sequential_persistent(m, g, B, labels, v, u);
   const int n_steps = m->L - 1;
   cudaStream_t user = m->stream;
   const bool direct = (m->prof_on && m->prof_mode == 1) || !m->use_graphs;
@@ -1905,6 +2034,8 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
     TF_TRY(dev_alloc(m, &m->seq_stats, (size_t)tf_model::MAX_CHAINS * 16 * B));
     if (const char* e = getenv("TARFLOW_SWEEP_GRAPH_ROWS")) m->sweep_graph_rows = atoll(e);
     if (const char* e = getenv("TARFLOW_GRAPHS")) m->use_graphs = atoi(e) != 0;
+    TF_TRY(seqp_setup(m));
+    if (const char* e = getenv("TARFLOW_SEQ_PERSIST")) m->seq_use_persist = atoi(e) != 0;
   }
   if (c.dtype == 0) {
     CU_OK(cudaFuncSetAttribute(f32::attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, f32::attention_smem_floats(128) * (int)sizeof(float)));
