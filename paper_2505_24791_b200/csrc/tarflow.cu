@@ -1178,8 +1178,8 @@ static int run_sequential_persistent(tf_model* m, int g, int B, const int* label
   const int L = m->L, D = m->D, nl = m->cfg.n_layers, n_steps = L - 1;
   constexpr size_t kL2Half = 64u << 20;  // what may be expected to stay in L2 from one step to the next
   const size_t weights = (size_t)nl * 12 * m->d * m->d * sizeof(bf16);
-  // All groups that fit, however few samples each (16 samples at width 512: 12.4 ms with four groups, 16.9 with one); the
-  // 16-sample kernel (shorter exchanges) where that is enough.
+  // All groups that fit, however few samples each (the groups run side by side and a step's length grows with a group's
+  // samples); the 16-sample kernel (shorter exchanges) where that is enough.
   const int i = B <= 16 * m->seqp_groups[0] ? 0 : 1;
   const SeqpShape sh = seqp_shape_of(m->d, 16 << i);
   const int want = B < m->seqp_groups[i] ? B : m->seqp_groups[i];
