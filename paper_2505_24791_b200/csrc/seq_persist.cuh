@@ -19,8 +19,10 @@
 // Per half layer:   gather rows -> tcgen05 (weights as the M operand) -> reduce-scatter -> attention | GELU -> all-gather ->
 //                   tcgen05 -> partial rows -> owner: residual + LayerNorm -> publish
 // Weights travel through a ring of TMA slots in the order in which they are used, ahead of the activations (a warp of its own
-// refills what has been used); where a block's weights exceed L2 they (and the next layer's cache rows) are prefetched into
-// L2 a layer ahead.  A step's head, update and embedding are done by the row's owner cluster on the CUDA cores.
+// refills what has been used), and so do, between a layer's first and second projection, the keys and values of earlier
+// tokens: up to 160 KB per CTA are on their way, where loads of the attending warps kept 32 KB (width 1024, 64 samples:
+// 36 of a block's 85 ms went to attention).  Where a block's weights exceed L2 they are prefetched into L2 a layer ahead.
+// A step's head, update and embedding are done by the row's owner cluster on the CUDA cores.
 // Clusters are of 4 CTAs (2 at width 128): with most of an SM's shared memory per CTA, 33 of those fit the GPU side by side,
 // but only 15 of 8, and width 1024 has 16 heads.
 // Control flow is uniform per warp and visibly so to the compiler (rank from blockIdx, warp index and flags through a
@@ -31,6 +33,7 @@
 #pragma once
 #include "common.cuh"
 #include "gemm_tc.cuh"
+#include "attention_mma.cuh"
 
 namespace seqp {
 
@@ -44,17 +47,18 @@ struct __align__(128) Layer {
   const float *ln1_g, *ln1_b, *b_qkv, *b_o, *ln2_g, *ln2_b, *b_1, *b_2;
 };
 struct Job {
+  CUtensorMap kmap, vmap;           // the caches as rows of 64, in boxes of 32 rows
   const Layer* layers;
   const float *lnf_g, *lnf_b, *w_in_t, *b_in, *pos, *cls, *b_out, *v;
   const bf16* w_out;
   float* u;
   const int* labels;
   bf16 *kc, *vc;
-  size_t layer_stride;              // cache elements per layer
+  int layer_rows;                   // cache rows of 64 per layer
   unsigned long long *xpart, *xrow; // exchange buffers
   int n_layers, B, rows, L, Dt, reversed;  // rows: samples per group (a group = one set of clusters); Dt: token dimension
   uint32_t seq0;
-  int prefetch_w, prefetch_kv;
+  int prefetch_w;
   float scale_log2e;
   int* err;
 };
@@ -72,25 +76,32 @@ struct Cfg {
   static constexpr int GW = QN * RPC / 32;         // warps of group 0: they hold the residual stream
   static constexpr int SPR = QN > 32 ? QN / 32 : 1, NE = CS * SPR, CE = CW / SPR;  // statistics of a row: NE entries of CE columns
   static constexpr int MT = N1 > 2 ? N1 / 2 : 1;   // 128-row output tiles of a CTA
-  static constexpr int NSLOT_MAX = (RT == 16 ? 163840 : 131072) / UNIT, NSLOT = NSLOT_MAX < 12 ? NSLOT_MAX : 12;
+  // at most 10 slots: the cache rows of a step are then requested after the first MLP product of the layer's last step, by
+  // when that step's row is in memory (with one layer there are 12 weight units in between)
+  static constexpr int NSLOT_MAX = (RT == 16 ? 163840 : 131072) / UNIT, NSLOT = NSLOT_MAX < 10 ? NSLOT_MAX : 10;
+  // cache rows of one sample travel in units of KPU keys, KVS slots each (their keys, then their values)
+  static constexpr int KVS = N1 == 1 ? 2 : 1, KPU = KVS * UNIT / 256, WPU = KPU / 16;
   static constexpr int MAXDT = D == 1024 ? 256 : 128;
   static constexpr int RING = 0, ACT = NSLOT * UNIT;  // activation tiles; a 64-row weight tile read as 128 rows may run on into them
   static constexpr int STG = ACT + 4 * RT * 128;      // what is sent to the peers, then what comes from them
   static constexpr int RECV = STG + RT * 1024;
   static constexpr int MERGE = RECV;                  // [sample][warp]: output, maximum, sum; q, k, v have left the place by then
-  static constexpr int QKV = RECV + (RT * 1024 > BL * NWARPS * 288 ? RT * 1024 : BL * NWARPS * 288);  // per sample: q fp32 [64], k, v bf16 [64]
-  static constexpr int SUM = QKV + BL * 512;
+  static constexpr int QKV = RECV + (RT * 1024 > BL * NWARPS * 288 ? RT * 1024 : BL * NWARPS * 288);
+  static constexpr int QROW = 640;                    // per sample, bf16 [64] each: q in three parts, the new k, the new v
+  static constexpr int ZERO = QKV + BL * QROW;        // 128 zero bytes
+  static constexpr int SUM = ZERO + 128;
   static constexpr int XN = SUM + (SGC - 1) * RPC * QN * 16;
   static constexpr int TOK = XN + RPC * CW * 4;
   static constexpr int STAT = TOK + RPC * MAXDT * 4;
   static constexpr int BIAS = STAT + RPC * NE * 8;
   static constexpr int BARS = BIAS + 192 * 4;
-  static constexpr int NBARS = 2 * NSLOT + 10;
+  static constexpr int NBARS = 3 * NSLOT + 10;
   static constexpr int TOTAL = BARS + NBARS * 8 + 32 + 1024;
   static constexpr uint32_t TMEM = RT == 16 ? 64 : 128;
   static_assert(sizeof(Layer) % sizeof(CUtensorMap) == 0, "tables of layers are stepped in tensor maps");
   static_assert(QN * RPC * SG == NTHREADS && SG * NSL == HEADS && NSL % NA == 0 && SGC > 1 && QN * RPC % 32 == 0 && NSLOT >= 4,
                 "thread layout of the residual rows");
+  static_assert(TOTAL <= 227 * 1024, "shared memory of a CTA");
   static_assert(N1 > 1 || NSLOT % 2 == 0, "pairs of 64-row tiles must not be split by the ring's end");
 };
 
@@ -191,79 +202,124 @@ __device__ __forceinline__ void tmem_cols8(uint32_t taddr, float (&v)[8]) {
 __device__ __forceinline__ void prefetch_tile(const CUtensorMap* map, int x, int y) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
-__device__ __forceinline__ void prefetch_bytes(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 o = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&o);
 }
 
-// The weight ring's filling side (one thread): where it stands in the order of use.
-struct Feed {
-  int t = 0, layer = 0, unit = 0, slot = 0;
-  uint32_t phase = 0;
-};
-// requests one unit after the other (a layer is 12 of them), each when the products that read its slot's last contents are done
+// The ring's filling side (one thread): requests one unit after the other in the order of use, each when its slot's last contents
+// have been used: weights by the products that read them, cache rows by the WPU warps that share a unit's tiles.
 template <int D, int RT>
-__device__ __forceinline__ void feed(const Job& job, Feed& f, uint32_t ring, uint32_t bars, int r, int c, bool prefetch_w, int mine,
-                                     size_t cache_row0) {
+__device__ __forceinline__ void feed(const Job& job, uint32_t ring, uint32_t bars, int r, int c, bool prefetch_w, int mine, int cache_row0) {
   using C = Cfg<D, RT>;
   constexpr int N1 = C::N1, CW = C::CW;
   const int n_steps = job.L - 1;
-#pragma unroll 1
-  while (f.t < n_steps) {
-    if (!wait_idle(bars + 8u * (C::NSLOT + f.slot), f.phase ^ 1u, job.err, TFERR_WAIT_EMPTY)) return;
-    const Layer* ly = job.layers + f.layer;
-    const int nx = f.layer + 1 < job.n_layers ? f.layer + 1 : 0;
-    const bool more = nx > 0 || f.t + 1 < n_steps;
-    const uint32_t full = bars + 8u * f.slot;
-    mbar_arrive_expect_tx(full, C::UNIT);
-    const int u = f.unit;
-#pragma unroll 1
-    for (int z = 0; z < N1; ++z) {  // the unit's 8 KB tiles
-      const CUtensorMap* map;
-      int x, y;
-      if (u < 2) {  // per slab: q, k
-        const int i = u * N1 + z;
-        map = &ly->qkv;
-        x = (r * N1 + (i >> 1)) * 64;
-        y = (i & 1) * D + c * HD;
-      } else if (u == 2) {  // v of every slab
-        map = &ly->qkv;
-        x = (r * N1 + z) * 64;
-        y = 2 * D + c * HD;
-      } else if (u == 3) {
-        map = &ly->wo;
-        x = c * HD;
-        y = r * CW + z * 64;
-      } else if (u < 8) {  // per slab: four blocks of 64 hidden units
-        const int i = (u - 4) * N1 + z;
-        map = &ly->w1;
-        x = (r * N1 + (i >> 2)) * 64;
-        y = c * UNITS + (i & 3) * 64;
-      } else {  // per slab of hidden units: the CTA's output rows
-        map = &ly->w2;
-        x = c * UNITS + (u - 8) * 64;
-        y = r * CW + z * 64;
+  int slot = 0;
+  uint32_t used = 0, rows_held = 0, phase_w = 0, phase_kv = 0;  // a bit per slot
+  auto acquire = [&](bool rows) {
+    const uint32_t bit = 1u << slot;
+    bool ok = true;
+    if (used & bit) {
+      if (rows_held & bit) {
+        ok = wait_idle(bars + 8u * (2 * C::NSLOT + slot), (phase_kv & bit) != 0, job.err, TFERR_WAIT_EMPTY);
+        phase_kv ^= bit;
+      } else {
+        ok = wait_idle(bars + 8u * (C::NSLOT + slot), (phase_w & bit) != 0, job.err, TFERR_WAIT_EMPTY);
+        phase_w ^= bit;
       }
-      tma_load_2d(ring + f.slot * C::UNIT + z * 8192, map, x, y, full);
-      if (prefetch_w && more) prefetch_tile(map + (nx - f.layer) * (int)(sizeof(Layer) / sizeof(CUtensorMap)), x, y);
     }
-    if (u == 4 && job.prefetch_kv && more && f.t > 0)
-      for (int p = 0; p < mine; ++p) {
-        const size_t at = nx * job.layer_stride + cache_row0 + (size_t)p * C::HEADS * job.L * HD;
-        prefetch_bytes(job.kc + at, (uint32_t)f.t * HD * 2);
-        prefetch_bytes(job.vc + at, (uint32_t)f.t * HD * 2);
+    used |= bit;
+    rows_held = rows ? rows_held | bit : rows_held & ~bit;
+    return ok;
+  };
+  auto next = [&]() { slot = slot + 1 == C::NSLOT ? 0 : slot + 1; };
+#pragma unroll 1
+  for (int t = 0; t < n_steps; ++t)
+#pragma unroll 1
+    for (int layer = 0; layer < job.n_layers; ++layer) {
+      const Layer* ly = job.layers + layer;
+      const int nx = layer + 1 < job.n_layers ? layer + 1 : 0;
+      const bool more = prefetch_w && (nx > 0 || t + 1 < n_steps);
+#pragma unroll 1
+      for (int u = 0; u < 12; ++u) {
+        if (u == 3) {
+#pragma unroll 1
+          for (int p = 0; p < mine; ++p)
+#pragma unroll 1
+            for (int j0 = 0; j0 < t; j0 += C::KPU) {
+              const int row = layer * job.layer_rows + cache_row0 + p * C::HEADS * job.L + j0;
+              const int boxes = ((t - j0 < C::KPU ? t - j0 : C::KPU) + 31) / 32;
+              if (!acquire(true)) return;
+              uint32_t at = ring + slot * C::UNIT, full = bars + 8u * slot;
+              mbar_arrive_expect_tx(full, boxes * (8192u / C::KVS));
+#pragma unroll 1
+              for (int b = 0; b < boxes; ++b) tma_load_2d(at + b * 4096, &job.kmap, 0, row + 32 * b, full);
+              next();
+              if (C::KVS == 2) {
+                if (!acquire(true)) return;
+                at = ring + slot * C::UNIT;
+                full = bars + 8u * slot;
+                mbar_arrive_expect_tx(full, boxes * 4096u);
+                next();
+              } else {
+                at += C::KPU * 128;
+              }
+#pragma unroll 1
+              for (int b = 0; b < boxes; ++b) tma_load_2d(at + b * 4096, &job.vmap, 0, row + 32 * b, full);
+            }
+        }
+        if (!acquire(false)) return;
+        const uint32_t full = bars + 8u * slot;
+        mbar_arrive_expect_tx(full, C::UNIT);
+#pragma unroll 1
+        for (int z = 0; z < N1; ++z) {  // the unit's 8 KB tiles
+          const CUtensorMap* map;
+          int x, y;
+          if (u < 2) {  // per slab: q, k
+            const int i = u * N1 + z;
+            map = &ly->qkv;
+            x = (r * N1 + (i >> 1)) * 64;
+            y = (i & 1) * D + c * HD;
+          } else if (u == 2) {  // v of every slab
+            map = &ly->qkv;
+            x = (r * N1 + z) * 64;
+            y = 2 * D + c * HD;
+          } else if (u == 3) {
+            map = &ly->wo;
+            x = c * HD;
+            y = r * CW + z * 64;
+          } else if (u < 8) {  // per slab: four blocks of 64 hidden units
+            const int i = (u - 4) * N1 + z;
+            map = &ly->w1;
+            x = (r * N1 + (i >> 2)) * 64;
+            y = c * UNITS + (i & 3) * 64;
+          } else {  // per slab of hidden units: the CTA's output rows
+            map = &ly->w2;
+            x = c * UNITS + (u - 8) * 64;
+            y = r * CW + z * 64;
+          }
+          tma_load_2d(ring + slot * C::UNIT + z * 8192, map, x, y, full);
+          if (more) prefetch_tile(map + (nx - layer) * (int)(sizeof(Layer) / sizeof(CUtensorMap)), x, y);
+        }
+        next();
       }
-    if (++f.slot == C::NSLOT) { f.slot = 0; f.phase ^= 1u; }
-    if (++f.unit == 12) {
-      f.unit = 0;
-      f.layer = nx;
-      if (nx == 0) ++f.t;
     }
-  }
+}
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t at) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(at) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t at) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(at) : "memory");
+}
+// x as the sum of three bf16: 24 bits, the whole fp32 mantissa
+__device__ __forceinline__ void split3(float x, float (&part)[3]) {
+  part[0] = __bfloat162float(__float2bfloat16_rn(x));
+  const float rest = x - part[0];
+  part[1] = __bfloat162float(__float2bfloat16_rn(rest));
+  part[2] = rest - part[1];
 }
 
 // grid: groups * HEADS clusters of CS CTAs (cooperative), 256 threads and a warp that moves the weights
@@ -280,17 +336,18 @@ seq_block_kernel(const __grid_constant__ Job job) {
   const int row0 = group * job.rows, nb = job.B - row0 < job.rows ? job.B - row0 : job.rows;  // this group's samples
   const int L = job.L, Dt = job.Dt, n_steps = L - 1, nl = job.n_layers;
   int* err = job.err;
-  auto bar = [&](int i) { return bars + 8u * (2 * C::NSLOT + i); };
+  auto bar = [&](int i) { return bars + 8u * (3 * C::NSLOT + i); };
   enum { B_IN0, B_IN1, B_RECV0, B_RECV1, B_ALL0, B_ALL1, B_OUT0, B_OUT1, B_STAT, B_HEAD };  // 0: attention half, 1: MLP half
   uint8_t* tail_mem = smem + C::BARS + C::NBARS * 8;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail_mem);
   volatile int* s_bad = reinterpret_cast<volatile int*>(tail_mem + 4);
 
   if (tid == 0) {
-    for (int i = 0; i < C::NBARS; ++i) mbar_init(bars + 8u * i, 1);
+    for (int i = 0; i < C::NBARS; ++i) mbar_init(bars + 8u * i, i / C::NSLOT == 2 ? C::WPU : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *s_bad = 0;
   }
+  if (tid < 8) *reinterpret_cast<uint4*>(smem + C::ZERO + 16 * tid) = make_uint4(0u, 0u, 0u, 0u);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM)
                  : "memory");
@@ -304,20 +361,17 @@ seq_block_kernel(const __grid_constant__ Job job) {
 
   // samples this CTA attends for: bl r .. bl r + mine - 1 of the group
   const int bl = (nb + CS - 1) / CS, mine = nb - r * bl < bl ? (nb - r * bl > 0 ? nb - r * bl : 0) : bl;
-  auto rows_of = [&](int p) { return ((size_t)(row0 + r * bl + p) * HEADS + c) * L * HD; };  // cache rows of (sample, head)
+  auto rows_of = [&](int p) { return ((row0 + r * bl + p) * HEADS + c) * L; };  // cache rows of (sample, head)
 
   if (warp == NWARPS) {
     // ==================================================================== weights
-    if (lane == 0) {
-      Feed fd;
-      feed<D, RT>(job, fd, sb + C::RING, bars, r, c, job.prefetch_w && group == 0, mine, rows_of(0));
-    }
+    if (lane == 0) feed<D, RT>(job, sb + C::RING, bars, r, c, job.prefetch_w && group == 0, mine, rows_of(0));
   } else {
     constexpr uint32_t idesc = make_idesc(RT);
-    // attention roles: the eight warps share every sample's keys (the same split whatever the batch), eight lanes share a key, four
-    // keys per lane group in flight
-    constexpr int KR = NWARPS * 4;  // keys apart in a lane group
-    const int sub = lane & 7, kgrp = warp * 4 + (lane >> 3);
+    // attention: a sample's keys are cut into tiles of 16, dealt out to eight sets whatever the batch; a set belongs to a warp.
+    // The operand rows of this lane: keys kr of a tile, values of keys vr (transposed on the way), parts of q
+    const int kr = lane & 15, vr = (lane & 7) + (lane >> 4) * 8;
+    const uint32_t k_piece = lane >> 4, v_piece = (lane >> 3) & 1, q_piece = lane >> 3;
     // hidden units this thread finishes: eight of them, samples fb, fb + FB, ...
     constexpr int FB = NTHREADS / (UPC / 8);
     const int u8 = (tid % (UPC / 8)) * 8, fb = tid / (UPC / 8);
@@ -519,30 +573,12 @@ seq_block_kernel(const __grid_constant__ Job job) {
           }
         }
         __syncwarp();
-        bf16 *kc = job.kc + (half >> 1) * job.layer_stride, *vc = job.vc + (half >> 1) * job.layer_stride;
-        uint4 kv[4], vv[4];  // rows of the cache in flight
-        auto fetch = [&](int p, int j0) {
-          const size_t base = rows_of(p) + sub * 8;
-          const bf16 *kr = kc + base, *vr = vc + base;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int j = j0 + k * KR + kgrp;
-            kv[k] = vv[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (j < t) {
-              kv[k] = __ldcg(reinterpret_cast<const uint4*>(kr + j * HD));
-              vv[k] = __ldcg(reinterpret_cast<const uint4*>(vr + j * HD));
-            }
-          }
-        };
         if (half == 1 && own > 0 && t + 1 < n_steps) {  // what the end of the step will read from memory: on its way to L2
           if (holder && my_row) prefetch_line(job.pos + (size_t)(t + 1) * D + col);
           const int per = (Dt + 31) / 32;
           if (tid < own * per) prefetch_line(job.v + token_at(tid / per, t + 1) + (tid % per) * 32);
         }
-        if (!mlp) {
-          if (tid < 192) s_bias[tid] = __ldg(ly->b_qkv + (tid >> 6) * D + c * HD + (tid & 63));
-          if (mine > 0) fetch(0, 0);  // rows of earlier tokens: on their way while q is computed
-        }
+        if (!mlp && tid < 192) s_bias[tid] = __ldg(ly->b_qkv + (tid >> 6) * D + c * HD + (tid & 63));
         {  // rows of the projection's input (this rank's columns) into swizzled [RT][64] operand tiles
           constexpr int IT = RT * QN / NTHREADS;
           unsigned long long w[IT][2];
@@ -652,104 +688,134 @@ seq_block_kernel(const __grid_constant__ Job job) {
                 const float4 y = *reinterpret_cast<const float4*>(src + k * C::BL * 192);
                 x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
               }
-              uint8_t* mem = smem + C::QKV + p * 512;
+              uint8_t* mem = smem + C::QKV + p * C::QROW;
               if (c4 < 16) {  // scores in base-2 units: softmax via exp2
-                *reinterpret_cast<float4*>(mem + 16 * c4) =
-                    make_float4(x.x * job.scale_log2e, x.y * job.scale_log2e, x.z * job.scale_log2e, x.w * job.scale_log2e);
+                float p0[3], p1[3], p2[3], p3[3];
+                split3(x.x * job.scale_log2e, p0);
+                split3(x.y * job.scale_log2e, p1);
+                split3(x.z * job.scale_log2e, p2);
+                split3(x.w * job.scale_log2e, p3);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) *reinterpret_cast<uint2*>(mem + k * 128 + 8 * c4) = make_uint2(pack_bf16(p0[k], p1[k]), pack_bf16(p2[k], p3[k]));
               } else {
                 const uint2 w2 = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-                *reinterpret_cast<uint2*>(mem + 256 + (c4 - 16) * 8) = w2;
-                *reinterpret_cast<uint2*>((c4 < 32 ? kc : vc) + rows_of(p) + (size_t)t * HD + (c4 & 15) * 4) = w2;
+                *reinterpret_cast<uint2*>(mem + 384 + (c4 - 16) * 8) = w2;
+                const size_t row = (size_t)(half >> 1) * job.layer_rows + rows_of(p) + t;
+                *reinterpret_cast<uint2*>((c4 < 32 ? job.kc : job.vc) + row * HD + (c4 & 15) * 4) = w2;
               }
             }
             cbar();
+            const int units = (t + C::KPU - 1) / C::KPU, tiles = t / 16 + 1, sets = tiles < NWARPS ? tiles : NWARPS;
 #pragma unroll 1
             for (int p = 0; p < mine; ++p) {
-              const uint8_t* mem = smem + C::QKV + p * 512;
-              float2 q2[4], o2[4];
-#pragma unroll
-              for (int i = 0; i < 4; i += 2) {
-                const float4 q4 = *reinterpret_cast<const float4*>(mem + sub * 32 + i * 8);
-                q2[i] = make_float2(q4.x, q4.y);
-                q2[i + 1] = make_float2(q4.z, q4.w);
-                o2[i] = o2[i + 1] = make_float2(0.f, 0.f);
+              // scores = K q and output = V^T p as 16 x 8 x 16 products; q and p are three columns (their bf16 parts) of the eight
+              const uint32_t mem = sb + C::QKV + p * C::QROW;
+              const int set = C::WPU == NWARPS ? warp : (warp + 4 * p) & 7;  // where a unit has four tiles the other warps begin the next sample
+              uint32_t qf[2][4];
+              {
+                const int n = lane & 7;
+                const uint32_t at = n < 3 ? mem + n * 128 : sb + C::ZERO;
+                ldsm4(qf[0], at + q_piece * 16);
+                ldsm4(qf[1], at + 64 + q_piece * 16);
               }
-              float m_run = -INFINITY, l_run = 0.f;
+              float o[4][4], m_run = -INFINITY, l_run = 0.f;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+              const int tile_end = tiles > units * C::WPU ? tiles : units * C::WPU;
 #pragma unroll 1
-              for (int j0 = 0; j0 <= t; j0 += 4 * KR) {
-                uint4 kn[4], vn[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  kn[k] = kv[k];
-                  vn[k] = vv[k];
+              for (int tile = set; tile < tile_end; tile += NWARPS) {
+                const int unit = tile / C::WPU, pos = slot + (p * units + unit) * C::KVS, wrap = pos / C::NSLOT, at = pos - wrap * C::NSLOT;
+                const int av = C::KVS == 1 ? at : at + 1 == C::NSLOT ? 0 : at + 1;  // the values' slot
+                if (unit < units) {
+                  const uint32_t parity = ring_parity ^ (uint32_t)(wrap & 1);
+                  if (!wait_bar(bars + 8u * at, parity, err, TFERR_WAIT_FULL)) alive = false;
+                  if (C::KVS == 2 && !wait_bar(bars + 8u * av, parity ^ (uint32_t)(av == 0), err, TFERR_WAIT_FULL)) alive = false;
+                  __syncwarp();
                 }
-                // the next round's rows (of the next sample after the last one) travel while this round is worked on
-                const bool on = j0 + 4 * KR <= t;
-                if (on || p + 1 < mine) fetch(on ? p : p + 1, on ? j0 + 4 * KR : 0);
-                float sc[4];
+                if (tile < tiles) {
+                  // rows that are not there (the last of them is the new token's) read the new row
+                  const uint32_t kbase = sb + C::RING + at * C::UNIT + (tile % C::WPU) * 2048;
+                  const uint32_t vbase = sb + C::RING + av * C::UNIT + (C::KVS == 1 ? C::KPU * 128 : 0) + (tile % C::WPU) * 2048;
+                  const bool kin = tile * 16 + kr < t, vin = tile * 16 + vr < t;
+                  const uint32_t kat = kin ? kbase + kr * 128 : mem + 384, kx = kin ? kr & 7 : 0;
+                  const uint32_t vat = vin ? vbase + vr * 128 : mem + 512, vx = vin ? vr & 7 : 0;
+                  float sa[4] = {0.f, 0.f, 0.f, 0.f}, sc[4] = {0.f, 0.f, 0.f, 0.f};
+                  uint32_t a[4][4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  if (j0 + k * KR + kgrp == t) {  // the new row
-                    kn[k] = *reinterpret_cast<const uint4*>(mem + 256 + sub * 16);
-                    vn[k] = *reinterpret_cast<const uint4*>(mem + 384 + sub * 16);
+                  for (int k = 0; k < 4; ++k) ldsm4(a[k], kat + (((2 * k + k_piece) ^ kx) << 4));
+#pragma unroll
+                  for (int k = 0; k < 4; k += 2) {
+                    attn::mma_bf16(sa, a[k], qf[k / 2][0], qf[k / 2][1]);
+                    attn::mma_bf16(sc, a[k + 1], qf[k / 2][2], qf[k / 2][3]);
                   }
-                  const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kn[k]);
-                  float2 s2 = fmul2(q2[0], __bfloat1622float2(k2[0]));
 #pragma unroll
-                  for (int i = 1; i < 4; ++i) s2 = ffma2(q2[i], __bfloat1622float2(k2[i]), s2);
-                  sc[k] = s2.x + s2.y;
+                  for (int k = 0; k < 4; ++k) ldsm4t(a[k], vat + (((2 * k + v_piece) ^ vx) << 4));
+                  // scores of keys lane / 4 and lane / 4 + 8, the same in all four lanes
+                  float s0 = (sa[0] + sc[0]) + (sa[1] + sc[1]), s1 = (sa[2] + sc[2]) + (sa[3] + sc[3]);
+#pragma unroll
+                  for (int off = 1; off < 4; off <<= 1) {
+                    s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+                    s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+                  }
+                  const int key = tile * 16 + (lane >> 2);
+                  if (key > t) s0 = -INFINITY;
+                  if (key + 8 > t) s1 = -INFINITY;
+                  float mx = fmaxf(s0, s1);
+#pragma unroll
+                  for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                  const float m_new = fmaxf(m_run, mx), corr = ex2_approx(m_run - m_new);  // a tile has a key: m_new is finite
+                  const float p0 = ex2_approx(s0 - m_new), p1 = ex2_approx(s1 - m_new);    // 0 for a masked key
+                  m_run = m_new;
+                  l_run = fmaf(l_run, corr, p0 + p1);
+                  // part n = lane / 4 of the probabilities of keys 2 (lane % 4), + 1, + 8, + 9
+                  const int src = (lane & 3) * 8, n = lane >> 2;
+                  float pk[4] = {__shfl_sync(0xffffffffu, p0, src), __shfl_sync(0xffffffffu, p0, src + 4), __shfl_sync(0xffffffffu, p1, src),
+                                 __shfl_sync(0xffffffffu, p1, src + 4)};
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+                    float part[3];
+                    split3(pk[k], part);
+                    pk[k] = n == 0 ? part[0] : n == 1 ? part[1] : n == 2 ? part[2] : 0.f;
+                  }
+                  const uint32_t b0 = pack_bf16(pk[0], pk[1]), b1 = pack_bf16(pk[2], pk[3]);
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) o[k][i] *= corr;
+                    attn::mma_bf16(o[k], a[k], b0, b1);
+                  }
                 }
-                __syncwarp();
-#pragma unroll
-                for (int off = 1; off < 8; off <<= 1)
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], off);
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                  if (j0 + k * KR + kgrp > t) sc[k] = -INFINITY;
-                const float m_new = fmaxf(fmaxf(m_run, fmaxf(sc[0], sc[1])), fmaxf(sc[2], sc[3]));
-                const float m_ref = m_new > -INFINITY ? m_new : 0.f;  // a group that has seen no key yet keeps its zeros
-                const float corr = ex2_approx(m_run - m_ref);         // 0 when m_run = -inf
-                l_run *= corr;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) o2[i] = fmul2(o2[i], make_float2(corr, corr));
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const float pj = ex2_approx(sc[k] - m_ref);  // 0 for a masked key
-                  l_run += pj;
-                  const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&vn[k]);
-#pragma unroll
-                  for (int i = 0; i < 4; ++i) o2[i] = ffma2(make_float2(pj, pj), __bfloat1622float2(v2[i]), o2[i]);
+                if (unit < units) {
+                  __syncwarp();
+                  if (elect_one()) {
+                    mbar_arrive(bars + 8u * (2 * C::NSLOT + at));
+                    if (C::KVS == 2) mbar_arrive(bars + 8u * (2 * C::NSLOT + av));
+                  }
+                  __syncwarp();
                 }
-                m_run = m_new;
-                __syncwarp();
               }
-              float o[8];
+              if (set < sets) {
+                float* mg = s_merge + (p * NWARPS + set) * 72;
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                o[2 * i] = o2[i].x;
-                o[2 * i + 1] = o2[i].y;
-              }
-              // the warp's four groups, then (through shared memory) the sample's warps
-              const float mw = fmaxf(fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 8)),
-                                     fmaxf(__shfl_xor_sync(0xffffffffu, m_run, 16), __shfl_xor_sync(0xffffffffu, m_run, 24)));
-              const float f = mw > -INFINITY ? ex2_approx(m_run - mw) : 0.f;
-              l_run *= f;
-              l_run += __shfl_xor_sync(0xffffffffu, l_run, 8);
-              l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);
+                for (int off = 4; off < 32; off <<= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, off);
 #pragma unroll
-              for (int i = 0; i < 8; ++i) o[i] *= f;
-#pragma unroll
-              for (int off = 8; off < 32; off <<= 1)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) o[i] += __shfl_xor_sync(0xffffffffu, o[i], off);
-              float* mg = s_merge + (p * NWARPS + warp) * 72;
-              if (lane < 8) {
-                *reinterpret_cast<float4*>(mg + 8 * lane) = make_float4(o[0], o[1], o[2], o[3]);
-                *reinterpret_cast<float4*>(mg + 8 * lane + 4) = make_float4(o[4], o[5], o[6], o[7]);
-                if (lane == 0) { mg[64] = mw; mg[65] = l_run; }
+                for (int k = 0; k < 4; ++k) {  // the three columns of channels 16 k + lane / 4, + 8
+                  float x = o[k][0] + o[k][1], y = o[k][2] + o[k][3];
+                  x += __shfl_xor_sync(0xffffffffu, x, 1);
+                  y += __shfl_xor_sync(0xffffffffu, y, 1);
+                  if ((lane & 3) == 0) {
+                    mg[16 * k + (lane >> 2)] = x;
+                    mg[16 * k + 8 + (lane >> 2)] = y;
+                  }
+                }
+                if (lane == 0) { mg[64] = m_run; mg[65] = l_run; }
               }
               __syncwarp();
+            }
+            {
+              const int pos = slot + mine * units * C::KVS, wraps = pos / C::NSLOT;
+              slot = pos - wraps * C::NSLOT;
+              ring_parity ^= (uint32_t)(wraps & 1);
             }
             cbar();
 #pragma unroll 1
@@ -757,14 +823,14 @@ seq_block_kernel(const __grid_constant__ Job job) {
               const int peer = i & (CS - 1), c8 = (i / CS) & 7, p = i / (8 * CS);
               const float* mg = s_merge + p * NWARPS * 72;
               float mx = mg[64];
-#pragma unroll
-              for (int k = 1; k < NWARPS; ++k) mx = fmaxf(mx, mg[k * 72 + 64]);
+#pragma unroll 1
+              for (int k = 1; k < sets; ++k) mx = fmaxf(mx, mg[k * 72 + 64]);
               float den = 0.f, num[8];
 #pragma unroll
               for (int z = 0; z < 8; ++z) num[z] = 0.f;
-#pragma unroll 4
-              for (int k = 0; k < NWARPS; ++k) {
-                const float e = ex2_approx(mg[k * 72 + 64] - mx);  // 0 for a warp without keys
+#pragma unroll 1
+              for (int k = 0; k < sets; ++k) {
+                const float e = ex2_approx(mg[k * 72 + 64] - mx);
                 den = fmaf(e, mg[k * 72 + 65], den);
                 const float4 a = *reinterpret_cast<const float4*>(mg + k * 72 + 8 * c8);
                 const float4 b = *reinterpret_cast<const float4*>(mg + k * 72 + 8 * c8 + 4);
@@ -776,6 +842,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
                         pack_bf16(num[2] * inv, num[3] * inv), pack_bf16(num[4] * inv, num[5] * inv), pack_bf16(num[6] * inv, num[7] * inv),
                         peer_addr(bar(B_ALL0), peer));
             }
+            fence_proxy_async_global();  // the new cache rows: the next step's bulk copies, long after the barriers below, read them
           }
         } else {
           // ---------------------------------------------------------------- bias + GELU

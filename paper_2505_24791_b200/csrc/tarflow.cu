@@ -8,6 +8,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <climits>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -212,6 +213,7 @@ struct tf_model {
   int seqp_groups[2] = {0, 0};                 // groups of 16 / 32 samples that fit the GPU side by side (0: not eligible)
   uint32_t seqp_seq = 1;                       // sequence number of the next exchange
   unsigned long long *seqp_part = nullptr, *seqp_row = nullptr;
+  CUtensorMap seqp_cache[2];                   // keys, values
   bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
   int seq_attn_threads = 0;  // TARFLOW_SEQ_ATTN_THREADS=128|256: CTA size of the step attention (0 = by the number of CTAs)
   int seq_kbn_force = 0;     // TARFLOW_SEQ_KBN
@@ -1142,6 +1144,10 @@ static int seqp_setup(tf_model* m) {
     if (groups * sh.row > row) row = groups * sh.row;
   }
   if (m->seqp_groups[0] == 0 || m->seqp_groups[1] == 0) return TF_OK;
+  const int64_t cache_rows = (int64_t)m->cfg.n_layers * m->cfg.max_batch * m->cfg.n_heads * m->L;
+  if (cache_rows > INT_MAX - 32) return TF_OK;
+  TF_TRY(make_map_bf16(&m->seqp_cache[0], m->kcache, cache_rows, seqp::HD, 32));
+  TF_TRY(make_map_bf16(&m->seqp_cache[1], m->vcache, cache_rows, seqp::HD, 32));
   TF_TRY(dev_alloc(m, &m->seqp_part, part));
   TF_TRY(dev_alloc(m, &m->seqp_row, row));
   CU_OK(cudaMemset(m->seqp_part, 0, part * sizeof(*m->seqp_part)));
@@ -1190,13 +1196,13 @@ static int run_sequential_persistent(tf_model* m, int g, int B, const int* label
   job.b_out = bw.b_out; job.w_out = reinterpret_cast<const bf16*>(bw.w_out.w);
   job.v = v; job.u = u; job.labels = labels;
   job.kc = reinterpret_cast<bf16*>(m->kcache); job.vc = reinterpret_cast<bf16*>(m->vcache);
-  job.layer_stride = (size_t)m->cfg.max_batch * L * m->d;
+  job.kmap = m->seqp_cache[0]; job.vmap = m->seqp_cache[1];
+  job.layer_rows = m->cfg.max_batch * m->cfg.n_heads * L;
   job.xpart = m->seqp_part; job.xrow = m->seqp_row;
   job.n_layers = nl; job.B = B; job.L = L; job.Dt = D; job.reversed = g & 1;
   job.seq0 = m->seqp_seq;
   m->seqp_seq += (uint32_t)((2 * nl + 1) * n_steps + 1);
   job.prefetch_w = weights > kL2Half;
-  job.prefetch_kv = (size_t)nl * B * L * m->d * 2 * sizeof(bf16) > kL2Half;
   job.scale_log2e = 1.4426950408889634f / sqrtf((float)m->hd);
   job.err = m->err;
   m->cur_rows = (int64_t)B * n_steps;
