@@ -106,7 +106,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
   static_assert(NUM_BARS * 8 <= 192, "barrier area");
   auto bar = [&](int i) { return bar_base + 8u * i; };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::Q_ALL + KV_RING + C::P_ALL + 192);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // uniform, and visibly so
   const int n_qt = (L + BQ - 1) / BQ;
   const int qt = n_qt - 1 - (int)blockIdx.x;  // longest tiles first
   const int head = blockIdx.y, slot = blockIdx.z;
@@ -216,7 +216,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
     // ------------------------------------------------------------------ softmax + output (warps 2..5)
     const int quad = warp & 3;
     const int r = quad * 32 + lane;            // row of this thread inside the query tile
-    const int qpos = q0 + r;                   // position in the sequence
     const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
     const uint32_t t_o = t_row + BKV;          // this row's slice of the output accumulator
     uint8_t* sPg = smem + C::Q_ALL + KV_RING;
@@ -228,8 +227,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
     for (int j = 0; j < n_kv && ok; ++j) {
       if (!mbar_wait(bar(B_SFULL), (uint32_t)(j & 1), err, TFERR_WAIT_TMEM_FULL)) { ok = false; break; }
       tcgen05_fence_after();
-      const int kv0 = j * BKV;
-      const bool diag = kv0 + BKV - 1 > q0;  // some key of this tile lies after some query of the tile
+      // How many 32-key halves of the tile this warp's 32 rows see; of the last one a diagonal half is seen in part.  Two of
+      // every query tile's key tiles lie on the diagonal (all of them at 128 tokens, two of three on average at 256), and
+      // three of their eight (warp, tile) halves hold no visible key: those cost a row of zeros instead of exponentials.
+      const int kv0 = j * BKV, ahead = q0 + quad * 32 - kv0;  // first row - first key, a multiple of 32
+      const int halves = ahead < 0 ? 0 : ahead < 32 ? 1 : 2;
       // the whole score row in one round of tensor-memory loads
       float s[BKV];
       tmem_ld_32x32b_x32_issue(t_row, *reinterpret_cast<float(*)[32]>(&s[0]));
@@ -238,24 +240,38 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
       tcgen05_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(B_SFREE));  // the tensor core may overwrite S with the next tile's scores
-      if (diag) {
-#pragma unroll
-        for (int i = 0; i < BKV; ++i)
-          if (kv0 + i > qpos) s[i] = -INFINITY;
-      }
-      float mx0 = s[0], mx1 = s[1];
-#pragma unroll
-      for (int i = 2; i < BKV; i += 4) {
-        mx0 = fmax3(mx0, s[i], s[i + 1]);
-        if (i + 3 < BKV) mx1 = fmax3(mx1, s[i + 2], s[i + 3]);
-      }
-      const float mx = fmaxf(mx0, mx1);  // finite from the first tile on: key 0 is visible to every row
       float corr = 1.f;
-      const bool bump = (mx - m_run) * scale_log2e > kLazy;  // also true on the first tile (m_run = -inf)
-      if (bump) {
-        corr = ex2_approx((m_run - mx) * scale_log2e);
-        m_run = mx;
-        l_run *= corr;
+      bool bump = false;
+      if (halves > 0) {
+        if (ahead == 0) {
+#pragma unroll
+          for (int i = 1; i < 32; ++i)
+            if (i > lane) s[i] = -INFINITY;
+        } else if (ahead == 32) {
+#pragma unroll
+          for (int i = 1; i < 32; ++i)
+            if (i > lane) s[32 + i] = -INFINITY;
+        }
+        float mx0 = s[0], mx1 = s[1];
+#pragma unroll
+        for (int i = 2; i < 32; i += 4) {
+          mx0 = fmax3(mx0, s[i], s[i + 1]);
+          if (i + 3 < 32) mx1 = fmax3(mx1, s[i + 2], s[i + 3]);
+        }
+        if (halves == 2) {
+#pragma unroll
+          for (int i = 32; i < 64; i += 4) {
+            mx0 = fmax3(mx0, s[i], s[i + 1]);
+            mx1 = fmax3(mx1, s[i + 2], s[i + 3]);
+          }
+        }
+        const float mx = fmaxf(mx0, mx1);                   // finite: the first key of a visible half is visible to every row
+        bump = (mx - m_run) * scale_log2e > kLazy;          // also true on the first tile (m_run = -inf)
+        if (bump) {
+          corr = ex2_approx((m_run - mx) * scale_log2e);
+          m_run = mx;
+          l_run *= corr;
+        }
       }
       // P was the A operand of the previous tile's product, which also has to be in the accumulator before a rescale
       if (j > 0) {
@@ -268,24 +284,35 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
       const float2 sc2 = make_float2(scale_log2e, scale_log2e), mb2 = make_float2(mb, mb);
       float2 lsum = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        uint32_t pk[4], pl[4];
+      for (int half = 0; half < 2; ++half) {
+        if (half < halves) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float2 e = ffma2(make_float2(s[8 * q + 2 * i], s[8 * q + 2 * i + 1]), sc2, mb2);
-          e.x = ex2_approx(e.x);  // exp2(-inf) = 0 for masked keys
-          e.y = ex2_approx(e.y);
-          lsum = fadd2(lsum, e);
-          const __nv_bfloat162 pb = __floats2bfloat162_rn(e.x, e.y);
-          pk[i] = *reinterpret_cast<const uint32_t*>(&pb);
-          if constexpr (SPLIT) {
-            const float2 hi = __bfloat1622float2(pb);
-            const __nv_bfloat162 pl2 = __floats2bfloat162_rn(e.x - hi.x, e.y - hi.y);
-            pl[i] = *reinterpret_cast<const uint32_t*>(&pl2);
+          for (int q = 4 * half; q < 4 * half + 4; ++q) {
+            uint32_t pk[4], pl[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              float2 e = ffma2(make_float2(s[8 * q + 2 * i], s[8 * q + 2 * i + 1]), sc2, mb2);
+              e.x = ex2_approx(e.x);  // exp2(-inf) = 0 for masked keys
+              e.y = ex2_approx(e.y);
+              lsum = fadd2(lsum, e);
+              const __nv_bfloat162 pb = __floats2bfloat162_rn(e.x, e.y);
+              pk[i] = *reinterpret_cast<const uint32_t*>(&pb);
+              if constexpr (SPLIT) {
+                const float2 hi = __bfloat1622float2(pb);
+                const __nv_bfloat162 pl2 = __floats2bfloat162_rn(e.x - hi.x, e.y - hi.y);
+                pl[i] = *reinterpret_cast<const uint32_t*>(&pl2);
+              }
+            }
+            *reinterpret_cast<uint4*>(sPg + swz128(r, q)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            if constexpr (SPLIT) *reinterpret_cast<uint4*>(sPg + P_BYTES + swz128(r, q)) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 4 * half; q < 4 * half + 4; ++q) {
+            *reinterpret_cast<uint4*>(sPg + swz128(r, q)) = make_uint4(0u, 0u, 0u, 0u);
+            if constexpr (SPLIT) *reinterpret_cast<uint4*>(sPg + P_BYTES + swz128(r, q)) = make_uint4(0u, 0u, 0u, 0u);
           }
         }
-        *reinterpret_cast<uint4*>(sPg + swz128(r, q)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        if constexpr (SPLIT) *reinterpret_cast<uint4*>(sPg + P_BYTES + swz128(r, q)) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
       }
       l_run += lsum.x + lsum.y;
       fence_proxy_async_smem();
@@ -332,7 +359,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
       if (lane == 0 && q0 + quad * 32 < L) {
         tma_store_3d(map_out, head * HD, q0 + quad * 32, slot, smem_u32(box));
         tma_store_commit();
-        tma_store_wait_all();
+        tma_store_wait_read();
       }
       if constexpr (SPLIT) {  // the low half of the output pair through the same box
         __syncwarp();
@@ -353,7 +380,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
         if (lane == 0 && q0 + quad * 32 < L) {
           tma_store_3d(map_out_lo, head * HD, q0 + quad * 32, slot, smem_u32(box));
           tma_store_commit();
-          tma_store_wait_all();
+          tma_store_wait_read();
         }
       }
     }
