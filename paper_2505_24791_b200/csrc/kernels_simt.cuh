@@ -2,6 +2,7 @@
 // attention (fp32 engine), single-query attention over the KV cache, update / forward epilogues
 // as stand-alone kernels, and Jacobi sweep control.
 #pragma once
+#include "attention_mma.cuh"
 #include "common.cuh"
 #include "epilogue.cuh"
 
@@ -102,122 +103,181 @@ embed_rows_kernel(const float* __restrict__ u, const int* __restrict__ idx, cons
 }
 
 // ------------------------------------------------------------------------------------------------
-// Embedding of R rows per CTA fused with the first LayerNorm of the block:
+// Embedding of rows fused with the first LayerNorm of the block:
 //   h[row, :]  = u[token] W_in^T + b_in + pos[l] (+ cls[y])          (fp32 residual stream)
 //   xn[row, :] = LayerNorm(h[row, :]) * gamma + beta                  (T; plus the "lo" half of a two-term pair)
-// Thread k owns columns 4k..4k+3 of all R rows (blockDim.x = d / 4 rounded up to whole warps, d % 4 == 0): per
-// token value one 16-byte weight load feeds 4 R FMAs, the R tokens sit in shared memory transposed ([D][R]) so
-// four rows come with one broadcast 16-byte read.  The row statistics (two-pass, eps 1e-5) are reduced over the
-// CTA's warps through shared memory.  h is bit-identical to embed_rows_kernel's.
+// A CTA owns R rows, its thread k columns 4k..4k+3 of all of them (blockDim.x = d / 4 rounded up to whole warps, d % 4 == 0).
+// fp32 products on the CUDA cores and the rows' way to memory bound it, one after the other in a CTA: two CTAs per SM overlap
+// them (50 399 rows of width 1024, 48 values per token: 367 -> 311 us; CTAs of 32 rows with one copy of the weights: 320).
+//   * the weights come through shared memory in two buffers of `cc` token values by cp.async, the first ones requested before the
+//     previous kernel has ended (256 rows: 20.9 -> 17.6 us);
+//   * the R tokens sit in shared memory transposed ([D][R]): a 16-byte broadcast read is two row pairs, each a packed FMA;
+//   * the row statistics (two-pass, eps 1e-5) are reduced for all R rows at once: a lane keeps half of the rows at every
+//     exchange (R + 1 shuffles instead of 5 R), and one read per row and warp collects them over the CTA's warps.
+// h is bit-identical to embed_rows_kernel's.
 // ------------------------------------------------------------------------------------------------
+constexpr int EMBED_THREADS = 256;                                          // of a CTA, at most
+constexpr int EMBED_WEIGHT_BYTES = 64 << 10, EMBED_TOKEN_BYTES = 40 << 10;  // of its shared memory, at most
+
+// Sums over the warp of R values per lane; lane l returns the total of value l / (32 / R).  The tree of every sum is warp_sum's.
+template <int R>
+__device__ __forceinline__ float warp_sum_rows(float (&v)[R], int lane) {
+#pragma unroll
+  for (int n = R / 2, o = 16; n > 0; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (int o = 16 / R; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
 template <class T, int R>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(EMBED_THREADS)
 embed_ln_rows_kernel(const float* __restrict__ u, const int* __restrict__ idx, const int* __restrict__ labels,
                      const float* __restrict__ w_in_t, const float* __restrict__ b_in, const float* __restrict__ pos,
                      const float* __restrict__ cls, float* __restrict__ h, const float* __restrict__ gamma,
                      const float* __restrict__ beta, T* __restrict__ xn, T* __restrict__ xn_lo, int L, int D, int d,
-                     int reversed, int n_rows) {
-  extern __shared__ __align__(16) float s_ut[];  // [D][R]
-  __shared__ float s_red[2][8][R];
-  __shared__ int s_l[R], s_b[R];
+                     int reversed, int n_rows, int cc) {
+  static_assert(R == 4 || R == 16, "rows per group");
+  constexpr int SPAN = 32 / R;                    // lanes that end up with the same row
+  extern __shared__ __align__(16) float s_emb[];  // two weight buffers [cc][d], then the tokens [D][R]
+  __shared__ float s_red[2][EMBED_THREADS / 32][R];
+  __shared__ int s_l[R], s_b[R], s_y[R];
+  const int k = threadIdx.x, warp = k >> 5, lane = k & 31, nwarps = blockDim.x >> 5, dv = d >> 2, row0 = blockIdx.x * R;
+  const bool act = k < dv;
+  float* s_ut = s_emb + 2 * cc * d;
+  auto stage = [&](int c0, int buf) {
+    const int n = (D - c0 < cc ? D - c0 : cc) * dv;
+    for (int i = k; i < n; i += blockDim.x) attn::cp_async16(s_emb + buf * cc * d + 4 * i, w_in_t + (size_t)c0 * d + 4 * i, true);
+  };
+  stage(0, 0);  // weights do not depend on the previous kernel
+  attn::cp_async_commit();
+  if (cc < D) stage(cc, 1);
+  attn::cp_async_commit();
   pdl_launch_dependents();
   pdl_wait();
-  const int row0 = blockIdx.x * R;
-  if (threadIdx.x < R) {
-    const int row = row0 + threadIdx.x;
+  if (k < R) {
+    const int row = row0 + k;
     int l = 0, b = -1;
     if (row < n_rows) {
       const int s = row / L;
       l = row - s * L;
       b = idx ? idx[s] : s;
     }
-    s_l[threadIdx.x] = l;
-    s_b[threadIdx.x] = b;
+    s_l[k] = l;
+    s_b[k] = b;
+    s_y[k] = cls != nullptr && b >= 0 ? labels[b] : 0;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < R * D; e += blockDim.x) {
+  for (int e = k; e < R * D; e += blockDim.x) {
     const int r = e / D, c = e - r * D, b = s_b[r];
     s_ut[c * R + r] = b >= 0 ? u[((size_t)b * L + tok_index(s_l[r], L, reversed)) * D + c] : 0.f;
   }
-  __syncthreads();
-  const int k = threadIdx.x, dv = d >> 2;
-  const bool act = k < dv;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = (blockDim.x + 31) >> 5;
-  float4 acc[R];
+  float2 acc[R / 2][4];  // rows 2p, 2p + 1; four columns
 #pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (act) {
-    const float4* w4 = reinterpret_cast<const float4*>(w_in_t) + k;
-#pragma unroll (R <= 4 ? 16 : 4)
-    for (int c = 0; c < D; ++c) {
-      const float4 w = __ldg(w4 + (size_t)c * dv);
+  for (int p = 0; p < R / 2; ++p)
 #pragma unroll
-      for (int r4 = 0; r4 < R; r4 += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(s_ut + c * R + r4);
-        const float xs[4] = {x.x, x.y, x.z, x.w};
+    for (int q = 0; q < 4; ++q) acc[p][q] = make_float2(0.f, 0.f);
+  for (int c0 = 0, buf = 0; c0 < D; c0 += cc, buf ^= 1) {
+    attn::cp_async_wait<1>();
+    __syncthreads();
+    const int n = D - c0 < cc ? D - c0 : cc;
+    if (act) {
+      const float* wp = s_emb + buf * cc * d + 4 * k;
+      const float* xp = s_ut + c0 * R;
+#pragma unroll 2
+      for (int c = 0; c < n; ++c) {
+        const float4 w = *reinterpret_cast<const float4*>(wp + c * d);
+        const float2 w2[4] = {make_float2(w.x, w.x), make_float2(w.y, w.y), make_float2(w.z, w.z), make_float2(w.w, w.w)};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          acc[r4 + q].x = fmaf(xs[q], w.x, acc[r4 + q].x);
-          acc[r4 + q].y = fmaf(xs[q], w.y, acc[r4 + q].y);
-          acc[r4 + q].z = fmaf(xs[q], w.z, acc[r4 + q].z);
-          acc[r4 + q].w = fmaf(xs[q], w.w, acc[r4 + q].w);
+        for (int p = 0; p < R / 2; p += 2) {
+          const float4 x = *reinterpret_cast<const float4*>(xp + c * R + 2 * p);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            acc[p][q] = ffma2(make_float2(x.x, x.y), w2[q], acc[p][q]);
+            acc[p + 1][q] = ffma2(make_float2(x.z, x.w), w2[q], acc[p + 1][q]);
+          }
         }
       }
     }
+    __syncthreads();
+    if (c0 + 2 * cc < D) stage(c0 + 2 * cc, buf);
+    attn::cp_async_commit();
   }
-  // residual stream row, first statistic
+  // residual stream rows, first statistic
   float4 bj = make_float4(0.f, 0.f, 0.f, 0.f);
   if (act) bj = reinterpret_cast<const float4*>(b_in)[k];
   float part[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int row = row0 + r;
+    float2(&a)[4] = acc[r / 2];
     part[r] = 0.f;
     if (act && row < n_rows) {
       const float4 p = __ldg(reinterpret_cast<const float4*>(pos) + (size_t)s_l[r] * dv + k);
-      float4 a = acc[r];
-      a.x += bj.x + p.x; a.y += bj.y + p.y; a.z += bj.z + p.z; a.w += bj.w + p.w;
+      float4 x = (r & 1) ? make_float4(a[0].y, a[1].y, a[2].y, a[3].y) : make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
+      x.x += bj.x + p.x; x.y += bj.y + p.y; x.z += bj.z + p.z; x.w += bj.w + p.w;
       if (cls != nullptr) {
-        const float4 cl = __ldg(reinterpret_cast<const float4*>(cls) + (size_t)labels[s_b[r]] * dv + k);
-        a.x += cl.x; a.y += cl.y; a.z += cl.z; a.w += cl.w;
+        const float4 cl = __ldg(reinterpret_cast<const float4*>(cls) + (size_t)s_y[r] * dv + k);
+        x.x += cl.x; x.y += cl.y; x.z += cl.z; x.w += cl.w;
       }
-      acc[r] = a;
-      reinterpret_cast<float4*>(h)[(size_t)row * dv + k] = a;
-      part[r] = (a.x + a.y) + (a.z + a.w);
+      reinterpret_cast<float4*>(h)[(size_t)row * dv + k] = x;
+      part[r] = (x.x + x.y) + (x.z + x.w);
+      if (r & 1) {
+        a[0].y = x.x; a[1].y = x.y; a[2].y = x.z; a[3].y = x.w;
+      } else {
+        a[0].x = x.x; a[1].x = x.y; a[2].x = x.z; a[3].x = x.w;
+      }
     }
   }
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const float v = warp_sum(part[r]);
-    if (lane == 0) s_red[0][warp][r] = v;
-  }
+  const int my_r = lane / SPAN;  // the row whose sums this lane holds after an exchange
+  float tot = warp_sum_rows<R>(part, lane);
+  if (lane % SPAN == 0) s_red[0][warp][my_r] = tot;
   __syncthreads();
   const float inv_d = 1.f / (float)d;
+  tot = 0.f;
+  for (int w = 0; w < nwarps; ++w) tot += s_red[0][w][my_r];
+  const float my_mean = tot * inv_d;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    float tot = 0.f;
-    for (int w = 0; w < nwarps; ++w) tot += s_red[0][w][r];
-    const float mean = tot * inv_d;
-    float sq = 0.f;
+    const float mean = __shfl_sync(0xffffffffu, my_mean, r * SPAN);
+    float2(&a)[4] = acc[r / 2];
+    part[r] = 0.f;
     if (act) {
-      acc[r].x -= mean; acc[r].y -= mean; acc[r].z -= mean; acc[r].w -= mean;
-      sq = (acc[r].x * acc[r].x + acc[r].y * acc[r].y) + (acc[r].z * acc[r].z + acc[r].w * acc[r].w);
+      if (r & 1) {
+        a[0].y -= mean; a[1].y -= mean; a[2].y -= mean; a[3].y -= mean;
+        part[r] = (a[0].y * a[0].y + a[1].y * a[1].y) + (a[2].y * a[2].y + a[3].y * a[3].y);
+      } else {
+        a[0].x -= mean; a[1].x -= mean; a[2].x -= mean; a[3].x -= mean;
+        part[r] = (a[0].x * a[0].x + a[1].x * a[1].x) + (a[2].x * a[2].x + a[3].x * a[3].x);
+      }
     }
-    part[r] = warp_sum(sq);
-    if (lane == 0) s_red[1][warp][r] = part[r];
   }
+  tot = warp_sum_rows<R>(part, lane);
+  if (lane % SPAN == 0) s_red[1][warp][my_r] = tot;
   __syncthreads();
-  if (!act) return;
-  const float4 g = reinterpret_cast<const float4*>(gamma)[k], bb = reinterpret_cast<const float4*>(beta)[k];
+  tot = 0.f;
+  for (int w = 0; w < nwarps; ++w) tot += s_red[1][w][my_r];
+  const float my_rstd = rsqrtf(tot * inv_d + 1e-5f);
+  float4 g = make_float4(0.f, 0.f, 0.f, 0.f), bb = g;
+  if (act) {
+    g = reinterpret_cast<const float4*>(gamma)[k];
+    bb = reinterpret_cast<const float4*>(beta)[k];
+  }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
+    const float rstd = __shfl_sync(0xffffffffu, my_rstd, r * SPAN);
     const int row = row0 + r;
-    if (row >= n_rows) continue;
-    float tot = 0.f;
-    for (int w = 0; w < nwarps; ++w) tot += s_red[1][w][r];
-    const float rstd = rsqrtf(tot * inv_d + 1e-5f);
-    const float o0 = acc[r].x * rstd * g.x + bb.x, o1 = acc[r].y * rstd * g.y + bb.y;
-    const float o2 = acc[r].z * rstd * g.z + bb.z, o3 = acc[r].w * rstd * g.w + bb.w;
+    if (!act || row >= n_rows) continue;
+    const float2(&a)[4] = acc[r / 2];
+    const float4 x = (r & 1) ? make_float4(a[0].y, a[1].y, a[2].y, a[3].y) : make_float4(a[0].x, a[1].x, a[2].x, a[3].x);
+    const float o0 = x.x * rstd * g.x + bb.x, o1 = x.y * rstd * g.y + bb.y;
+    const float o2 = x.z * rstd * g.z + bb.z, o3 = x.w * rstd * g.w + bb.w;
     if constexpr (sizeof(T) == 4) {
       reinterpret_cast<float4*>(xn)[(size_t)row * dv + k] = make_float4(o0, o1, o2, o3);
     } else {

@@ -558,15 +558,20 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   int ethreads = d < 256 ? d : 256;
   m->cur_rows = M;
   // embedding fused with the first LayerNorm when a thread can own four columns of a row
-  const bool fused_embed = d % 4 == 0 && d <= 1024 && (size_t)16 * D * sizeof(float) <= 40 * 1024;
+  const bool fused_embed = d % 4 == 0 && d <= 1024 && (size_t)16 * D * sizeof(float) <= EMBED_TOKEN_BYTES;
   if (fused_embed) {
     const LayerW& l0 = bw.layers[0];
-    if (M <= m->small_m_rows)  // few rows: four per CTA instead of sixteen, for four times the CTAs
-      LAUNCH_PDL(m, KC_EMBED, (embed_ln_rows_kernel<T, 4>), (M + 3) / 4, ((d / 4 + 31) / 32) * 32, 4 * D * sizeof(float), u_src,
-                 idx, labels, bw.w_in_t, bw.b_in, bw.pos, bw.cls, m->h, l0.ln1_g, l0.ln1_b, xn, xn_lo, L, D, d, rev, M);
+    const bool few = M <= m->small_m_rows;  // few rows: four per CTA instead of sixteen, for four times the CTAs
+    const int R = few ? 4 : 16, threads = ((d / 4 + 31) / 32) * 32;
+    int cc = EMBED_WEIGHT_BYTES / (2 * d * (int)sizeof(float));  // token values per weight buffer
+    cc = cc > D ? D : cc;
+    const size_t smem = (size_t)(2 * cc * d + R * D) * sizeof(float);
+    if (few)
+      LAUNCH_PDL(m, KC_EMBED, (embed_ln_rows_kernel<T, 4>), (M + 3) / 4, threads, smem, u_src, idx, labels, bw.w_in_t, bw.b_in, bw.pos,
+                 bw.cls, m->h, l0.ln1_g, l0.ln1_b, xn, xn_lo, L, D, d, rev, M, cc);
     else
-      LAUNCH_PDL(m, KC_EMBED, (embed_ln_rows_kernel<T, 16>), (M + 15) / 16, ((d / 4 + 31) / 32) * 32, 16 * D * sizeof(float), u_src,
-                 idx, labels, bw.w_in_t, bw.b_in, bw.pos, bw.cls, m->h, l0.ln1_g, l0.ln1_b, xn, xn_lo, L, D, d, rev, M);
+      LAUNCH_PDL(m, KC_EMBED, (embed_ln_rows_kernel<T, 16>), (M + 15) / 16, threads, smem, u_src, idx, labels, bw.w_in_t, bw.b_in, bw.pos,
+                 bw.cls, m->h, l0.ln1_g, l0.ln1_b, xn, xn_lo, L, D, d, rev, M, cc);
   } else {
     LAUNCH_PDL(m, KC_EMBED, embed_rows_kernel<16>, (M + 15) / 16, ethreads, 16 * D * sizeof(float), u_src, idx, labels,
                bw.w_in_t, bw.b_in, bw.pos, bw.cls, m->h, L, D, d, rev, M);
@@ -1952,6 +1957,10 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
   CU_OK(cudaMemset(m->ctrl, 0, CTRL_WORDS * sizeof(int)));
   CU_OK(cudaMemset(m->err, 0, sizeof(int)));
   CU_OK(cudaMemset(m->iters_sample, 0, (size_t)c.n_blocks * B * sizeof(int)));
+  for (const auto kern : {embed_ln_rows_kernel<bf16, 4>, embed_ln_rows_kernel<bf16, 16>})
+    CU_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, EMBED_WEIGHT_BYTES + EMBED_TOKEN_BYTES));
+  for (const auto kern : {embed_ln_rows_kernel<float, 4>, embed_ln_rows_kernel<float, 16>})
+    CU_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, EMBED_WEIGHT_BYTES + EMBED_TOKEN_BYTES));
   CU_OK(cudaMallocHost(&m->ctrl_host, HOST_WORDS * sizeof(int)));
   memset(m->ctrl_host, 0, HOST_WORDS * sizeof(int));
   m->block_ev.assign(c.n_blocks + 1, nullptr);
