@@ -1,0 +1,49 @@
+"""The sequentially decoded block as one launch, at the edges of its split of the work.
+
+bf16 engine: the cooperative kernel runs groups of at most 16 or 32 samples side by side and cuts the cache into 16-key tiles
+and units of 64 or 128 keys; 132 tokens cross both, the batches leave groups and ranks short or without samples.  fp32 engine:
+1, 2 or 4 samples per cluster.
+"""
+import numpy as np
+import pytest
+
+from oracle import tarflow_oracle as O
+from paper_2505_24791_b200 import synth
+from tests.gpu_util import Model, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+REL_L2, MAX_ABS = 2e-2, 5e-2  # bf16 engine against the fp64 oracle: the tolerances of every other bf16 test
+PATHS = 5e-3                  # two orders of summation of the same bf16 products: the bound used for the other step kernels
+FP32_MAX = 1e-4               # fp32 engine against the fp64 oracle
+
+
+@pytest.mark.parametrize("width,batch,classes", [(128, 1, 0), (128, 40, 0), (256, 15, 10), (256, 130, 0), (512, 3, 0), (512, 65, 10),
+                                                 (1024, 1, 0), (1024, 18, 10), (1024, 33, 0)])
+def test_bf16_block_in_one_launch(monkeypatch, width, batch, classes):
+    cfg = synth.config("cfg2", H=24, W=22, n_blocks=1, n_layers=2, width=width, n_heads=width // 64, n_classes=classes)
+    z = synth.make_latents(cfg, 7, B=batch)
+    lab = synth.make_labels(cfg, B=batch) if classes else None
+    out = {}
+    for path in ("0", "1"):
+        monkeypatch.setenv("TARFLOW_SEQ_PERSIST", path)
+        with Model(cfg, max_batch=batch) as m:
+            out[path] = m.inverse_sequential(z, lab)
+            pick = sorted({0, batch // 2, batch - 1})
+            if path == "1":  # a sample's arithmetic depends neither on the batch nor on its place in it
+                for p in pick:
+                    alone = m.inverse_sequential(z[p:p + 1], None if lab is None else lab[p:p + 1])
+                    assert np.array_equal(alone[0], out[path][p])
+            xo = O.model_inverse_sequential(m.blocks, z[pick], None if lab is None else lab[pick], cfg)
+        x = out[path][pick]
+        assert np.isfinite(out[path]).all() and rel_l2(x, xo) <= REL_L2 and np.abs(x - xo).max() <= MAX_ABS
+    assert rel_l2(out["1"], out["0"]) <= PATHS
+
+
+@pytest.mark.parametrize("batch", [1, 17, 37])
+def test_fp32_block_in_one_launch(batch):
+    cfg = synth.config("cfg1", H=14, W=10, n_blocks=1)
+    z = synth.make_latents(cfg, 8, B=batch)
+    with Model(cfg, max_batch=batch) as m:
+        x = m.inverse_sequential(z, None)
+        assert np.abs(x - O.model_inverse_sequential(m.blocks, z, None, cfg)).max() <= FP32_MAX
