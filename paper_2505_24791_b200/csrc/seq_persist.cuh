@@ -33,7 +33,6 @@
 #pragma once
 #include "common.cuh"
 #include "gemm_tc.cuh"
-#include "attention_mma.cuh"
 
 namespace seqp {
 
@@ -87,9 +86,8 @@ struct Cfg {
   static constexpr int RECV = STG + RT * 1024;
   static constexpr int MERGE = RECV;                  // [sample][warp]: output, maximum, sum; q, k, v have left the place by then
   static constexpr int QKV = RECV + (RT * 1024 > BL * NWARPS * 288 ? RT * 1024 : BL * NWARPS * 288);
-  static constexpr int QROW = 640;                    // per sample, bf16 [64] each: q in three parts, the new k, the new v
-  static constexpr int ZERO = QKV + BL * QROW;        // 128 zero bytes
-  static constexpr int SUM = ZERO + 128;
+  static constexpr int QROW = 512;                    // per sample: q fp32 [64], the new k, the new v bf16 [64]
+  static constexpr int SUM = QKV + BL * QROW;
   static constexpr int XN = SUM + (SGC - 1) * RPC * QN * 16;
   static constexpr int TOK = XN + RPC * CW * 4;
   static constexpr int STAT = TOK + RPC * MAXDT * 4;
@@ -308,20 +306,6 @@ __device__ __forceinline__ void feed(const Job& job, uint32_t ring, uint32_t bar
     }
 }
 
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t at) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(at) : "memory");
-}
-__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t at) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(at) : "memory");
-}
-// x as the sum of three bf16: 24 bits, the whole fp32 mantissa
-__device__ __forceinline__ void split3(float x, float (&part)[3]) {
-  part[0] = __bfloat162float(__float2bfloat16_rn(x));
-  const float rest = x - part[0];
-  part[1] = __bfloat162float(__float2bfloat16_rn(rest));
-  part[2] = rest - part[1];
-}
-
 // grid: groups * HEADS clusters of CS CTAs (cooperative), 256 threads and a warp that moves the weights
 template <int D, int RT>
 __global__ void __launch_bounds__(NTHREADS + 32, 1)
@@ -347,7 +331,6 @@ seq_block_kernel(const __grid_constant__ Job job) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *s_bad = 0;
   }
-  if (tid < 8) *reinterpret_cast<uint4*>(smem + C::ZERO + 16 * tid) = make_uint4(0u, 0u, 0u, 0u);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM)
                  : "memory");
@@ -368,10 +351,9 @@ seq_block_kernel(const __grid_constant__ Job job) {
     if (lane == 0) feed<D, RT>(job, sb + C::RING, bars, r, c, job.prefetch_w && group == 0, mine, rows_of(0));
   } else {
     constexpr uint32_t idesc = make_idesc(RT);
-    // attention: a sample's keys are cut into tiles of 16, dealt out to eight sets whatever the batch; a set belongs to a warp.
-    // The operand rows of this lane: keys kr of a tile, values of keys vr (transposed on the way), parts of q
-    const int kr = lane & 15, vr = (lane & 7) + (lane >> 4) * 8;
-    const uint32_t k_piece = lane >> 4, v_piece = (lane >> 3) & 1, q_piece = lane >> 3;
+    // attention: a sample's keys are cut into tiles of 16, dealt out to eight sets whatever the batch; a set belongs to a warp,
+    // eight lanes share a key (eight channels each), the warp's four groups of lanes take every fourth key
+    const int sub = lane & 7, kgrp = lane >> 3;
     // hidden units this thread finishes: eight of them, samples fb, fb + FB, ...
     constexpr int FB = NTHREADS / (UPC / 8);
     const int u8 = (tid % (UPC / 8)) * 8, fb = tid / (UPC / 8);
@@ -380,6 +362,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
     const int rpc = (nb + HEADS - 1) / HEADS, own0 = c * rpc, own = nb - own0 < rpc ? (nb - own0 > 0 ? nb - own0 : 0) : rpc;
     const int q = tid % QN, lrow = (tid / QN) % C::RPC, g = tid / (QN * C::RPC), col = r * CW + 4 * q;
     const bool my_row = lrow < own, holder = warp < C::GW;
+    const float* cls_row = job.cls != nullptr && my_row ? job.cls + (size_t)job.labels[row0 + own0 + lrow] * D : nullptr;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 h = zero4;
     float4* s_sum = reinterpret_cast<float4*>(smem + C::SUM);
@@ -460,8 +443,8 @@ seq_block_kernel(const __grid_constant__ Job job) {
               if (holder) {
                 const float4 p = ld4(job.pos + (size_t)t * D);
                 add.x += p.x; add.y += p.y; add.z += p.z; add.w += p.w;
-                if (job.cls != nullptr) {
-                  const float4 y = ld4(job.cls + (size_t)job.labels[row0 + own0 + lrow] * D);
+                if (cls_row != nullptr) {
+                  const float4 y = ld4(cls_row);
                   add.x += y.x; add.y += y.y; add.z += y.z; add.w += y.w;
                 }
                 h = zero4;
@@ -690,16 +673,11 @@ seq_block_kernel(const __grid_constant__ Job job) {
               }
               uint8_t* mem = smem + C::QKV + p * C::QROW;
               if (c4 < 16) {  // scores in base-2 units: softmax via exp2
-                float p0[3], p1[3], p2[3], p3[3];
-                split3(x.x * job.scale_log2e, p0);
-                split3(x.y * job.scale_log2e, p1);
-                split3(x.z * job.scale_log2e, p2);
-                split3(x.w * job.scale_log2e, p3);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) *reinterpret_cast<uint2*>(mem + k * 128 + 8 * c4) = make_uint2(pack_bf16(p0[k], p1[k]), pack_bf16(p2[k], p3[k]));
+                *reinterpret_cast<float4*>(mem + 16 * c4) =
+                    make_float4(x.x * job.scale_log2e, x.y * job.scale_log2e, x.z * job.scale_log2e, x.w * job.scale_log2e);
               } else {
                 const uint2 w2 = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-                *reinterpret_cast<uint2*>(mem + 384 + (c4 - 16) * 8) = w2;
+                *reinterpret_cast<uint2*>(mem + 256 + (c4 - 16) * 8) = w2;
                 const size_t row = (size_t)(half >> 1) * job.layer_rows + rows_of(p) + t;
                 *reinterpret_cast<uint2*>((c4 < 32 ? job.kc : job.vc) + row * HD + (c4 & 15) * 4) = w2;
               }
@@ -708,19 +686,17 @@ seq_block_kernel(const __grid_constant__ Job job) {
             const int units = (t + C::KPU - 1) / C::KPU, tiles = t / 16 + 1, sets = tiles < NWARPS ? tiles : NWARPS;
 #pragma unroll 1
             for (int p = 0; p < mine; ++p) {
-              // scores = K q and output = V^T p as 16 x 8 x 16 products; q and p are three columns (their bf16 parts) of the eight
-              const uint32_t mem = sb + C::QKV + p * C::QROW;
+              const uint8_t* mem = smem + C::QKV + p * C::QROW;
               const int set = C::WPU == NWARPS ? warp : (warp + 4 * p) & 7;  // where a unit has four tiles the other warps begin the next sample
-              uint32_t qf[2][4];
-              {
-                const int n = lane & 7;
-                const uint32_t at = n < 3 ? mem + n * 128 : sb + C::ZERO;
-                ldsm4(qf[0], at + q_piece * 16);
-                ldsm4(qf[1], at + 64 + q_piece * 16);
-              }
-              float o[4][4], m_run = -INFINITY, l_run = 0.f;
+              float2 q2[4], o2[4];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+              for (int i = 0; i < 4; i += 2) {
+                const float4 q4 = *reinterpret_cast<const float4*>(mem + sub * 32 + i * 8);
+                q2[i] = make_float2(q4.x, q4.y);
+                q2[i + 1] = make_float2(q4.z, q4.w);
+                o2[i] = o2[i + 1] = make_float2(0.f, 0.f);
+              }
+              float m_run = -INFINITY, l_run = 0.f;  // of this group of lanes
               const int tile_end = tiles > units * C::WPU ? tiles : units * C::WPU;
 #pragma unroll 1
               for (int tile = set; tile < tile_end; tile += NWARPS) {
@@ -733,57 +709,47 @@ seq_block_kernel(const __grid_constant__ Job job) {
                   __syncwarp();
                 }
                 if (tile < tiles) {
-                  // rows that are not there (the last of them is the new token's) read the new row
-                  const uint32_t kbase = sb + C::RING + at * C::UNIT + (tile % C::WPU) * 2048;
-                  const uint32_t vbase = sb + C::RING + av * C::UNIT + (C::KVS == 1 ? C::KPU * 128 : 0) + (tile % C::WPU) * 2048;
-                  const bool kin = tile * 16 + kr < t, vin = tile * 16 + vr < t;
-                  const uint32_t kat = kin ? kbase + kr * 128 : mem + 384, kx = kin ? kr & 7 : 0;
-                  const uint32_t vat = vin ? vbase + vr * 128 : mem + 512, vx = vin ? vr & 7 : 0;
-                  float sa[4] = {0.f, 0.f, 0.f, 0.f}, sc[4] = {0.f, 0.f, 0.f, 0.f};
-                  uint32_t a[4][4];
+                  const uint8_t* kbase = smem + C::RING + at * C::UNIT + (tile % C::WPU) * 2048;
+                  const uint8_t* vbase = smem + C::RING + av * C::UNIT + (C::KVS == 1 ? C::KPU * 128 : 0) + (tile % C::WPU) * 2048;
+                  uint4 kn[4], vn[4];
 #pragma unroll
-                  for (int k = 0; k < 4; ++k) ldsm4(a[k], kat + (((2 * k + k_piece) ^ kx) << 4));
+                  for (int k = 0; k < 4; ++k) {  // rows that are not in the ring (the first of them is the new token's) read the new row
+                    const int row = 4 * k + kgrp;
+                    const bool in = tile * 16 + row < t;
+                    kn[k] = *reinterpret_cast<const uint4*>(in ? kbase + swz128(row, sub) : mem + 256 + sub * 16);
+                    vn[k] = *reinterpret_cast<const uint4*>(in ? vbase + swz128(row, sub) : mem + 384 + sub * 16);
+                  }
+                  float sc[4];
 #pragma unroll
-                  for (int k = 0; k < 4; k += 2) {
-                    attn::mma_bf16(sa, a[k], qf[k / 2][0], qf[k / 2][1]);
-                    attn::mma_bf16(sc, a[k + 1], qf[k / 2][2], qf[k / 2][3]);
+                  for (int k = 0; k < 4; ++k) {
+                    const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kn[k]);
+                    float2 s2 = fmul2(q2[0], __bfloat1622float2(k2[0]));
+#pragma unroll
+                    for (int i = 1; i < 4; ++i) s2 = ffma2(q2[i], __bfloat1622float2(k2[i]), s2);
+                    sc[k] = s2.x + s2.y;
                   }
 #pragma unroll
-                  for (int k = 0; k < 4; ++k) ldsm4t(a[k], vat + (((2 * k + v_piece) ^ vx) << 4));
-                  // scores of keys lane / 4 and lane / 4 + 8, the same in all four lanes
-                  float s0 = (sa[0] + sc[0]) + (sa[1] + sc[1]), s1 = (sa[2] + sc[2]) + (sa[3] + sc[3]);
+                  for (int off = 1; off < 8; off <<= 1)
 #pragma unroll
-                  for (int off = 1; off < 4; off <<= 1) {
-                    s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-                    s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+                    for (int k = 0; k < 4; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], off);
+#pragma unroll
+                  for (int k = 0; k < 4; ++k)
+                    if (tile * 16 + 4 * k + kgrp > t) sc[k] = -INFINITY;
+                  const float m_new = fmaxf(fmaxf(m_run, fmaxf(sc[0], sc[1])), fmaxf(sc[2], sc[3]));
+                  const float m_ref = m_new > -INFINITY ? m_new : 0.f;  // a group that has seen no key yet keeps its zeros
+                  const float corr = ex2_approx(m_run - m_ref);         // 0 when m_run = -inf
+                  l_run *= corr;
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) o2[i] = fmul2(o2[i], make_float2(corr, corr));
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+                    const float pj = ex2_approx(sc[k] - m_ref);  // 0 for a masked key
+                    l_run += pj;
+                    const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&vn[k]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) o2[i] = ffma2(make_float2(pj, pj), __bfloat1622float2(v2[i]), o2[i]);
                   }
-                  const int key = tile * 16 + (lane >> 2);
-                  if (key > t) s0 = -INFINITY;
-                  if (key + 8 > t) s1 = -INFINITY;
-                  float mx = fmaxf(s0, s1);
-#pragma unroll
-                  for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-                  const float m_new = fmaxf(m_run, mx), corr = ex2_approx(m_run - m_new);  // a tile has a key: m_new is finite
-                  const float p0 = ex2_approx(s0 - m_new), p1 = ex2_approx(s1 - m_new);    // 0 for a masked key
                   m_run = m_new;
-                  l_run = fmaf(l_run, corr, p0 + p1);
-                  // part n = lane / 4 of the probabilities of keys 2 (lane % 4), + 1, + 8, + 9
-                  const int src = (lane & 3) * 8, n = lane >> 2;
-                  float pk[4] = {__shfl_sync(0xffffffffu, p0, src), __shfl_sync(0xffffffffu, p0, src + 4), __shfl_sync(0xffffffffu, p1, src),
-                                 __shfl_sync(0xffffffffu, p1, src + 4)};
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) {
-                    float part[3];
-                    split3(pk[k], part);
-                    pk[k] = n == 0 ? part[0] : n == 1 ? part[1] : n == 2 ? part[2] : 0.f;
-                  }
-                  const uint32_t b0 = pack_bf16(pk[0], pk[1]), b1 = pack_bf16(pk[2], pk[3]);
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) o[k][i] *= corr;
-                    attn::mma_bf16(o[k], a[k], b0, b1);
-                  }
                 }
                 if (unit < units) {
                   __syncwarp();
@@ -794,21 +760,25 @@ seq_block_kernel(const __grid_constant__ Job job) {
                   __syncwarp();
                 }
               }
-              if (set < sets) {
-                float* mg = s_merge + (p * NWARPS + set) * 72;
+              if (set < sets) {  // the warp's four groups; a lane keeps the half of the channels that its partner gives up
+                const float mw = fmaxf(fmaxf(m_run, __shfl_xor_sync(0xffffffffu, m_run, 8)),
+                                       fmaxf(__shfl_xor_sync(0xffffffffu, m_run, 16), __shfl_xor_sync(0xffffffffu, m_run, 24)));
+                const float f = ex2_approx(m_run - mw);  // mw is finite: the set has a key; 0 for a group without one
+                l_run *= f;
+                l_run += __shfl_xor_sync(0xffffffffu, l_run, 8);
+                l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);
+                float2 a[2];
 #pragma unroll
-                for (int off = 4; off < 32; off <<= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, off);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {  // the three columns of channels 16 k + lane / 4, + 8
-                  float x = o[k][0] + o[k][1], y = o[k][2] + o[k][3];
-                  x += __shfl_xor_sync(0xffffffffu, x, 1);
-                  y += __shfl_xor_sync(0xffffffffu, y, 1);
-                  if ((lane & 3) == 0) {
-                    mg[16 * k + (lane >> 2)] = x;
-                    mg[16 * k + 8 + (lane >> 2)] = y;
-                  }
+                for (int i = 0; i < 2; ++i) {  // channels 0-3 stay with the groups 0 and 2, 4-7 with 1 and 3
+                  const float2 x = fmul2(o2[i], make_float2(f, f)), y = fmul2(o2[i + 2], make_float2(f, f));
+                  const float2 keep = kgrp & 1 ? y : x, send = kgrp & 1 ? x : y;
+                  a[i] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, send.x, 8), keep.y + __shfl_xor_sync(0xffffffffu, send.y, 8));
                 }
-                if (lane == 0) { mg[64] = m_run; mg[65] = l_run; }
+                const float2 keep = kgrp & 2 ? a[1] : a[0], send = kgrp & 2 ? a[0] : a[1];
+                float* mg = s_merge + (p * NWARPS + set) * 72;
+                *reinterpret_cast<float2*>(mg + 8 * sub + 4 * (kgrp & 1) + (kgrp & 2)) =
+                    make_float2(keep.x + __shfl_xor_sync(0xffffffffu, send.x, 16), keep.y + __shfl_xor_sync(0xffffffffu, send.y, 16));
+                if (lane == 0) { mg[64] = mw; mg[65] = l_run; }
               }
               __syncwarp();
             }
@@ -819,28 +789,37 @@ seq_block_kernel(const __grid_constant__ Job job) {
             }
             cbar();
 #pragma unroll 1
-            for (int i = tid; i < mine * 8 * CS; i += NTHREADS) {  // all-gather: (receiving CTA, eight channels, sample)
-              const int peer = i & (CS - 1), c8 = (i / CS) & 7, p = i / (8 * CS);
-              const float* mg = s_merge + p * NWARPS * 72;
-              float mx = mg[64];
-#pragma unroll 1
-              for (int k = 1; k < sets; ++k) mx = fmaxf(mx, mg[k * 72 + 64]);
+            for (int i = tid; i < mine * 64; i += NTHREADS) {  // the sets (eight lanes per eight channels of a sample), all-gather
+              const int k = i & 7, c8 = (i >> 3) & 7, p = i >> 6;
+              const float* mg = s_merge + (p * NWARPS + k) * 72;
+              const bool has = k < sets;
+              const float m_set = has ? mg[64] : -INFINITY;
+              float mx = m_set;
+#pragma unroll
+              for (int off = 1; off < 8; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
               float den = 0.f, num[8];
 #pragma unroll
               for (int z = 0; z < 8; ++z) num[z] = 0.f;
-#pragma unroll 1
-              for (int k = 0; k < sets; ++k) {
-                const float e = ex2_approx(mg[k * 72 + 64] - mx);
-                den = fmaf(e, mg[k * 72 + 65], den);
-                const float4 a = *reinterpret_cast<const float4*>(mg + k * 72 + 8 * c8);
-                const float4 b = *reinterpret_cast<const float4*>(mg + k * 72 + 8 * c8 + 4);
-                num[0] = fmaf(e, a.x, num[0]); num[1] = fmaf(e, a.y, num[1]); num[2] = fmaf(e, a.z, num[2]); num[3] = fmaf(e, a.w, num[3]);
-                num[4] = fmaf(e, b.x, num[4]); num[5] = fmaf(e, b.y, num[5]); num[6] = fmaf(e, b.z, num[6]); num[7] = fmaf(e, b.w, num[7]);
+              if (has) {
+                const float e = ex2_approx(m_set - mx);
+                den = e * mg[65];
+                const float4 a = *reinterpret_cast<const float4*>(mg + 8 * c8), b = *reinterpret_cast<const float4*>(mg + 8 * c8 + 4);
+                num[0] = e * a.x; num[1] = e * a.y; num[2] = e * a.z; num[3] = e * a.w;
+                num[4] = e * b.x; num[5] = e * b.y; num[6] = e * b.z; num[7] = e * b.w;
+              }
+              __syncwarp();
+#pragma unroll
+              for (int off = 1; off < 8; off <<= 1) {
+                den += __shfl_xor_sync(0xffffffffu, den, off);
+#pragma unroll
+                for (int z = 0; z < 8; ++z) num[z] += __shfl_xor_sync(0xffffffffu, num[z], off);
               }
               const float inv = 1.f / den;
-              st_async4(peer_addr(sb + C::ACT + swz128(r * bl + p, c8), peer), pack_bf16(num[0] * inv, num[1] * inv),
-                        pack_bf16(num[2] * inv, num[3] * inv), pack_bf16(num[4] * inv, num[5] * inv), pack_bf16(num[6] * inv, num[7] * inv),
-                        peer_addr(bar(B_ALL0), peer));
+              if (k < CS)
+                st_async4(peer_addr(sb + C::ACT + swz128(r * bl + p, c8), k), pack_bf16(num[0] * inv, num[1] * inv),
+                          pack_bf16(num[2] * inv, num[3] * inv), pack_bf16(num[4] * inv, num[5] * inv), pack_bf16(num[6] * inv, num[7] * inv),
+                          peer_addr(bar(B_ALL0), k));
+              __syncwarp();
             }
             fence_proxy_async_global();  // the new cache rows: the next step's bulk copies, long after the barriers below, read them
           }
