@@ -789,8 +789,8 @@ seq_block_kernel(const __grid_constant__ Job job) {
             }
             cbar();
 #pragma unroll 1
-            for (int i = tid; i < mine * 64; i += NTHREADS) {  // the sets (eight lanes per eight channels of a sample), all-gather
-              const int k = i & 7, c8 = (i >> 3) & 7, p = i >> 6;
+            for (int i = warp; i < mine * 2; i += NWARPS) {  // the sets (eight lanes per eight channels of a sample), all-gather
+              const int k = lane & 7, c8 = (i & 1) * 4 + (lane >> 3), p = i >> 1;
               const float* mg = s_merge + (p * NWARPS + k) * 72;
               const bool has = k < sets;
               const float m_set = has ? mg[64] : -INFINITY;
