@@ -202,6 +202,11 @@ __device__ __forceinline__ void prefetch_tile(const CUtensorMap* map, int x, int
 }
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
+__device__ __forceinline__ uint4 lds128(uint32_t at) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+  return v;
+}
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 o = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&o);
@@ -709,15 +714,15 @@ seq_block_kernel(const __grid_constant__ Job job) {
                   __syncwarp();
                 }
                 if (tile < tiles) {
-                  const uint8_t* kbase = smem + C::RING + at * C::UNIT + (tile % C::WPU) * 2048;
-                  const uint8_t* vbase = smem + C::RING + av * C::UNIT + (C::KVS == 1 ? C::KPU * 128 : 0) + (tile % C::WPU) * 2048;
+                  const uint32_t kbase = sb + C::RING + at * C::UNIT + (tile % C::WPU) * 2048, new_row = sb + C::QKV + p * C::QROW + 256 + sub * 16;
+                  const uint32_t vbase = sb + C::RING + av * C::UNIT + (C::KVS == 1 ? C::KPU * 128 : 0) + (tile % C::WPU) * 2048;
                   uint4 kn[4], vn[4];
 #pragma unroll
                   for (int k = 0; k < 4; ++k) {  // rows that are not in the ring (the first of them is the new token's) read the new row
                     const int row = 4 * k + kgrp;
                     const bool in = tile * 16 + row < t;
-                    kn[k] = *reinterpret_cast<const uint4*>(in ? kbase + swz128(row, sub) : mem + 256 + sub * 16);
-                    vn[k] = *reinterpret_cast<const uint4*>(in ? vbase + swz128(row, sub) : mem + 384 + sub * 16);
+                    kn[k] = lds128(in ? kbase + swz128(row, sub) : new_row);
+                    vn[k] = lds128(in ? vbase + swz128(row, sub) : new_row + 128);
                   }
                   float sc[4];
 #pragma unroll
