@@ -96,7 +96,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
   constexpr int KV_STAGES = C::KV_STAGES, KV_RING = C::KV_RING;
   extern __shared__ uint8_t smem_attn_raw[];
   pdl_launch_dependents();  // the next kernel of the stream may be scheduled; it waits for this one to complete
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_attn_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(smem_attn_raw);
   const uint32_t sQ = smem_u32(smem), sK = sQ + C::Q_ALL, sV = sK + KV_STAGES * C::K_SLOT, sP = sV + KV_STAGES * C::V_SLOT;
   const uint32_t bar_base = sP + C::P_ALL;
   // barriers: 0 q_full, then k_full[st], k_empty[st], v_full[st], v_empty[st], s_full, s_free, p_ready, o_done

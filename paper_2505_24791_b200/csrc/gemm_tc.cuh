@@ -29,6 +29,9 @@ constexpr int NUM_THREADS = 64 + 32 * NUM_EPI_WARPS;
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;  // 2 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Dynamic shared memory from the next 1024-byte boundary on.  By an offset, not by rounding the pointer as an integer: from that
+// the compiler cannot tell the address space any more, and every access becomes a generic one.
+__device__ __forceinline__ uint8_t* align1024(uint8_t* p) { return p + ((1024u - (smem_u32(p) & 1023u)) & 1023u); }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
   unsigned long long t;
@@ -215,7 +218,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   pdl_launch_dependents();  // the next kernel of the stream may be scheduled; it waits for this one to complete
 
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(smem_raw);
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar_base = smem_base + SL::BAR_OFFSET;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };

@@ -92,7 +92,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   using SL = Smem2;
   extern __shared__ uint8_t smem_raw2[];
   pdl_launch_dependents();  // the next kernel of the stream may be scheduled; it waits for this one to complete
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw2) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(smem_raw2);
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar_base = smem_base + SL::BAR_OFFSET;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };

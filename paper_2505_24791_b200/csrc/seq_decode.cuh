@@ -281,7 +281,7 @@ seq_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
   constexpr int W_BYTES = 128 * 64 * 2, A_BYTES = RT * 64 * 2, STAGE = W_BYTES + A_BYTES;
   constexpr uint32_t TMEM_COLS = RT < 32 ? 32 : RT;
   extern __shared__ uint8_t smem_seq_tc[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_seq_tc) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(smem_seq_tc);
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar_base = smem_base + NS * STAGE;  // full[0..NS-1], done
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + NS * STAGE + 96);

@@ -318,7 +318,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
   using C = Cfg<D, RT>;
   constexpr int HEADS = C::HEADS, CS = C::CS, N1 = C::N1, CW = C::CW, QN = C::QN, SG = C::SG, NSL = C::NSL, UPC = C::UPC, NE = C::NE, NA = C::NA;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align1024(smem_raw);
   const uint32_t sb = smem_u32(smem), bars = sb + C::BARS;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int r = blockIdx.x % CS, cl = blockIdx.x / CS, c = cl % HEADS, group = cl / HEADS;  // r: rank in the cluster
