@@ -217,8 +217,9 @@ struct tf_model {
   bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
   int seq_attn_threads = 0;  // TARFLOW_SEQ_ATTN_THREADS=128|256: CTA size of the step attention (0 = by the number of CTAs)
   int seq_kbn_force = 0;     // TARFLOW_SEQ_KBN
-  // Jacobi sweeps over few rows are replayed from graphs: one per (block, single-term slots, two-term slots, buffers)
-  std::map<std::tuple<int, int, int, const void*, const void*, const void*, const void*>, SeqGraph> sweep_graphs;
+  // Jacobi sweeps over few rows are replayed from graphs: one per (block, single-term slots, two-term slots, buffers).  The
+  // current slot list is one of the buffers: idx and idx_tmp change places after every sweep of more than FIN_CHUNK samples.
+  std::map<std::tuple<int, int, int, const void*, const void*, const void*, const void*, const void*>, SeqGraph> sweep_graphs;
   int small_m_rows = 1024;      // TARFLOW_SMALL_M_ROWS: sweeps of at most this many rows use 128 x 128 single-CTA tiles
   int split_m_rows = 4096;      // TARFLOW_SPLIT_M_ROWS: up to this many rows the residual projections on pair tiles are cut in K too
   bool small_m_split = true;    // TARFLOW_SMALL_M_SPLIT=0: the residual projections of such sweeps keep whole-K tiles
@@ -1406,7 +1407,8 @@ static int run_jacobi_block(tf_model* m, int g, int B, const int* labels, const 
     // captured once per (block, single-term slots, two-term slots) and replayed as a graph afterwards.
     const bool as_graph = m->use_graphs && m->cap_stream != nullptr && !m->prof_on && n_active <= FIN_CHUNK && (int64_t)(first ? 1 : n_active) * m->L <= m->sweep_graph_rows;
     if (as_graph) {
-      const auto key = std::make_tuple(g, first ? -1 - n_lp : n_lp, n_hp, (const void*)v, (const void*)u, (const void*)labels, (const void*)iters_row);
+      const auto key = std::make_tuple(g, first ? -1 - n_lp : n_lp, n_hp, (const void*)v, (const void*)u, (const void*)labels, (const void*)iters_row,
+                                       (const void*)m->idx);
       auto it = m->sweep_graphs.find(key);
       if (it == m->sweep_graphs.end() && m->sweep_graphs.size() < 2048) {
         tf_model::SeqGraph sg;

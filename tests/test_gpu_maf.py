@@ -175,3 +175,18 @@ def test_bf16_mnist_shape_ragged_k_and_head_width():
         xf, _, itf, rc = m.jacobi(z[:3], -1.0, 5)                   # fixed sweeps: the same iterate as the oracle's
         xfo, _ = MO.model_inverse(m.blocks, z[:3], -1.0, 5)
         assert rc == 0 and rel_l2(xf, xfo) <= 2e-2 and np.abs(xf - xfo).max() <= 5e-2
+
+
+def test_calls_of_changing_batch_on_one_handle_give_the_same_result():
+    """Sweeps of more than 1024 samples write the new slot list to a second buffer, sweeps of few rows are replayed from
+    graphs that hold the buffers' addresses: 9 large sweeps (3 blocks x 3) leave the other buffer current."""
+    cfg = synth.maf_config("maf_ising", D=64, hidden=128, n_blocks=3)
+    with Maf(cfg, 1100) as m:
+        z = synth.make_maf_latents(cfg, 24, B=1100)
+        first = {B: m.jacobi(z[:B], 1e-3, m.D + 1) for B in (3, 60, 500)}
+        for _ in range(2):
+            _, _, _, rc = m.jacobi(z, -1.0, 3)
+            assert rc == 0
+            for B, (x0, ib0, its0, rc0) in first.items():
+                x, ib, its, rc = m.jacobi(z[:B], 1e-3, m.D + 1)
+                assert rc == rc0 == 0 and np.array_equal(x, x0) and np.array_equal(its, its0) and np.array_equal(ib, ib0), B
