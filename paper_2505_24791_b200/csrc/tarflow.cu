@@ -217,6 +217,7 @@ struct tf_model {
   bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
   int seq_attn_threads = 0;  // TARFLOW_SEQ_ATTN_THREADS=128|256: CTA size of the step attention (0 = by the number of CTAs)
   int seq_kbn_force = 0;     // TARFLOW_SEQ_KBN
+  bool seq_nc_forced = false;  // TARFLOW_SEQ_NC is set
   // Jacobi sweeps over few rows are replayed from graphs: one per (block, single-term slots, two-term slots, buffers).  The
   // current slot list is one of the buffers: idx and idx_tmp change places after every sweep of more than FIN_CHUNK samples.
   std::map<std::tuple<int, int, int, const void*, const void*, const void*, const void*, const void*>, SeqGraph> sweep_graphs;
@@ -1181,8 +1182,10 @@ static int seqp_setup(tf_model* m) {
 // Batches that need more than one launch go to the chain of kernels, whose cost hardly grows with the batch (width 1024,
 // 96 samples: 135 ms in two launches).
 static bool seqp_on(const tf_model* m, int B) {
-  return !m->seqp_layers.empty() && m->seq_use_persist && m->seq_use_tc && !m->seq_fin && !m->seq_fuse_gelu && m->seq_fuse_tail < 0 &&
-         B <= 32 * m->seqp_groups[1];
+  // a switch of the step kernels asks for the chain they belong to
+  const bool chain_wanted = !m->seq_use_tc || m->seq_fin || m->seq_fuse_gelu || m->seq_fuse_tail >= 0 || m->seq_chains_force > 0 ||
+                            m->seq_kbn_force > 0 || m->seq_attn_threads > 0 || m->seq_nc_forced || !m->seq_kbn8;
+  return !m->seqp_layers.empty() && m->seq_use_persist && !chain_wanted && B <= 32 * m->seqp_groups[1];
 }
 
 static int run_sequential_persistent(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
@@ -2046,6 +2049,7 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
     if (const char* e = getenv("TARFLOW_SEQ_KBN")) m->seq_kbn_force = atoi(e);
     if (const char* e = getenv("TARFLOW_SEQ_FIN")) m->seq_fin = atoi(e) != 0;
     if (const char* e = getenv("TARFLOW_SEQ_ATTN_THREADS")) m->seq_attn_threads = atoi(e);
+    m->seq_nc_forced = getenv("TARFLOW_SEQ_NC") != nullptr;
     TF_TRY(dev_alloc(m, &m->seq_tickets, (size_t)tf_model::MAX_CHAINS * tf_model::SEQ_TICKETS));
     CU_OK(cudaMemset(m->seq_tickets, 0, (size_t)tf_model::MAX_CHAINS * tf_model::SEQ_TICKETS * sizeof(int)));
     TF_TRY(dev_alloc(m, &m->seq_stats, (size_t)tf_model::MAX_CHAINS * 16 * B));
