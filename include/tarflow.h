@@ -30,8 +30,9 @@
  *     them: an id outside [0, n_classes) makes the call return TF_EINVAL (no table is ever indexed with it).
  *   - Tuning aids read from the environment (bf16 engine, sequential decoding only; results are unchanged
  *     up to summation order): TARFLOW_SEQ_PERSIST=0 decodes every block by the chain of step kernels instead of one
- *     cooperative launch (widths 128, 256, 512 and 1024 with an MLP ratio of 4, batches that fit the GPU at once); every
- *     other TARFLOW_SEQ_* switch with a value other than its default selects that chain too.  TARFLOW_SEQ_MMA=1 selects the mma.sync step GEMM instead of the tcgen05 one,
+ *     cooperative launch (widths 128, 256, 512 and 1024 with an MLP ratio of 4, batches that fit the GPU at once; where
+ *     CUDA refuses that launch the chain runs too); every other TARFLOW_SEQ_* switch with a value other than its
+ *     default selects that chain.  TARFLOW_SEQ_MMA=1 selects the mma.sync step GEMM instead of the tcgen05 one,
  *     TARFLOW_SEQ_KBN=1|2|4 the 64-wide k slabs per CTA of the tcgen05 step GEMM, TARFLOW_SEQ_NC=8|16|32|64
  *     the column-slice width of the mma.sync step GEMM, TARFLOW_SEQ_FUSE_GELU=1 lets the MLP-up step GEMM
  *     apply bias + GELU itself when its reduction fits one CTA (K <= 512), TARFLOW_SEQ_FUSE_TAIL=0|1 switches the one-kernel
@@ -340,6 +341,14 @@ int tf_selftest_wait_timeout(tf_model* m, int32_t limit_us, void* cuda_stream);
  * negative = error).  It synchronises the stream.  A substitute for a memory checker where none can be run.
  */
 int64_t tf_debug_check_guards(tf_model* m, void* cuda_stream);
+
+/*
+ * tf_debug_set -- brings about, for tests, what is otherwise rare.  Affects the given model only.
+ *   TF_DEBUG_REFUSE_BLOCK_LAUNCH  value != 0: the launch that decodes a block at once asks for more shared memory than a CTA
+ *                                 can have, so that the CUDA runtime turns it down and the chain of step kernels runs.
+ */
+#define TF_DEBUG_REFUSE_BLOCK_LAUNCH 0
+int tf_debug_set(tf_model* m, int32_t what, int64_t value);
 
 /* tf_device_bytes -- device memory owned by the model (weights + workspace + KV cache), bytes. */
 int64_t tf_device_bytes(tf_model* m);

@@ -76,6 +76,7 @@ def lib():
         L.tf_selftest_wait_timeout.argtypes = [vp, i32, vp]
         L.tf_debug_check_guards.argtypes = [vp, vp]
         L.tf_debug_check_guards.restype = C.c_int64
+        L.tf_debug_set.argtypes = [vp, i32, C.c_int64]
         L.tf_launch_count.argtypes = [vp]
         L.tf_launch_count.restype = C.c_int64
         L.tf_device_bytes.argtypes = [vp]
@@ -260,6 +261,13 @@ def tf_debug_check_guards(m, stream=None):
     if n < 0:
         _check(int(n))
     return int(n)
+
+
+TF_DEBUG_REFUSE_BLOCK_LAUNCH = 0
+
+
+def tf_debug_set(m, what, value):
+    return _check(lib().tf_debug_set(m, int(what), int(value)))
 
 
 def tf_launch_count(m):

@@ -215,6 +215,7 @@ struct tf_model {
   unsigned long long *seqp_part = nullptr, *seqp_row = nullptr;
   CUtensorMap seqp_cache[2];                   // keys, values
   bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
+  bool seqp_debug_refuse = false;              // tf_debug_set: the launch asks for what no CTA can have
   int seq_attn_threads = 0;  // TARFLOW_SEQ_ATTN_THREADS=128|256: CTA size of the step attention (0 = by the number of CTAs)
   int seq_kbn_force = 0;     // TARFLOW_SEQ_KBN
   bool seq_nc_forced = false;  // TARFLOW_SEQ_NC is set
@@ -291,6 +292,9 @@ struct tf_model {
       cur_start = get_event();
       cudaEventRecord(cur_start, stream);
     }
+  }
+  void drop() {  // the launch announced by pre() did not take place
+    if (prof_on && !prof_suspend) ev_pool.push_back(cur_start);
   }
   void post(int cls) {
     ++launches;
@@ -1107,7 +1111,9 @@ static SeqpShape seqp_shape_of(int d, int rt) {
   return d == 1024 ? seqp_shape<1024, 32>() : d == 512 ? seqp_shape<512, 32>() : d == 256 ? seqp_shape<256, 32>() : seqp_shape<128, 32>();
 }
 
-// launches (max_clusters == nullptr), or asks how many clusters fit the GPU side by side
+constexpr int kLaunchRefused = 1;
+// Launches (max_clusters == nullptr), or asks how many clusters fit the GPU side by side.  Returns kLaunchRefused when the
+// launch was turned down and the context is none the worse for it (fewer SMs than at load, a tool that allows no such launch).
 static int seqp_launch(tf_model* m, const SeqpShape& sh, int groups, const seqp::Job* job, int* max_clusters) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(groups * sh.heads * sh.cs);
@@ -1129,9 +1135,12 @@ static int seqp_launch(tf_model* m, const SeqpShape& sh, int groups, const seqp:
     }
     return TF_OK;
   }
+  if (m->seqp_debug_refuse) lc.dynamicSmemBytes = 1u << 20;
   const cudaError_t e = cudaLaunchKernelEx(&lc, sh.kern, *job);
-  if (e != cudaSuccess) return fail(TF_ECUDA, "seq_block_kernel launch failed: %s", cudaGetErrorString(e));
-  return TF_OK;
+  if (e == cudaSuccess) return TF_OK;
+  cudaGetLastError();
+  if (cudaPeekAtLastError() == cudaSuccess && e != cudaErrorLaunchFailure) return kLaunchRefused;  // an error of the context stays
+  return fail(TF_ECUDA, "seq_block_kernel launch failed: %s", cudaGetErrorString(e));
 }
 
 // at load: whether the shape fits, the layers' tables, the exchange buffers
@@ -1188,6 +1197,7 @@ static bool seqp_on(const tf_model* m, int B) {
   return !m->seqp_layers.empty() && m->seq_use_persist && !chain_wanted && B <= 32 * m->seqp_groups[1];
 }
 
+// TF_OK, kLaunchRefused (nothing has run) or an error
 static int run_sequential_persistent(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
   const BlockW& bw = m->blocks[g];
   const int L = m->L, D = m->D, nl = m->cfg.n_layers, n_steps = L - 1;
@@ -1216,13 +1226,17 @@ static int run_sequential_persistent(tf_model* m, int g, int B, const int* label
   job.err = m->err;
   m->cur_rows = (int64_t)B * n_steps;
   m->pre(KC_SEQ_BLOCK);
-  TF_TRY(seqp_launch(m, sh, (B + job.rows - 1) / job.rows, &job, nullptr));
-  m->post(KC_SEQ_BLOCK);
-  return TF_OK;
+  const int r = seqp_launch(m, sh, (B + job.rows - 1) / job.rows, &job, nullptr);
+  if (r == TF_OK) m->post(KC_SEQ_BLOCK);
+  else m->drop();
+  return r;
 }
 
 static int run_sequential_block_bf16(tf_model* m, int g, int B, const int* labels, const float* v, float* u) {
-  if (seqp_on(m, B)) return run_sequential_persistent(m, g, B, labels, v, u);
+  if (seqp_on(m, B)) {
+    const int r = run_sequential_persistent(m, g, B, labels, v, u);
+    if (r != kLaunchRefused) return r;  // refused: the chain of kernels needs no cooperation
+  }
   const int n_steps = m->L - 1;
   cudaStream_t user = m->stream;
   const bool direct = (m->prof_on && m->prof_mode == 1) || !m->use_graphs;
@@ -2558,6 +2572,15 @@ int64_t tf_debug_check_guards(tf_model* m, void* cuda_stream) {
   CU_OK(cudaStreamSynchronize(st));
   if (bad != 0) fail(TF_OK, "%d guard words next to the model's device buffers were overwritten", bad);
   return bad;
+}
+
+int tf_debug_set(tf_model* m, int32_t what, int64_t value) {
+  g_err[0] = 0;
+  if (!m) return fail(TF_EINVAL, "model is NULL");
+  switch (what) {
+    case TF_DEBUG_REFUSE_BLOCK_LAUNCH: m->seqp_debug_refuse = value != 0; return TF_OK;
+  }
+  return fail(TF_EINVAL, "unknown debug setting %d", what);
 }
 
 int tf_profile_enable(tf_model* m, int32_t on) {

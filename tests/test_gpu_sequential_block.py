@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 from oracle import tarflow_oracle as O
-from paper_2505_24791_b200 import synth
+from paper_2505_24791_b200 import binding, synth
 from tests.gpu_util import Model, rel_l2
 
 pytestmark = pytest.mark.gpu
@@ -47,3 +47,23 @@ def test_fp32_block_in_one_launch(batch):
     with Model(cfg, max_batch=batch) as m:
         x = m.inverse_sequential(z, None)
         assert np.abs(x - O.model_inverse_sequential(m.blocks, z, None, cfg)).max() <= FP32_MAX
+
+
+def test_bf16_block_whose_launch_is_refused_runs_as_a_chain(monkeypatch):
+    cfg = synth.config("cfg2", H=12, W=12, n_blocks=2, n_layers=1, width=128, n_heads=2)
+    z = synth.make_latents(cfg, 9, B=5)
+    monkeypatch.setenv("TARFLOW_SEQ_PERSIST", "0")
+    with Model(cfg, max_batch=5) as m:
+        chain = m.inverse_sequential(z, None)
+    monkeypatch.delenv("TARFLOW_SEQ_PERSIST")
+    with Model(cfg, max_batch=5) as m:
+        at_once = m.inverse_sequential(z, None)
+        binding.tf_debug_set(m.m, binding.TF_DEBUG_REFUSE_BLOCK_LAUNCH, 1)
+        for profile in (0, 2):
+            binding.tf_profile_enable(m.m, profile)
+            assert np.array_equal(m.inverse_sequential(z, None), chain)
+        binding.tf_profile_enable(m.m, 0)
+        x, _, _, rc = m.inverse(z, None, [0, 1], 1e-3, m.L + 1)    # nothing of the refusal is left for later launches to report
+        assert rc == 0 and np.isfinite(x).all()
+        binding.tf_debug_set(m.m, binding.TF_DEBUG_REFUSE_BLOCK_LAUNCH, 0)
+        assert np.array_equal(m.inverse_sequential(z, None), at_once)
