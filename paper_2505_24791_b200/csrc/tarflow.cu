@@ -14,6 +14,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -215,6 +216,7 @@ struct tf_model {
   unsigned long long *seqp_part = nullptr, *seqp_row = nullptr;
   CUtensorMap seqp_cache[2];                   // keys, values
   bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
+  int seqp_turn = -1;                          // device whose SeqpTurn this model shares (-1: none)
   bool seqp_debug_refuse = false;              // tf_debug_set: the launch asks for what no CTA can have
   int seq_attn_threads = 0;  // TARFLOW_SEQ_ATTN_THREADS=128|256: CTA size of the step attention (0 = by the number of CTAs)
   int seq_kbn_force = 0;     // TARFLOW_SEQ_KBN
@@ -1143,6 +1145,37 @@ static int seqp_launch(tf_model* m, const SeqpShape& sh, int groups, const seqp:
   return fail(TF_ECUDA, "seq_block_kernel launch failed: %s", cudaGetErrorString(e));
 }
 
+// The one-launch blocks of a device take turns.  The CTAs of such a launch wait on one another, so two of them that start side
+// by side (two models, two streams) could each hold SMs that the other one's missing CTAs need, until the waits run out.  Every
+// launch therefore waits for the one before it; the event lives as long as a model that may launch.  A chain of launches on
+// one stream is ordered anyway and pays for an event record and a wait per block.
+struct SeqpTurn {
+  std::mutex mu;
+  int models = 0;
+  cudaEvent_t done = nullptr;
+};
+static SeqpTurn g_seqp_turn[kMaxDevices];
+static int seqp_turn_join(tf_model* m) {
+  const int dev = current_device();
+  if (dev < 0) return fail(TF_ECUDA, "no usable current device");
+  SeqpTurn& t = g_seqp_turn[dev];
+  std::lock_guard<std::mutex> lock(t.mu);
+  if (t.models == 0) CU_OK(cudaEventCreateWithFlags(&t.done, cudaEventDisableTiming));
+  ++t.models;
+  m->seqp_turn = dev;
+  return TF_OK;
+}
+static void seqp_turn_leave(tf_model* m) {
+  if (m->seqp_turn < 0) return;
+  SeqpTurn& t = g_seqp_turn[m->seqp_turn];
+  std::lock_guard<std::mutex> lock(t.mu);
+  if (--t.models == 0) {
+    cudaEventDestroy(t.done);
+    t.done = nullptr;
+  }
+  m->seqp_turn = -1;
+}
+
 // at load: whether the shape fits, the layers' tables, the exchange buffers
 static int seqp_setup(tf_model* m) {
   const int d = m->d;
@@ -1162,6 +1195,7 @@ static int seqp_setup(tf_model* m) {
   if (m->seqp_groups[0] == 0 || m->seqp_groups[1] == 0) return TF_OK;
   const int64_t cache_rows = (int64_t)m->cfg.n_layers * m->cfg.max_batch * m->cfg.n_heads * m->L;
   if (cache_rows > INT_MAX - 32) return TF_OK;
+  TF_TRY(seqp_turn_join(m));
   TF_TRY(make_map_bf16(&m->seqp_cache[0], m->kcache, cache_rows, seqp::HD, 32));
   TF_TRY(make_map_bf16(&m->seqp_cache[1], m->vcache, cache_rows, seqp::HD, 32));
   TF_TRY(dev_alloc(m, &m->seqp_part, part));
@@ -1225,10 +1259,17 @@ static int run_sequential_persistent(tf_model* m, int g, int B, const int* label
   job.scale_log2e = 1.4426950408889634f / sqrtf((float)m->hd);
   job.err = m->err;
   m->cur_rows = (int64_t)B * n_steps;
-  m->pre(KC_SEQ_BLOCK);
-  const int r = seqp_launch(m, sh, (B + job.rows - 1) / job.rows, &job, nullptr);
-  if (r == TF_OK) m->post(KC_SEQ_BLOCK);
-  else m->drop();
+  int r;
+  {
+    SeqpTurn& turn = g_seqp_turn[m->seqp_turn];
+    std::lock_guard<std::mutex> lock(turn.mu);
+    CU_OK(cudaStreamWaitEvent(m->stream, turn.done, 0));
+    m->pre(KC_SEQ_BLOCK);
+    r = seqp_launch(m, sh, (B + job.rows - 1) / job.rows, &job, nullptr);
+    if (r == TF_OK) m->post(KC_SEQ_BLOCK);
+    else m->drop();
+    if (r == TF_OK) CU_OK(cudaEventRecord(turn.done, m->stream));
+  }
   return r;
 }
 
@@ -2249,6 +2290,7 @@ void tf_free(tf_model* m) {
   if (!m) return;
   cudaDeviceSynchronize();
   m->prof_collect();
+  seqp_turn_leave(m);
   for (cudaEvent_t e : m->ev_pool) cudaEventDestroy(e);
   for (cudaEvent_t e : m->block_ev) if (e) cudaEventDestroy(e);
   for (auto& kv : m->seq_graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);

@@ -4,8 +4,11 @@ bf16 engine: the cooperative kernel runs groups of at most 16 or 32 samples side
 and units of 64 or 128 keys; 132 tokens cross both, the batches leave groups and ranks short or without samples.  fp32 engine:
 1, 2 or 4 samples per cluster.
 """
+import threading
+
 import numpy as np
 import pytest
+import torch
 
 from oracle import tarflow_oracle as O
 from paper_2505_24791_b200 import binding, synth
@@ -67,3 +70,35 @@ def test_bf16_block_whose_launch_is_refused_runs_as_a_chain(monkeypatch):
         assert rc == 0 and np.isfinite(x).all()
         binding.tf_debug_set(m.m, binding.TF_DEBUG_REFUSE_BLOCK_LAUNCH, 0)
         assert np.array_equal(m.inverse_sequential(z, None), at_once)
+
+
+def test_bf16_blocks_of_two_models_on_two_streams():
+    """Launches whose CTAs wait on one another take turns: two handles, two threads, two streams, as many blocks as each decodes."""
+    cfg = synth.config("cfg2", H=12, W=12, n_blocks=4, n_layers=2, width=256, n_heads=4)
+    B = 70   # more than half of the GPU's SMs each
+    z = torch.from_numpy(synth.make_latents(cfg, 10, B=B)).cuda()
+    with Model(cfg, max_batch=B) as a, Model(cfg, max_batch=B) as b:
+        want = a.inverse_sequential(z.cpu().numpy(), None)
+        got, failed = {}, []
+
+        def decode(m, name):
+            try:
+                stream = torch.cuda.Stream()
+                with torch.cuda.stream(stream):
+                    x = torch.empty_like(z)
+                    for _ in range(8):
+                        x.fill_(float("nan"))
+                        binding.tf_inverse_sequential(m.m, z, None, B, x)
+                        got.setdefault(name, []).append(x.cpu().numpy())
+            except Exception as e:  # noqa: BLE001 -- reported below, by the test's own thread
+                failed.append(e)
+
+        torch.cuda.synchronize()
+        threads = [threading.Thread(target=decode, args=(m, n)) for n, m in (("a", a), ("b", b))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert not failed, failed
+        for name in ("a", "b"):
+            assert len(got[name]) == 8 and all(np.array_equal(x, want) for x in got[name])
