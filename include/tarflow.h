@@ -31,7 +31,8 @@
  *   - Tuning aids read from the environment (bf16 engine, sequential decoding only; results are unchanged
  *     up to summation order): TARFLOW_SEQ_PERSIST=0 decodes every block by the chain of step kernels instead of one
  *     cooperative launch (widths 128, 256, 512 and 1024 with an MLP ratio of 4, batches that fit the GPU at once; where
- *     CUDA refuses that launch the chain runs too); every other TARFLOW_SEQ_* switch with a value other than its
+ *     CUDA refuses that launch the chain runs too; models of one process take turns with it, processes that share a GPU
+ *     through MPS should switch it off); every other TARFLOW_SEQ_* switch with a value other than its
  *     default selects that chain.  TARFLOW_SEQ_MMA=1 selects the mma.sync step GEMM instead of the tcgen05 one,
  *     TARFLOW_SEQ_KBN=1|2|4 the 64-wide k slabs per CTA of the tcgen05 step GEMM, TARFLOW_SEQ_NC=8|16|32|64
  *     the column-slice width of the mma.sync step GEMM, TARFLOW_SEQ_FUSE_GELU=1 lets the MLP-up step GEMM
@@ -346,8 +347,11 @@ int64_t tf_debug_check_guards(tf_model* m, void* cuda_stream);
  * tf_debug_set -- brings about, for tests, what is otherwise rare.  Affects the given model only.
  *   TF_DEBUG_REFUSE_BLOCK_LAUNCH  value != 0: the launch that decodes a block at once asks for more shared memory than a CTA
  *                                 can have, so that the CUDA runtime turns it down and the chain of step kernels runs.
+ *   TF_DEBUG_EXCHANGE_NUMBER      the next sequence number of the words such a launch exchanges, at least the current one and
+ *                                 at most 2^32 - 1 (a number that long decoding reaches by itself).
  */
 #define TF_DEBUG_REFUSE_BLOCK_LAUNCH 0
+#define TF_DEBUG_EXCHANGE_NUMBER 1
 int tf_debug_set(tf_model* m, int32_t what, int64_t value);
 
 /* tf_device_bytes -- device memory owned by the model (weights + workspace + KV cache), bytes. */

@@ -263,7 +263,7 @@ def tf_debug_check_guards(m, stream=None):
     return int(n)
 
 
-TF_DEBUG_REFUSE_BLOCK_LAUNCH = 0
+TF_DEBUG_REFUSE_BLOCK_LAUNCH, TF_DEBUG_EXCHANGE_NUMBER = 0, 1
 
 
 def tf_debug_set(m, what, value):

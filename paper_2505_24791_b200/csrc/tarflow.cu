@@ -214,6 +214,7 @@ struct tf_model {
   int seqp_groups[2] = {0, 0};                 // groups of 16 / 32 samples that fit the GPU side by side (0: not eligible)
   uint32_t seqp_seq = 1;                       // sequence number of the next exchange
   unsigned long long *seqp_part = nullptr, *seqp_row = nullptr;
+  size_t seqp_part_words = 0, seqp_row_words = 0;
   CUtensorMap seqp_cache[2];                   // keys, values
   bool seq_use_persist = true;                 // TARFLOW_SEQ_PERSIST=0: the chain of kernels
   int seqp_turn = -1;                          // device whose SeqpTurn this model shares (-1: none)
@@ -1200,6 +1201,8 @@ static int seqp_setup(tf_model* m) {
   TF_TRY(make_map_bf16(&m->seqp_cache[1], m->vcache, cache_rows, seqp::HD, 32));
   TF_TRY(dev_alloc(m, &m->seqp_part, part));
   TF_TRY(dev_alloc(m, &m->seqp_row, row));
+  m->seqp_part_words = part;
+  m->seqp_row_words = row;
   CU_OK(cudaMemset(m->seqp_part, 0, part * sizeof(*m->seqp_part)));
   CU_OK(cudaMemset(m->seqp_row, 0, row * sizeof(*m->seqp_row)));
   for (BlockW& bw : m->blocks) {
@@ -1253,8 +1256,16 @@ static int run_sequential_persistent(tf_model* m, int g, int B, const int* label
   job.layer_rows = m->cfg.max_batch * m->cfg.n_heads * L;
   job.xpart = m->seqp_part; job.xrow = m->seqp_row;
   job.n_layers = nl; job.B = B; job.L = L; job.Dt = D; job.reversed = g & 1;
+  // Words are recognised by their sequence number alone.  Before the numbers would start over (34 680 a call at 256 tokens and
+  // eight blocks of eight layers) what is left of them in the buffers is cleared, rows that few batches reach included.
+  const uint32_t numbers = (uint32_t)((2 * nl + 1) * n_steps + 1);
+  if (UINT32_MAX - m->seqp_seq < numbers) {
+    CU_OK(cudaMemsetAsync(m->seqp_part, 0, m->seqp_part_words * sizeof(*m->seqp_part), m->stream));
+    CU_OK(cudaMemsetAsync(m->seqp_row, 0, m->seqp_row_words * sizeof(*m->seqp_row), m->stream));
+    m->seqp_seq = 1;
+  }
   job.seq0 = m->seqp_seq;
-  m->seqp_seq += (uint32_t)((2 * nl + 1) * n_steps + 1);
+  m->seqp_seq += numbers;
   job.prefetch_w = weights > kL2Half;
   job.scale_log2e = 1.4426950408889634f / sqrtf((float)m->hd);
   job.err = m->err;
@@ -2621,6 +2632,10 @@ int tf_debug_set(tf_model* m, int32_t what, int64_t value) {
   if (!m) return fail(TF_EINVAL, "model is NULL");
   switch (what) {
     case TF_DEBUG_REFUSE_BLOCK_LAUNCH: m->seqp_debug_refuse = value != 0; return TF_OK;
+    case TF_DEBUG_EXCHANGE_NUMBER:
+      if (value < (int64_t)m->seqp_seq || value > (int64_t)UINT32_MAX) return fail(TF_EINVAL, "sequence numbers only grow, up to 2^32 - 1");
+      m->seqp_seq = (uint32_t)value;
+      return TF_OK;
   }
   return fail(TF_EINVAL, "unknown debug setting %d", what);
 }

@@ -102,3 +102,24 @@ def test_bf16_blocks_of_two_models_on_two_streams():
         assert not failed, failed
         for name in ("a", "b"):
             assert len(got[name]) == 8 and all(np.array_equal(x, want) for x in got[name])
+
+
+@pytest.mark.parametrize("before_the_end", [1, 0, -1])
+def test_bf16_block_when_the_exchange_numbers_start_over(before_the_end):
+    """A batch of 40 leaves words in rows that a batch of 1 does not touch.  Started over at the end of the 32-bit range, the
+    numbers of the batch of 1 end where those words' numbers begin: the second batch of 40 must not take them for its own."""
+    cfg = synth.config("cfg2", H=12, W=12, n_blocks=1, n_layers=2, width=128, n_heads=2)
+    numbers = (2 * cfg["n_layers"] + 1) * (synth.seq_len(cfg) - 1) + 1   # of one block
+    z = synth.make_latents(cfg, 11, B=40)
+    with Model(cfg, max_batch=40) as m:
+        want = m.inverse_sequential(z, None)
+        alone = m.inverse_sequential(z[:1], None)
+        last = 2 ** 32 - 1
+        # the whole block still fits, one number is missing, or nearly all of them are
+        start = {1: last - numbers, 0: last - numbers + 1, -1: last - 1}[before_the_end]
+        binding.tf_debug_set(m.m, binding.TF_DEBUG_EXCHANGE_NUMBER, start)
+        assert np.array_equal(m.inverse_sequential(z[:1], None), alone)
+        for _ in range(2):
+            assert np.array_equal(m.inverse_sequential(z, None), want)
+        with pytest.raises(binding.TarflowError):
+            binding.tf_debug_set(m.m, binding.TF_DEBUG_EXCHANGE_NUMBER, 1)
