@@ -75,8 +75,8 @@ struct Cfg {
   static constexpr int GW = QN * RPC / 32;         // warps of group 0: they hold the residual stream
   static constexpr int SPR = QN > 32 ? QN / 32 : 1, NE = CS * SPR, CE = CW / SPR;  // statistics of a row: NE entries of CE columns
   static constexpr int MT = N1 > 2 ? N1 / 2 : 1;   // 128-row output tiles of a CTA
-  // at most 10 slots: the cache rows of a step are then requested after the first MLP product of the layer's last step, by
-  // when that step's row is in memory (with one layer there are 12 weight units in between)
+  // at most 10 slots: the cache rows of a step are then requested when the previous layer's first MLP product has freed a slot,
+  // and the wait for that layer's new rows (B_ROWS) costs nothing
   static constexpr int NSLOT_MAX = (RT == 16 ? 163840 : 131072) / UNIT, NSLOT = NSLOT_MAX < 10 ? NSLOT_MAX : 10;
   // cache rows of one sample travel in units of KPU keys, KVS slots each (their keys, then their values)
   static constexpr int KVS = N1 == 1 ? 2 : 1, KPU = KVS * UNIT / 256, WPU = KPU / 16;
@@ -93,7 +93,7 @@ struct Cfg {
   static constexpr int STAT = TOK + RPC * MAXDT * 4;
   static constexpr int BIAS = STAT + RPC * NE * 8;
   static constexpr int BARS = BIAS + 192 * 4;
-  static constexpr int NBARS = 3 * NSLOT + 10;
+  static constexpr int NBARS = 3 * NSLOT + 11;
   static constexpr int TOTAL = BARS + NBARS * 8 + 32 + 1024;
   static constexpr uint32_t TMEM = RT == 16 ? 64 : 128;
   static_assert(sizeof(Layer) % sizeof(CUtensorMap) == 0, "tables of layers are stepped in tensor maps");
@@ -213,9 +213,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 }
 
 // The ring's filling side (one thread): requests one unit after the other in the order of use, each when its slot's last contents
-// have been used: weights by the products that read them, cache rows by the WPU warps that share a unit's tiles.
+// have been used: weights by the products that read them, cache rows by the WPU warps that share a unit's tiles.  Before a layer's
+// cache rows it waits on rows_bar for the new rows of the layer walked before it (and so of all earlier ones, this layer's in the
+// step before among them): their writers have fenced the async proxy, and the arrival orders the bulk copies after those stores.
 template <int D, int RT>
-__device__ __forceinline__ void feed(const Job& job, uint32_t ring, uint32_t bars, int r, int c, bool prefetch_w, int mine, int cache_row0) {
+__device__ __forceinline__ void feed(const Job& job, uint32_t ring, uint32_t bars, uint32_t rows_bar, int r, int c, bool prefetch_w, int mine, int cache_row0) {
   using C = Cfg<D, RT>;
   constexpr int N1 = C::N1, CW = C::CW;
   const int n_steps = job.L - 1;
@@ -247,7 +249,9 @@ __device__ __forceinline__ void feed(const Job& job, uint32_t ring, uint32_t bar
       const bool more = prefetch_w && (nx > 0 || t + 1 < n_steps);
 #pragma unroll 1
       for (int u = 0; u < 12; ++u) {
-        if (u == 3) {
+        if (u == 3 && mine > 0) {
+          const int before = t * job.n_layers + layer - 1;  // every phase is waited for, in order
+          if (before >= 0 && !wait_idle(rows_bar, (uint32_t)before & 1u, job.err, TFERR_WAIT_FULL)) return;
 #pragma unroll 1
           for (int p = 0; p < mine; ++p)
 #pragma unroll 1
@@ -326,7 +330,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
   const int L = job.L, Dt = job.Dt, n_steps = L - 1, nl = job.n_layers;
   int* err = job.err;
   auto bar = [&](int i) { return bars + 8u * (3 * C::NSLOT + i); };
-  enum { B_IN0, B_IN1, B_RECV0, B_RECV1, B_ALL0, B_ALL1, B_OUT0, B_OUT1, B_STAT, B_HEAD };  // 0: attention half, 1: MLP half
+  enum { B_IN0, B_IN1, B_RECV0, B_RECV1, B_ALL0, B_ALL1, B_OUT0, B_OUT1, B_STAT, B_HEAD, B_ROWS };  // 0: attention half, 1: MLP half
   uint8_t* tail_mem = smem + C::BARS + C::NBARS * 8;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail_mem);
   volatile int* s_bad = reinterpret_cast<volatile int*>(tail_mem + 4);
@@ -353,7 +357,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
 
   if (warp == NWARPS) {
     // ==================================================================== weights
-    if (lane == 0) feed<D, RT>(job, sb + C::RING, bars, r, c, job.prefetch_w && group == 0, mine, rows_of(0));
+    if (lane == 0) feed<D, RT>(job, sb + C::RING, bars, bar(B_ROWS), r, c, job.prefetch_w && group == 0, mine, rows_of(0));
   } else {
     constexpr uint32_t idesc = make_idesc(RT);
     // attention: a sample's keys are cut into tiles of 16, dealt out to eight sets whatever the batch; a set belongs to a warp,
@@ -826,7 +830,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
                           peer_addr(bar(B_ALL0), k));
               __syncwarp();
             }
-            fence_proxy_async_global();  // the new cache rows: the next step's bulk copies, long after the barriers below, read them
+            fence_proxy_async_global();  // the new cache rows: bulk copies read them from the next step on
           }
         } else {
           // ---------------------------------------------------------------- bias + GELU
@@ -893,6 +897,8 @@ seq_block_kernel(const __grid_constant__ Job job) {
         }
         advance(mlp ? 4 : 1);
         cbar();
+        if (tid == 0 && !mlp && mine > 0) mbar_arrive(bar(B_ROWS));  // every thread has fenced its new cache rows
+        __syncwarp();
         tcgen05_fence_after();
         if ((warp & 3) * 32 < CW) {  // accumulator lane = column, column = sample; warps 4-7: the second output tile or half of the samples
           constexpr int NB = C::MT == 2 ? RT : RT / 2;

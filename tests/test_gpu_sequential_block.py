@@ -104,6 +104,19 @@ def test_bf16_blocks_of_two_models_on_two_streams():
             assert len(got[name]) == 8 and all(np.array_equal(x, want) for x in got[name])
 
 
+@pytest.mark.parametrize("width,batch", [(128, 9), (512, 5), (1024, 6)])
+def test_bf16_block_of_one_layer_reads_the_rows_it_has_just_written(width, batch):
+    """With one layer a step's new keys and values are read by bulk copies of the very next layer walked; 150 tokens fill several
+    units of the ring."""
+    cfg = synth.config("cfg2", H=30, W=20, n_blocks=1, n_layers=1, width=width, n_heads=width // 64)
+    z = synth.make_latents(cfg, 12, B=batch)
+    with Model(cfg, max_batch=batch) as m:
+        x = m.inverse_sequential(z, None)
+        xo = O.model_inverse_sequential(m.blocks, z, None, cfg)
+        assert rel_l2(x, xo) <= REL_L2 and np.abs(x - xo).max() <= MAX_ABS
+        assert all(np.array_equal(m.inverse_sequential(z, None), x) for _ in range(5))
+
+
 @pytest.mark.parametrize("before_the_end", [1, 0, -1])
 def test_bf16_block_when_the_exchange_numbers_start_over(before_the_end):
     """A batch of 40 leaves words in rows that a batch of 1 does not touch.  Started over at the end of the 32-bit range, the
