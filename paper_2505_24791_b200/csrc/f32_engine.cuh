@@ -461,7 +461,7 @@ seq_cluster_kernel(const __grid_constant__ SeqPlan P, const float* __restrict__ 
     if (threadIdx.x == 0) tc::mbar_arrive_expect_tx(tc::smem_u32(bar), (uint32_t)bytes);
   };
   auto arrived = [&](uint64_t* bar, uint32_t parity) {
-    if (tc::mbar_wait(tc::smem_u32(bar), parity, err, TFERR_WAIT_FULL)) return true;
+    if (tc::mbar_wait<true>(tc::smem_u32(bar), parity, err, TFERR_WAIT_FULL)) return true;
     s_failed = 1;
     return false;
   };

@@ -48,24 +48,37 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// CLUSTER: the phase is completed by other CTAs of the cluster (their stores into this CTA's shared memory, their arrivals), so
+// that the wait has to acquire at cluster scope what they released; otherwise everything comes from this CTA and its own copies.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
+  if constexpr (CLUSTER)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 // Bounded wait.  Returns false (after recording `code`) when `limit_ns` of wall time pass or another role
 // already reported a failure.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, int* err, int code, unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
   unsigned long long t0 = globaltimer_ns();
   for (uint32_t spin = 1;; ++spin) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
     if ((spin & 255u) == 0) {
       if (*reinterpret_cast<volatile int*>(err) != 0) return false;
       if (globaltimer_ns() - t0 > limit_ns) {
@@ -75,8 +88,9 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, i
     }
   }
 }
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err, int code) {
-  return mbar_wait_limit(bar, parity, err, code, WAIT_LIMIT_NS);
+  return mbar_wait_limit<CLUSTER>(bar, parity, err, code, WAIT_LIMIT_NS);
 }
 
 // Self-test of the bounded wait: one thread waits on an mbarrier that nothing ever arrives on.  The wait runs out

@@ -43,11 +43,14 @@ constexpr int NTHREADS = 256, NWARPS = 8, HD = 64, UNITS = 256;  // compute thre
 // what a layer needs, in device memory; tensor maps have boxes of 64 rows x 64 k
 struct __align__(128) Layer {
   CUtensorMap qkv, wo, w1, w2;
-  const float *ln1_g, *ln1_b, *b_qkv, *b_o, *ln2_g, *ln2_b, *b_1, *b_2;
 };
+// A layer's vectors, one after the other, in units of the width.  They are addressed by arithmetic: the waits at cluster scope
+// leave nothing in L1, so a table of pointers would cost a second trip to L2 before each of them.
+enum Vec { V_LN1G = 0, V_LN1B = 1, V_BQKV = 2, V_BO = 5, V_LN2G = 6, V_LN2B = 7, V_B1 = 8, V_B2 = 12, V_COUNT = 13 };
 struct Job {
   CUtensorMap kmap, vmap;           // the caches as rows of 64, in boxes of 32 rows
   const Layer* layers;
+  const float* vecs;                // [n_layers][V_COUNT][width]
   const float *lnf_g, *lnf_b, *w_in_t, *b_in, *pos, *cls, *b_out, *v;
   const bf16* w_out;
   float* u;
@@ -134,9 +137,11 @@ __device__ __forceinline__ bool elect_one() {
 }
 // Bounded wait; the slow path is a call, because a layer's code is run through once and jumps over inlined slow paths miss in the
 // instruction cache (about 85 cycles each).
-__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int* err, int code) { return mbar_wait(bar, parity, err, code); }
+template <bool CLUSTER>
+__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int* err, int code) { return mbar_wait<CLUSTER>(bar, parity, err, code); }
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, int* err, int code) {
-  return mbar_try_wait(bar, parity) || wait_slow(bar, parity, err, code);
+  return mbar_try_wait<CLUSTER>(bar, parity) || wait_slow<CLUSTER>(bar, parity, err, code);
 }
 // the same for a warp that waits while others work: it sleeps between polls
 __device__ __noinline__ bool wait_idle(uint32_t bar, uint32_t parity, int* err, int code) {
@@ -390,6 +395,10 @@ seq_block_kernel(const __grid_constant__ Job job) {
       if (!wait_bar(bar(b), parity, err, code)) alive = false;
       __syncwarp();
     };
+    auto await_peers = [&](int b, uint32_t parity) {
+      if (!wait_bar<true>(bar(b), parity, err, TFERR_WAIT_FULL)) alive = false;
+      __syncwarp();
+    };
     // unit u of the phase has arrived: its address (warp 0); the products of unit u have been issued; next phase
     auto take = [&](int u) {
       const int s = slot + u, wrap = s >= C::NSLOT;
@@ -412,7 +421,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
     };
     // one warp polls, everybody else waits at the compute warps' barrier
     auto meet = [&](int b, uint32_t parity) {
-      if (warp == 0) await(b, parity, TFERR_WAIT_FULL);
+      if (warp == 0) await_peers(b, parity);
       cbar();
     };
     auto ld4 = [&](const float* p) { return __ldg(reinterpret_cast<const float4*>(p + col)); };
@@ -434,7 +443,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
       if (__shfl_sync(0xffffffffu, *s_bad, 0) != 0) break;
 #pragma unroll 1
       for (int half = 0; half <= 2 * nl; ++half) {
-        const Layer* ly = job.layers + (half >> 1);
+        const float* vec = job.vecs + (size_t)(half >> 1) * (V_COUNT * D);
         const int mlp = half & 1;                                   // which half of the layer follows
         const uint32_t lp = (uint32_t)(t * nl + (half >> 1)) & 1u;  // parity of its barriers
         // ================================================================== residual rows of this cluster
@@ -443,9 +452,9 @@ seq_block_kernel(const __grid_constant__ Job job) {
 #pragma unroll
           for (int i = 0; i < NA; ++i) sum[i] = zero4;
           if (holder && my_row) {
-            gg = ld4(half == 2 * nl ? job.lnf_g : mlp ? ly->ln2_g : ly->ln1_g);
-            bb = ld4(half == 2 * nl ? job.lnf_b : mlp ? ly->ln2_b : ly->ln1_b);
-            add = ld4(half == 0 ? job.b_in : mlp ? ly->b_o : ly[-1].b_2);
+            gg = ld4(half == 2 * nl ? job.lnf_g : vec + (mlp ? V_LN2G : V_LN1G) * D);
+            bb = ld4(half == 2 * nl ? job.lnf_b : vec + (mlp ? V_LN2B : V_LN1B) * D);
+            add = ld4(half == 0 ? job.b_in : mlp ? vec + V_BO * D : vec - (V_COUNT - V_B2) * D);
           }
           if (half == 0) {  // embedding of token t
             if (my_row) {
@@ -524,7 +533,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
               st_async2(peer_addr(sb + C::STAT + (lrow * NE + r * C::SPR + (QN > 32 ? q >> 5 : 0)) * 8, ql), __float_as_uint(wmean),
                         __float_as_uint(m2), peer_addr(bar(B_STAT), ql));
             __syncwarp();
-            await(B_STAT, stat_parity, TFERR_WAIT_FULL);
+            await_peers(B_STAT, stat_parity);
             const float2* st = reinterpret_cast<const float2*>(smem + C::STAT) + lrow * NE;
             float mean = 0.f;
 #pragma unroll
@@ -570,7 +579,9 @@ seq_block_kernel(const __grid_constant__ Job job) {
           const int per = (Dt + 31) / 32;
           if (tid < own * per) prefetch_line(job.v + token_at(tid / per, t + 1) + (tid % per) * 32);
         }
-        if (!mlp && tid < 192) s_bias[tid] = __ldg(ly->b_qkv + (tid >> 6) * D + c * HD + (tid & 63));
+        // stored below, once the rows are here: the waits at cluster scope leave nothing in L1, so this is a trip to L2
+        float bias_qkv = 0.f;
+        if (!mlp && tid < 192) bias_qkv = __ldg(vec + V_BQKV * D + (tid >> 6) * D + c * HD + (tid & 63));
         {  // rows of the projection's input (this rank's columns) into swizzled [RT][64] operand tiles
           constexpr int IT = RT * QN / NTHREADS;
           unsigned long long w[IT][2];
@@ -599,6 +610,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
               *reinterpret_cast<uint2*>(smem + C::ACT + (q >> 4) * (RT * 128) + swz128(row, (q & 15) >> 1) + (q & 1) * 8) =
                   make_uint2((uint32_t)w[k][0], (uint32_t)w[k][1]);
           }
+          if (!mlp && tid < 192) s_bias[tid] = bias_qkv;
           fence_proxy_async_smem();
           __syncwarp();
         }
@@ -847,8 +859,8 @@ seq_block_kernel(const __grid_constant__ Job job) {
             }
             tcgen05_fence_before();
           }
-          const float4 bias0 = __ldg(reinterpret_cast<const float4*>(ly->b_1 + c * UNITS + r * UPC + u8));
-          const float4 bias1 = __ldg(reinterpret_cast<const float4*>(ly->b_1 + c * UNITS + r * UPC + u8 + 4));
+          const float4 bias0 = __ldg(reinterpret_cast<const float4*>(vec + V_B1 * D + c * UNITS + r * UPC + u8));
+          const float4 bias1 = __ldg(reinterpret_cast<const float4*>(vec + V_B1 * D + c * UNITS + r * UPC + u8 + 4));
           fence_proxy_async_smem();
           cbar();
           if (tid < CS)
@@ -878,7 +890,7 @@ seq_block_kernel(const __grid_constant__ Job job) {
         // ------------------------------------------------------------------ output projection and this cluster's partial rows
         __syncwarp();
         if (warp == 0) {
-          await(B_ALL0 + mlp, lp, TFERR_WAIT_FULL);
+          await_peers(B_ALL0 + mlp, lp);
           fence_proxy_async_smem();  // the tiles were written through the generic proxy
 #pragma unroll 1
           for (int u = 0; u < (mlp ? 4 : 1); ++u) {

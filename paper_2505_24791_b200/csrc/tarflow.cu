@@ -211,6 +211,7 @@ struct tf_model {
   bool seq_fin = false;
   // bf16 engine: blocks decoded by one cooperative launch (seq_persist.cuh)
   std::vector<seqp::Layer*> seqp_layers;       // per block, device memory
+  std::vector<float*> seqp_vecs;
   int seqp_groups[2] = {0, 0};                 // groups of 16 / 32 samples that fit the GPU side by side (0: not eligible)
   uint32_t seqp_seq = 1;                       // sequence number of the next exchange
   unsigned long long *seqp_part = nullptr, *seqp_row = nullptr;
@@ -1207,14 +1208,20 @@ static int seqp_setup(tf_model* m) {
   CU_OK(cudaMemset(m->seqp_row, 0, row * sizeof(*m->seqp_row)));
   for (BlockW& bw : m->blocks) {
     std::vector<seqp::Layer> table;
+    float* vecs = nullptr;
+    TF_TRY(dev_alloc(m, &vecs, (size_t)seqp::V_COUNT * d * bw.layers.size()));
+    m->seqp_vecs.push_back(vecs);
     for (LayerW& lw : bw.layers) {
       seqp::Layer ly;
       TF_TRY(make_map_bf16(&ly.qkv, lw.w_qkv.w, lw.w_qkv.N, lw.w_qkv.K, 64));
       TF_TRY(make_map_bf16(&ly.wo, lw.w_o.w, lw.w_o.N, lw.w_o.K, 64));
       TF_TRY(make_map_bf16(&ly.w1, lw.w_1.w, lw.w_1.N, lw.w_1.K, 64));
       TF_TRY(make_map_bf16(&ly.w2, lw.w_2.w, lw.w_2.N, lw.w_2.K, 64));
-      ly.ln1_g = lw.ln1_g; ly.ln1_b = lw.ln1_b; ly.b_qkv = lw.b_qkv; ly.b_o = lw.b_o;
-      ly.ln2_g = lw.ln2_g; ly.ln2_b = lw.ln2_b; ly.b_1 = lw.b_1; ly.b_2 = lw.b_2;
+      const float* parts[] = {lw.ln1_g, lw.ln1_b, lw.b_qkv, lw.b_o, lw.ln2_g, lw.ln2_b, lw.b_1, lw.b_2};
+      const int starts[] = {seqp::V_LN1G, seqp::V_LN1B, seqp::V_BQKV, seqp::V_BO, seqp::V_LN2G, seqp::V_LN2B, seqp::V_B1, seqp::V_B2, seqp::V_COUNT};
+      for (int i = 0; i < 8; ++i)
+        CU_OK(cudaMemcpy(vecs + (size_t)starts[i] * d, parts[i], (size_t)(starts[i + 1] - starts[i]) * d * sizeof(float), cudaMemcpyDeviceToDevice));
+      vecs += (size_t)seqp::V_COUNT * d;
       table.push_back(ly);
     }
     seqp::Layer* dev = nullptr;
@@ -1248,6 +1255,7 @@ static int run_sequential_persistent(tf_model* m, int g, int B, const int* label
   seqp::Job job = {};
   job.rows = (B + want - 1) / want;
   job.layers = m->seqp_layers[g];
+  job.vecs = m->seqp_vecs[g];
   job.lnf_g = bw.lnf_g; job.lnf_b = bw.lnf_b; job.w_in_t = bw.w_in_t; job.b_in = bw.b_in; job.pos = bw.pos; job.cls = bw.cls;
   job.b_out = bw.b_out; job.w_out = reinterpret_cast<const bf16*>(bw.w_out.w);
   job.v = v; job.u = u; job.labels = labels;
