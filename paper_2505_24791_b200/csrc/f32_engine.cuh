@@ -536,6 +536,8 @@ seq_cluster_kernel(const __grid_constant__ SeqPlan P, const float* __restrict__ 
             } else if (j < t && (pr != pr0 || jb >= ng)) {
               kv = *reinterpret_cast<const float4*>(kcache + row0 + (size_t)j * hd);
               vv = *reinterpret_cast<const float4*>(vcache + row0 + (size_t)j * hd);
+            } else if (j > t) {  // masked: what is in the registers may be another sample's, and 0 x NaN is NaN
+              vv = make_float4(0.f, 0.f, 0.f, 0.f);
             }
             float x = fmaf(qv.x, kv.x, fmaf(qv.y, kv.y, fmaf(qv.z, kv.z, qv.w * kv.w)));
             for (int off = lpk >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);

@@ -136,3 +136,17 @@ def test_bf16_block_when_the_exchange_numbers_start_over(before_the_end):
             assert np.array_equal(m.inverse_sequential(z, None), want)
         with pytest.raises(binding.TarflowError):
             binding.tf_debug_set(m.m, binding.TF_DEBUG_EXCHANGE_NUMBER, 1)
+
+
+def test_fp32_sample_that_diverges_leaves_its_cluster_mates_alone():
+    """Four samples share a cluster here and a CTA has five heads, 20 (sample, head) pairs for 16 warps: a warp goes on to the
+    pair of another sample with the first one's rows still in its registers."""
+    cfg = synth.config("cfg1", H=16, W=12, n_blocks=1, n_layers=1, width=160, n_heads=40, mlp_ratio=1)
+    z = synth.make_latents(cfg, 13, B=80)
+    with Model(cfg, max_batch=80) as m:
+        want = m.inverse_sequential(z, None)
+        assert np.isfinite(want).all()
+        z[4] = 3e38
+        x = m.inverse_sequential(z, None)
+        others = np.arange(80) != 4
+        assert not np.isfinite(x[4]).all() and np.array_equal(x[others], want[others])
