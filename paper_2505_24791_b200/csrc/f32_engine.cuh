@@ -21,14 +21,17 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // ---------------------------------------------------------------------------------------------
 // C[M,N] = A[M,K] W[N,K]^T, K % 4 == 0.  BM x BN tile per CTA of (BM / TM) (BN / 4) KS threads: KS groups of threads share
 // a tile and take turns along K (their sums are added in group order at the end), a thread owns TM x 4 outputs and reads
-// both operands four k at a time.  32-wide k slabs arrive through a deep ring of cp.async stages (the first weight
+// both operands four k at a time.  KS is the same for every tile, so that an output's order of summation does not depend on
+// the number of rows (two groups for the widest tile: 4096 rows of width 128 forward 502 us instead of 512, 20 000 rows of an MLP
+// flow of width 512 1.60 ms instead of 1.55; 64 x 32 and 32 x 64 tiles with four: 549 us).  32-wide k slabs arrive through a deep ring of cp.async stages (the first weight
 // slabs are requested before the wait on the previous kernel), so that a short K is one memory latency, not one per slab.  Row n of W sits at slot (n % 4) (BN / 4) + n / 4 of a slab, so
 // that the column quads of a quarter warp lie in different banks.
 // Why: the 64 x 64 tile this replaces left 8 to 24 CTAs for 256 rows and two barriers per 16 k; 256 x 128 x 512 took
 // 48 us.
 // ---------------------------------------------------------------------------------------------
 constexpr int GK = 32, GPITCH = GK + 4;
-template <int BM, int BN, int TM, int KS>
+constexpr int KS = 4;
+template <int BM, int BN, int TM>
 struct GemmCfg {
   static constexpr int GSTAGES = BM + BN > 64 ? 4 : 8;
   static constexpr int GROUP = (BM / TM) * (BN / 4), THREADS = GROUP * KS;
@@ -38,10 +41,10 @@ struct GemmCfg {
   static_assert((KS - 1) * GROUP * TM * 4 <= GSTAGES * STAGE, "the groups' sums must fit the ring");
 };
 
-template <int BM, int BN, int TM, int KS, class Epi>
-__global__ void __launch_bounds__(GemmCfg<BM, BN, TM, KS>::THREADS)
+template <int BM, int BN, int TM, class Epi>
+__global__ void __launch_bounds__(GemmCfg<BM, BN, TM>::THREADS)
 gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, int M, int N, int K, Epi epi) {
-  using C = GemmCfg<BM, BN, TM, KS>;
+  using C = GemmCfg<BM, BN, TM>;
   constexpr int GSTAGES = C::GSTAGES;
   extern __shared__ __align__(16) float s_ring[];
   pdl_launch_dependents();
@@ -103,24 +106,22 @@ gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, int M, int
         }
     }
   }
-  if constexpr (KS > 1) {
-    cp_async_wait<0>();
-    __syncthreads();
-    if (grp > 0) {
+  cp_async_wait<0>();
+  __syncthreads();
+  if (grp > 0) {
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
-        *reinterpret_cast<float4*>(s_ring + (((grp - 1) * TM + i) * C::GROUP + gt) * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    }
-    __syncthreads();
-    if (grp > 0) return;
-#pragma unroll
-    for (int g = 1; g < KS; ++g)
-#pragma unroll
-      for (int i = 0; i < TM; ++i) {
-        const float4 o = *reinterpret_cast<const float4*>(s_ring + (((g - 1) * TM + i) * C::GROUP + gt) * 4);
-        acc[i][0] += o.x; acc[i][1] += o.y; acc[i][2] += o.z; acc[i][3] += o.w;
-      }
+    for (int i = 0; i < TM; ++i)
+      *reinterpret_cast<float4*>(s_ring + (((grp - 1) * TM + i) * C::GROUP + gt) * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
   }
+  __syncthreads();
+  if (grp > 0) return;
+#pragma unroll
+  for (int g = 1; g < KS; ++g)
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const float4 o = *reinterpret_cast<const float4*>(s_ring + (((g - 1) * TM + i) * C::GROUP + gt) * 4);
+      acc[i][0] += o.x; acc[i][1] += o.y; acc[i][2] += o.z; acc[i][3] += o.w;
+    }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int row = m0 + ty * TM + i, col0 = n0 + tx * 4;
@@ -255,6 +256,7 @@ attention_kernel(const float* __restrict__ qkv, float* __restrict__ out, int L, 
 // (No = 2 D rounded up to 4, Dp = D rounded up to 4; zero padded), which stays in global memory where it does not fit.
 // ---------------------------------------------------------------------------------------------
 constexpr int SC = 8, ST = 512, SW = ST / 32;  // CTAs per cluster, threads and warps per CTA
+constexpr int AU = 8;                          // parts into which the attention of a CTA's heads is cut for one sample, at least
 struct SeqPlan {
   int n_layers = 0, heads = 0, hd = 0, d = 0, D = 0, L = 0, owners = 0;  // owners = CTAs that hold heads
   int off[SC + 1] = {0}, nown[SC] = {0}, nu[SC] = {0};
@@ -278,7 +280,7 @@ struct SeqPlan {
       if (nu[r] > nx) nx = nu[r];
       if (nown[r] > no) no = nown[r];
     }
-    return recv_floats(S) + 2 * S * d + S * nq + S * no * hd + S * nx + S * pad4(D) + (S * no > SW ? S * no : SW) * (hd + 4) +
+    return recv_floats(S) + 2 * S * d + S * nq + S * no * hd + S * nx + S * pad4(D) + S * (no > AU ? no : AU) * (hd + 4) +
            2 * S * pad4(D) + 2 * d;
   }
 };
@@ -413,7 +415,7 @@ seq_cluster_kernel(const __grid_constant__ SeqPlan P, const float* __restrict__ 
   float* att = w; w += S * nown * hd;
   float* hid = w; w += S * nu;
   float* tok = w; w += S * Dp;
-  float* part = w; w += (S * nown > SW ? S * nown : SW) * (hd + 4);
+  float* part = w; w += S * (nown > AU ? nown : AU) * (hd + 4);
   float* vnext = w; w += 2 * S * Dp;
   float* pnext = w;
   const float* fixed = s_mem + P.n_layers * layer_floats;  // lnf_g lnf_b b_in
@@ -441,11 +443,12 @@ seq_cluster_kernel(const __grid_constant__ SeqPlan P, const float* __restrict__ 
     if (r == 0 && b0 + s < B) u[((size_t)(b0 + s) * L + tok_index(0, L, reversed)) * D + c] = x;
   }
   const float scale = 1.0f / sqrtf((float)hd);
-  // attention: a (sample, own head) pair has wpp warps, hd / 4 lanes share a key (a power of two)
+  // Attention: hd / 4 lanes share a key (a power of two); the keys of a (sample, own head) pair are dealt to wpp units of a
+  // warp's work, whatever S, so that a sample's sums do not depend on how many samples share the cluster (as many as S leaves
+  // warps for: 1-4 % shorter blocks; 16 units instead of 8: 5-15 % longer ones from two samples on).  Unit i of the S nown wpp units is part i % wpp of pair i / wpp, a warp takes every SW-th.
   const int lpk = hd >> 2, llog = 31 - __clz(lpk), klog = 5 - llog, kpw = 1 << klog;  // kpw keys per warp and round
-  const int pairs = S * nown, wpp = pairs >= SW || pairs == 0 ? 1 : SW / pairs, wpairs = SW / wpp;
-  const int pr0 = warp / wpp, sub = lane & (lpk - 1), wi = warp - pr0 * wpp, grp = wi * kpw + (lane >> llog), ng = wpp * kpw;
-  const FastDiv by_nown(nown), by_3hd(3 * hd), by_hd(hd);
+  const int pairs = S * nown, wpp = nown >= AU || nown == 0 ? 1 : AU / nown, ng = wpp * kpw, sub = lane & (lpk - 1);
+  const FastDiv by_nown(nown), by_3hd(3 * hd), by_hd(hd), by_wpp(wpp);
   const size_t layer_cache = (size_t)max_batch * P.heads * L * hd;
   auto cache_row = [&](int layer, int s, int hl) {
     return layer * layer_cache + ((size_t)(sample(s) * P.heads + r + SC * hl) * L) * hd;
@@ -497,8 +500,9 @@ seq_cluster_kernel(const __grid_constant__ SeqPlan P, const float* __restrict__ 
       const float *w_qkv = wl, *b_qkv = w_qkv + d * nq, *w_o = b_qkv + nq, *w_1 = w_o + nown * hd * d, *b_1 = w_1 + d * nu,
                   *w_2 = b_1 + nu, *vec = w_2 + nu * d;
       if (nown > 0) {
-        // this lane's first key and value row, unless it is the new token's
+        // this lane's first key and value row of the warp's first unit, unless it is the new token's
         float4 k0 = make_float4(0.f, 0.f, 0.f, 0.f), v0 = k0;
+        const int pr0 = by_wpp(warp), grp = (warp - pr0 * wpp) * kpw + (lane >> llog);
         if (pr0 < pairs && grp < t) {
           const int s = by_nown(pr0);
           const size_t at = cache_row(layer, s, pr0 - s * nown) + (size_t)grp * hd + 4 * sub;
@@ -519,49 +523,82 @@ seq_cluster_kernel(const __grid_constant__ SeqPlan P, const float* __restrict__ 
             }
         });
         __syncthreads();
-        // online softmax per warp over its keys, then the warps of a pair are merged
-        for (int pr = pr0; pr < pairs; pr += wpairs) {
-          const int s = by_nown(pr), hl = pr - s * nown;
-          const float* mine = qkv + s * nq + hl * 3 * hd + 4 * sub;
-          const size_t row0 = cache_row(layer, s, hl) + 4 * sub;
-          const float4 qv = *reinterpret_cast<const float4*>(mine);
-          float m = -INFINITY, l = 0.f;
-          float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int jb = wi * kpw; jb <= t; jb += ng) {
-            const int j = jb + (lane >> llog);
-            float4 kv = k0, vv = v0;
-            if (j == t) {
-              kv = *reinterpret_cast<const float4*>(mine + hd);
-              vv = *reinterpret_cast<const float4*>(mine + 2 * hd);
-            } else if (j < t && (pr != pr0 || jb >= ng)) {
-              kv = *reinterpret_cast<const float4*>(kcache + row0 + (size_t)j * hd);
-              vv = *reinterpret_cast<const float4*>(vcache + row0 + (size_t)j * hd);
-            } else if (j > t) {  // masked: what is in the registers may be another sample's, and 0 x NaN is NaN
-              vv = make_float4(0.f, 0.f, 0.f, 0.f);
+        // online softmax of every unit that has a key, two units of a warp at a time, then the units of a pair are merged
+        constexpr int G = S > 2 ? 2 : 1;
+        for (int unit0 = warp; unit0 < pairs * wpp; unit0 += G * SW) {
+          const float* mine[G];
+          size_t row0[G];
+          float4 qv[G], o[G];
+          float m[G], l[G];
+          int first[G], lead = t + 1;  // a unit's first key; the smaller of them
+#pragma unroll
+          for (int i = 0; i < G; ++i) {
+            const int unit = unit0 + i * SW, pr = by_wpp(unit < pairs * wpp ? unit : unit0), s = by_nown(pr), hl = pr - s * nown;
+            first[i] = unit < pairs * wpp ? (unit - pr * wpp) * kpw : t + 1;
+            lead = first[i] < lead ? first[i] : lead;
+            mine[i] = qkv + s * nq + hl * 3 * hd + 4 * sub;
+            row0[i] = cache_row(layer, s, hl) + 4 * sub;
+            qv[i] = *reinterpret_cast<const float4*>(mine[i]);
+            m[i] = -INFINITY;
+            l[i] = 0.f;
+            o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+          for (int r0 = 0; lead + r0 <= t; r0 += ng) {
+            float4 kv[G], vv[G];
+            float x[G], mx[G];
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              const int j = first[i] + r0 + (lane >> llog);
+              kv[i] = vv[i] = make_float4(0.f, 0.f, 0.f, 0.f);  // masked keys: what is in memory may be NaN, and so is 0 x NaN
+              if (j == t) {
+                kv[i] = *reinterpret_cast<const float4*>(mine[i] + hd);
+                vv[i] = *reinterpret_cast<const float4*>(mine[i] + 2 * hd);
+              } else if (j < t) {
+                if (i == 0 && unit0 == warp && r0 == 0) {
+                  kv[i] = k0;
+                  vv[i] = v0;
+                } else {
+                  kv[i] = *reinterpret_cast<const float4*>(kcache + row0[i] + (size_t)j * hd);
+                  vv[i] = *reinterpret_cast<const float4*>(vcache + row0[i] + (size_t)j * hd);
+                }
+              }
+              x[i] = fmaf(qv[i].x, kv[i].x, fmaf(qv[i].y, kv[i].y, fmaf(qv[i].z, kv[i].z, qv[i].w * kv[i].w)));
             }
-            float x = fmaf(qv.x, kv.x, fmaf(qv.y, kv.y, fmaf(qv.z, kv.z, qv.w * kv.w)));
-            for (int off = lpk >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-            x = j <= t ? x * scale : -INFINITY;
-            float mx = x;
-            for (int off = lpk; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            const float mn = fmaxf(m, mx);  // key jb is visible: finite
-            const float corr = expf(m - mn), p = expf(x - mn);
-            m = mn;
-            l = fmaf(l, corr, p);
-            o.x = fmaf(o.x, corr, p * vv.x); o.y = fmaf(o.y, corr, p * vv.y);
-            o.z = fmaf(o.z, corr, p * vv.z); o.w = fmaf(o.w, corr, p * vv.w);
+            for (int off = lpk >> 1; off > 0; off >>= 1)
+#pragma unroll
+              for (int i = 0; i < G; ++i) x[i] += __shfl_xor_sync(0xffffffffu, x[i], off);
+#pragma unroll
+            for (int i = 0; i < G; ++i) mx[i] = x[i] = first[i] + r0 + (lane >> llog) <= t ? x[i] * scale : -INFINITY;
+            for (int off = lpk; off < 32; off <<= 1)
+#pragma unroll
+              for (int i = 0; i < G; ++i) mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], off));
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              if (G > 1 && first[i] + r0 > t) continue;  // this unit has no more keys
+              const float mn = fmaxf(m[i], mx[i]);       // its first key is visible: finite
+              const float corr = expf(m[i] - mn), p = expf(x[i] - mn);
+              m[i] = mn;
+              l[i] = fmaf(l[i], corr, p);
+              o[i].x = fmaf(o[i].x, corr, p * vv[i].x); o[i].y = fmaf(o[i].y, corr, p * vv[i].y);
+              o[i].z = fmaf(o[i].z, corr, p * vv[i].z); o[i].w = fmaf(o[i].w, corr, p * vv[i].w);
+            }
           }
-          for (int off = lpk; off < 32; off <<= 1) {
-            l += __shfl_xor_sync(0xffffffffu, l, off);
-            o.x += __shfl_xor_sync(0xffffffffu, o.x, off); o.y += __shfl_xor_sync(0xffffffffu, o.y, off);
-            o.z += __shfl_xor_sync(0xffffffffu, o.z, off); o.w += __shfl_xor_sync(0xffffffffu, o.w, off);
+          for (int off = lpk; off < 32; off <<= 1)
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+              o[i].x += __shfl_xor_sync(0xffffffffu, o[i].x, off); o[i].y += __shfl_xor_sync(0xffffffffu, o[i].y, off);
+              o[i].z += __shfl_xor_sync(0xffffffffu, o[i].z, off); o[i].w += __shfl_xor_sync(0xffffffffu, o[i].w, off);
+            }
+#pragma unroll
+          for (int i = 0; i < G; ++i) {
+            float* pt = part + (unit0 + i * SW) * (hd + 4);
+            if (first[i] <= t && lane < lpk) *reinterpret_cast<float4*>(pt + 4 * lane) = o[i];
+            if (first[i] <= t && lane == 0) { pt[hd] = m[i]; pt[hd + 1] = l[i]; }
           }
-          float* pt = part + (pr * wpp + wi) * (hd + 4);
-          if (lane < lpk) *reinterpret_cast<float4*>(pt + 4 * lane) = o;
-          if (lane == 0) { pt[hd] = m; pt[hd + 1] = l; }
         }
         __syncthreads();
-        const int aw = (t + kpw) >> klog < wpp ? (t + kpw) >> klog : wpp;  // warps of a pair that saw a key
+        const int aw = (t + kpw) >> klog < wpp ? (t + kpw) >> klog : wpp;  // units of a pair that have a key
         for (int i = threadIdx.x; i < pairs * hd; i += ST) {
           const int pr = by_hd(i), c = i - pr * hd;
           const float* pt = part + pr * wpp * (hd + 4);

@@ -460,10 +460,10 @@ static int launch_gemm_tc2(tf_model* m, int cls, const CUtensorMap& ma, const CU
   return TF_OK;
 }
 
-template <int BM, int BN, int TM, int KS, class Epi>
+template <int BM, int BN, int TM, class Epi>
 static int launch_gemm_f32(tf_model* m, int cls, const float* A, const Matrix& W, int M, const Epi& epi) {
-  using C = f32::GemmCfg<BM, BN, TM, KS>;
-  auto kern = f32::gemm_kernel<BM, BN, TM, KS, Epi>;
+  using C = f32::GemmCfg<BM, BN, TM>;
+  auto kern = f32::gemm_kernel<BM, BN, TM, Epi>;
   static bool configured[kMaxDevices] = {false};  // per instantiation and device
   const int dev = current_device();
   if (dev < 0) return fail(TF_ECUDA, "no usable current device");
@@ -483,9 +483,9 @@ static int launch_gemm_simt(tf_model* m, int cls, const T* A, const Matrix& W, i
   if constexpr (sizeof(T) == 4) {
     if (W.K % 4 == 0) {
       auto tiles = [&](int bm, int bn) { return ((M + bm - 1) / bm) * ((W.N + bn - 1) / bn); };
-      if (tiles(64, 64) >= 2 * m->num_sms) return launch_gemm_f32<64, 64, 4, 2>(m, cls, A, W, M, epi);
-      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, 2, 4>(m, cls, A, W, M, epi);
-      return launch_gemm_f32<16, 32, 1, 4>(m, cls, A, W, M, epi);
+      if (tiles(64, 64) >= 2 * m->num_sms) return launch_gemm_f32<64, 64, 8>(m, cls, A, W, M, epi);
+      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, 2>(m, cls, A, W, M, epi);
+      return launch_gemm_f32<16, 32, 1>(m, cls, A, W, M, epi);
     }
   }
   dim3 grid((W.N + 63) / 64, (M + 63) / 64);

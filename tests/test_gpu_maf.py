@@ -190,3 +190,19 @@ def test_calls_of_changing_batch_on_one_handle_give_the_same_result():
             for B, (x0, ib0, its0, rc0) in first.items():
                 x, ib, its, rc = m.jacobi(z[:B], 1e-3, m.D + 1)
                 assert rc == rc0 == 0 and np.array_equal(x, x0) and np.array_equal(its, its0) and np.array_equal(ib, ib0), B
+
+
+def test_fp32_sample_does_not_depend_on_the_batch():
+    """A batch whose products take the widest tiles of the fp32 engine, and parts of it."""
+    cfg = synth.maf_config("maf_tiny")
+    B = 20000
+    with Maf(cfg, B) as m:
+        z = synth.make_maf_latents(cfg, 25, B=B)
+        x, _, its, rc = m.jacobi(z, 1e-6, m.D + 1)
+        zf, ld = m.forward(z)
+        assert rc == 0
+        for pick in (slice(7, 8), slice(100, 140), slice(0, 3000)):
+            xp, _, itp, _ = m.jacobi(z[pick], 1e-6, m.D + 1)
+            zp, lp = m.forward(z[pick])
+            assert np.array_equal(xp, x[pick]) and np.array_equal(itp, its[:, pick]), pick
+            assert np.array_equal(zp, zf[pick]) and np.array_equal(lp, ld[pick]), pick

@@ -150,3 +150,23 @@ def test_fp32_sample_that_diverges_leaves_its_cluster_mates_alone():
         x = m.inverse_sequential(z, None)
         others = np.arange(80) != 4
         assert not np.isfinite(x[4]).all() and np.array_equal(x[others], want[others])
+
+
+@pytest.mark.parametrize("over", [{}, dict(width=96, n_heads=3, n_blocks=1), dict(H=14, W=10, width=160, n_heads=40, mlp_ratio=1, n_layers=1)])
+def test_fp32_sample_does_not_depend_on_the_batch(over):
+    """Every direction of the fp32 engine, one sample alone, a few, and as part of a batch that fills clusters with two or four
+    samples and the products' widest tiles: the same bits."""
+    cfg = synth.config("cfg1", **over)
+    K, B = cfg["n_blocks"], 90
+    z = synth.make_latents(cfg, 14, B=B)
+    with Model(cfg, max_batch=B) as m:
+        calls = {"sequential": lambda x: (m.inverse_sequential(x, None),),
+                 "jacobi": lambda x: m.inverse(x, None, [1] * K, 1e-5, m.L + 1)[::2],
+                 "forward": lambda x: m.forward(x, None)}
+        for name, call in calls.items():
+            whole = call(z)
+            for pick in (slice(0, 1), slice(57, 60), slice(B - 30, B)):
+                part = call(z[pick])
+                assert np.array_equal(part[0], whole[0][pick]), (name, pick)
+                if name != "sequential":   # sweep counts [blocks, samples], log-determinants
+                    assert np.array_equal(part[1], whole[1][..., pick]), (name, pick)
