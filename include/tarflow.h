@@ -329,9 +329,11 @@ int tf_trace_read_l2(tf_model* m, int32_t block, int32_t B, float* l2_host, int3
 
 /*
  * tf_selftest_wait_timeout -- exercises the bounded-wait path without any fault: launches one CTA whose thread
- * waits, for at most limit_us microseconds (1 .. 1 000 000), on an mbarrier that nothing arrives on.  The wait runs
- * out, the kernel records its code in the model's error word and returns; the call then synchronises and returns
- * what any synchronising call would: TF_ETIMEOUT, once, with the word cleared.  The model remains usable.
+ * waits, for at most limit_us microseconds (1 .. 1 000 000), on an mbarrier that nothing arrives on; then one that polls
+ * a word nothing writes, then one that waits for an mbarrier between naps (the forms of wait of the one-launch block, with
+ * a limit of 1000 microseconds each).  Each wait runs out, the kernel records its code in the model's error word and
+ * returns; after each the call synchronises.  It returns what any synchronising call would, TF_ETIMEOUT, once, with the
+ * word cleared, and TF_ECUDA if one of the waits did not run out.  The model remains usable.
  */
 int tf_selftest_wait_timeout(tf_model* m, int32_t limit_us, void* cuda_stream);
 

@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(256) forward_affine_kernel(const float* __rest
 // maxdiff, ctrl[3] = number of active samples in the hp phase (the tail of idx); ctrl[CTRL_SWEEP] = sweeps finished in
 // this block, ctrl[CTRL_TAU] / ctrl[CTRL_SWITCH] = bits of tau and of the escalation threshold.
 // ------------------------------------------------------------------------------------------------
-constexpr int CTRL_WORDS = 16, CTRL_LABEL_FLAG = 5, CTRL_SWEEP = 8, CTRL_TAU = 9, CTRL_SWITCH = 10, CTRL_SEQ = 11;
+constexpr int CTRL_WORDS = 16, CTRL_LABEL_FLAG = 5, CTRL_SWEEP = 8, CTRL_TAU = 9, CTRL_SWITCH = 10, CTRL_SEQ = 11, CTRL_SELFTEST = 12;
 // Words of the pinned host array the last sweep-control kernel of a sweep fills (the device error word among them);
 // HOST_SEQ is stored after all others and counts the sweeps of this model, so the host can poll it.
 enum { HOST_ACTIVE, HOST_BAD, HOST_ERR, HOST_TOP, HOST_TWO_TERM, HOST_LABEL, HOST_SEQ, HOST_WORDS = 8 };

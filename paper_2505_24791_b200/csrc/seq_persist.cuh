@@ -144,6 +144,7 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, int* err
   return mbar_try_wait<CLUSTER>(bar, parity) || wait_slow<CLUSTER>(bar, parity, err, code);
 }
 // the same for a warp that waits while others work: it sleeps between polls
+template <unsigned long long LIMIT_NS = WAIT_LIMIT_NS>
 __device__ __noinline__ bool wait_idle(uint32_t bar, uint32_t parity, int* err, int code) {
   const unsigned long long t0 = globaltimer_ns();
   for (;;) {
@@ -155,7 +156,7 @@ __device__ __noinline__ bool wait_idle(uint32_t bar, uint32_t parity, int* err, 
     if (ok) return true;
     __nanosleep(100);
     const unsigned long long dt = globaltimer_ns() - t0;
-    if (dt > WAIT_LIMIT_NS) {
+    if (dt > LIMIT_NS) {
       atomicCAS(err, 0, code);
       return false;
     }
@@ -177,19 +178,38 @@ __device__ __forceinline__ void ll_load2(const unsigned long long* p, unsigned l
 __device__ __forceinline__ bool ll_here(unsigned long long a, unsigned long long b, uint32_t seq) {
   return (uint32_t)(a >> 32) == seq && (uint32_t)(b >> 32) == seq;
 }
-struct Spin {  // bound of a polling loop
+template <int CODE = TFERR_WAIT_FULL, unsigned long long LIMIT_NS = WAIT_LIMIT_NS>
+struct SpinOf {  // bound of a polling loop
   unsigned n = 0;
   unsigned long long t0 = 0;
   __device__ __noinline__ bool check(int* err) {
     if (*reinterpret_cast<volatile int*>(err) != 0) return false;
     const unsigned long long now = globaltimer_ns();
     if (n == 256u) t0 = now;
-    if (now - t0 <= WAIT_LIMIT_NS) return true;
-    atomicCAS(err, 0, TFERR_WAIT_FULL);
+    if (now - t0 <= LIMIT_NS) return true;
+    atomicCAS(err, 0, CODE);
     return false;
   }
   __device__ __forceinline__ bool more(int* err) { return (++n & 255u) != 0 || check(err); }
 };
+using Spin = SpinOf<>;
+
+// Self-test of the two other forms of bounded wait: one thread polls a word that nothing writes (which = 0) or waits between naps
+// for an mbarrier that nothing arrives on (1).  The wait runs out after a millisecond, is recorded, and the kernel returns normally.
+__global__ void wait_selftest_kernel(int* err, int which, const unsigned long long* word) {
+  constexpr unsigned long long kLimit = 1000000ull;
+  __shared__ __align__(8) unsigned long long idle;
+  if (threadIdx.x != 0) return;
+  if (which == 0) {
+    unsigned long long a, b;
+    SpinOf<TFERR_WAIT_SELFTEST, kLimit> spin;
+    do ll_load2(word, a, b);
+    while (!ll_here(a, b, 1u) && spin.more(err));
+  } else {
+    mbar_init(smem_u32(&idle), 1);
+    wait_idle<kLimit>(smem_u32(&idle), 0u, err, TFERR_WAIT_SELFTEST);
+  }
+}
 
 // eight accumulator columns of this thread's tensor-memory lane
 __device__ __forceinline__ void tmem_cols8(uint32_t taddr, float (&v)[8]) {

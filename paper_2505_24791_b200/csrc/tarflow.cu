@@ -2612,7 +2612,16 @@ int tf_selftest_wait_timeout(tf_model* m, int32_t limit_us, void* cuda_stream) {
   m->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   LAUNCH(m, KC_CTRL, tc::wait_selftest_kernel, 1, 32, 0, m->err, (unsigned long long)limit_us * 1000ull);
   TF_TRY(check_launch("wait_selftest_kernel"));
-  return sync_check(m);
+  int r = sync_check(m);
+  // the polled pair of words is a part of the control words that nothing writes: zero, where the number waited for is 1
+  for (int which = 0; which < 2 && r == TF_ETIMEOUT; ++which) {
+    CU_OK(cudaMemsetAsync(m->ctrl + CTRL_SELFTEST, 0, 4 * sizeof(int), m->stream));
+    LAUNCH(m, KC_CTRL, seqp::wait_selftest_kernel, 1, 32, 0, m->err, which,
+           reinterpret_cast<const unsigned long long*>(m->ctrl + CTRL_SELFTEST));
+    TF_TRY(check_launch("seqp::wait_selftest_kernel"));
+    r = sync_check(m);
+  }
+  return r == TF_OK ? fail(TF_ECUDA, "a wait that nothing satisfies did not run out") : r;
 }
 
 int64_t tf_debug_check_guards(tf_model* m, void* cuda_stream) {

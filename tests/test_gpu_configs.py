@@ -200,7 +200,7 @@ def test_bounded_wait_runs_out_is_reported_once_and_model_recovers(sweep_model):
     x_before, _, _, rc = m.inverse(z, lab, [1, 1], -1.0, 3)
     assert rc == 0
     with pytest.raises(binding.TarflowError) as e:
-        binding.tf_selftest_wait_timeout(m.m, 1000)
+        binding.tf_selftest_wait_timeout(m.m, 1000)   # an mbarrier, a polled word, an mbarrier between naps
     assert e.value.code == binding.TF_ETIMEOUT and "code 9" in str(e.value)
     x_after, _, _, rc = m.inverse(z, lab, [1, 1], -1.0, 3)
     assert rc == 0 and np.array_equal(x_before, x_after)
