@@ -21,7 +21,8 @@
 // Weights travel through a ring of TMA slots in the order in which they are used, ahead of the activations (a warp of its own
 // refills what has been used), and so do, between a layer's first and second projection, the keys and values of earlier
 // tokens: up to 160 KB per CTA are on their way, where loads of the attending warps kept 32 KB (width 1024, 64 samples:
-// 36 of a block's 85 ms went to attention).  Where a block's weights exceed L2 they are prefetched into L2 a layer ahead.
+// 36 of a block's 85 ms went to attention).  Where a block's weights exceed half of L2 they are prefetched into L2 a layer
+// ahead.
 // A step's head, update and embedding are done by the row's owner cluster on the CUDA cores.
 // Clusters are of 4 CTAs (2 at width 128): with most of an SM's shared memory per CTA, 33 of those fit the GPU side by side,
 // but only 15 of 8, and width 1024 has 16 heads.
