@@ -114,6 +114,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
   const int n_kv = ((q0 + BQ < L ? q0 + BQ : L) + BKV - 1) / BKV;  // key tiles that hold a visible key
 
   if (threadIdx.x == 0) {
+    prefetch_map(&map_qkv);
+    prefetch_map(&map_kv);
+    if constexpr (SPLIT) {
+      prefetch_map(&map_qkv_lo);
+      prefetch_map(&map_kv_lo);
+    }
     for (int i = 0; i < NUM_BARS; ++i) mbar_init(bar(i), (i == B_PREADY || i == B_SFREE) ? 4 : 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -127,12 +133,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (threadIdx.x == 64) {
+    prefetch_map(map_out);
+    if constexpr (SPLIT) prefetch_map(map_out_lo);
+  }
   pdl_wait();  // set-up above overlaps the previous kernel's tail; q, k, v and the error word are complete from here on
-  const bool dead = *reinterpret_cast<volatile int*>(err) != 0;
+  // After an earlier failure no product is issued; the producer's first loads need not wait for the error word.
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0 && !dead) {
+    if (lane == 0) {
       mbar_arrive_expect_tx(bar(0), C::Q_ALL);
       tma_load_3d(sQ, &map_qkv, head * HD, q0, slot, bar(0));
       if constexpr (SPLIT) tma_load_3d(sQ + Q_BYTES, &map_qkv_lo, head * HD, q0, slot, bar(0));
@@ -153,7 +163,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && !dead) {
+    if (lane == 0 && *reinterpret_cast<volatile int*>(err) == 0) {
       constexpr uint32_t idesc_s = make_idesc_attn(BQ, BKV, 0), idesc_o = make_idesc_attn(BQ, HD, 1);
       bool ok = mbar_wait(bar(0), 0u, err, TFERR_WAIT_FULL);
       const uint64_t qdesc = make_smem_desc(sQ);
@@ -223,7 +233,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
     // most kLazy / scale_log2e, so probabilities stay below 2^kLazy and the accumulator is rescaled only rarely
     constexpr float kLazy = 8.f;
     float m_run = -INFINITY, l_run = 0.f;
-    bool ok = !dead;
+    bool ok = *reinterpret_cast<volatile int*>(err) == 0;
     for (int j = 0; j < n_kv && ok; ++j) {
       if (!mbar_wait(bar(B_SFULL), (uint32_t)(j & 1), err, TFERR_WAIT_TMEM_FULL)) { ok = false; break; }
       tcgen05_fence_after();

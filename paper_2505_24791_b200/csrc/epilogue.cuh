@@ -18,6 +18,7 @@ namespace tc {  // defined in gemm_tc.cuh
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, uint32_t src);
 __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, int x, int y, uint32_t src);
 __device__ __forceinline__ void tma_store_commit();
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map);
 __device__ __forceinline__ void tma_store_wait_read();
 __device__ __forceinline__ void fence_proxy_async_smem();
 __device__ __forceinline__ uint32_t swz128(int r, int k);
@@ -442,6 +443,10 @@ struct EpiStoreTma {
   const float* bias;  // may be null
   const CUtensorMap* tmap;
   const CUtensorMap* tmap_lo;  // null = single term
+  __device__ __forceinline__ void prefetch() const {
+    tc::prefetch_map(tmap);
+    if (tmap_lo != nullptr) tc::prefetch_map(tmap_lo);
+  }
   static constexpr bool kRowwise = false;
   static constexpr bool kRowReduce = false;
   static constexpr int kTmaCols = 64;
@@ -507,6 +512,7 @@ struct EpiStoreTma {
 struct EpiResidTma {
   const float* bias;
   const CUtensorMap* tmap;  // fp32 [rows, d], box 32 columns x 32 rows, 128-byte swizzle
+  __device__ __forceinline__ void prefetch() const { tc::prefetch_map(tmap); }
   static constexpr bool kRowwise = false;
   static constexpr bool kRowReduce = false;
   static constexpr int kTmaCols = 32;
@@ -535,6 +541,7 @@ struct EpiResidTma {
 struct EpiStoreF32Tma {
   const float* bias;
   const CUtensorMap* tmap;
+  __device__ __forceinline__ void prefetch() const { tc::prefetch_map(tmap); }
   static constexpr bool kRowwise = false;
   static constexpr bool kRowReduce = false;
   static constexpr int kTmaCols = 32;

@@ -104,6 +104,10 @@ __global__ void wait_selftest_kernel(int* err, unsigned long long limit_ns) {
   }
 }
 
+// Brings a tensor map into the descriptor cache ahead of its first use (maps are written once, at load or by the host).
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -246,7 +250,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // ksplit > 1 (bulk-store epilogues only): every output tile is computed ksplit times, each over its own range of
   // k slabs, and slice s stores its partial tile part_rows * s rows further down; the consumer adds the slices in
   // index order.  Tile index = (m tile, n tile, slice) with the slice fastest.
-  const int num_tiles_all = tiles_m * tiles_n * ksplit;
+  const int num_tiles = tiles_m * tiles_n * ksplit;
   // split != 0: A is an error-compensated pair (hi + lo); the K loop runs over [A_hi | A_lo] against
   // [W | W], i.e. both products accumulate into the same TMEM tile.
   const int kb_per_pass = (K + BK - 1) / BK;
@@ -272,12 +276,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   }
   tcgen05_fence_before();
   __syncthreads();
+    prefetch_map(&map_a);
+    prefetch_map(&map_w);
+    if (split) prefetch_map(&map_a_lo);
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // everything above (barriers, tensor memory) overlaps the previous kernel's tail; its activations and the
-  // error word are complete from here on.  After an earlier failure the CTA walks an empty tile list.
+  if constexpr (Epi::kTmaCols > 0) {
+    if (threadIdx.x == 64) epi.prefetch();
+  }
+  // everything above (barriers, tensor memory, tensor maps) overlaps the previous kernel's tail; its activations and the
+  // error word are complete from here on.  After an earlier failure no product is issued.  The producer does not wait for the
+  // error word (a trip to L2 before the first load): its waits notice it, and the teardown lets its copies land.
   pdl_wait();
-  const int num_tiles = *reinterpret_cast<volatile int*>(err) != 0 ? 0 : num_tiles_all;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -307,7 +317,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       constexpr uint32_t idesc = make_idesc(BN);
       int stage = 0;
       uint32_t phase = 0;
-      bool ok = true;
+      bool ok = *reinterpret_cast<volatile int*>(err) == 0;
       int it = 0;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++it) {
         const int acc = it & 1;
@@ -338,7 +348,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int quad = warp & 3;  // TMEM lane quadrant this warp may read
     const int cgroup = (warp - 2) >> 2;  // which of the NUM_EPI_WARPS/4 column groups of a quadrant
     float* stage_out = reinterpret_cast<float*>(smem + SL::STAGE_OUT_OFFSET) + (warp - 2) * (32 * 33);
-    bool ok = true;
+    bool ok = *reinterpret_cast<volatile int*>(err) == 0;
     int it = 0;
     if constexpr (Epi::kTmaCols > 0) {
       // Bulk-store epilogue: each warp owns NCH adjacent 32-column chunks of its 32 rows; values leave the

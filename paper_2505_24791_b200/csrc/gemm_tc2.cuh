@@ -131,6 +131,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   }
   if (warp == 1) {  // pair-wide allocation: the same warp in both CTAs, same destination
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
+    prefetch_map(&map_a);
+    prefetch_map(&map_w);
+    if (split) prefetch_map(&map_a_lo);
                  "r"(TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -140,15 +143,16 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   cluster_sync_all();  // the peer's barriers exist before anything signals them
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // everything above (barriers, tensor memory, cluster handshake) overlaps the previous kernel's tail; its
+  if (threadIdx.x == 64) epi.prefetch();
+  // everything above (barriers, tensor memory, cluster handshake, tensor maps) overlaps the previous kernel's tail; its
   // activations and the error word are complete from here on
   pdl_wait();
-  // an earlier kernel failed: both CTAs skip the work (the leader's view decides, so the pair agrees)
-  const bool dead = *reinterpret_cast<volatile int*>(err) != 0;
+  // An earlier kernel failed: no product is issued (the leader's view decides, so the pair agrees).  The producers do not wait
+  // for the error word (a trip to L2 before the first load): their waits notice it, and the teardown lets their copies land.
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
-    if (lane == 0 && !dead) {
+    if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -171,7 +175,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (lane == 0 && rank == 0 && !dead) {
+    if (lane == 0 && rank == 0 && *reinterpret_cast<volatile int*>(err) == 0) {
       constexpr uint32_t idesc = make_idesc_pair(2 * BM, BN2);
       int stage = 0;
       uint32_t phase = 0;
@@ -213,7 +217,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     uint8_t* box = smem + SL::STAGE_OUT_OFFSET + (warp - 2) * 4096;
     const uint32_t box_addr = smem_u32(box);
     float* tile_bias = reinterpret_cast<float*>(smem + SL::TILE_BIAS_OFFSET);
-    bool ok = !dead;
+    bool ok = *reinterpret_cast<volatile int*>(err) == 0;
     int it = 0;
     // this thread's bias of the next tile is fetched one tile ahead, so its latency is off the epilogue's path
     float next_bias = 0.f;
