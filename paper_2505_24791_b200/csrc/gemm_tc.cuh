@@ -209,6 +209,19 @@ __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, float (&v)[32
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Weights with a block structure (masked layers whose units are sorted by degree): `bounds[j]` is the range of k slabs outside
+// which columns 128 j .. 128 j + 127 have no weight; a tile's loop runs over the union of its groups.  null: all slabs.
+struct SlabRange { int begin, end; };
+__device__ __forceinline__ SlabRange slab_range(const int2* bounds, int n0, int bn, int N, int slabs) {
+  if (bounds == nullptr) return {0, slabs};
+  int2 b = __ldg(bounds + n0 / 128);
+  if (bn > 128 && n0 + 128 < N) {
+    const int2 b2 = __ldg(bounds + n0 / 128 + 1);
+    b = make_int2(min(b.x, b2.x), max(b.y, b2.y));
+  }
+  return {b.x, b.y};
+}
+
 template <int BN, int STAGES>
 struct SmemLayout {
   static constexpr int A_BYTES = BM * BK * 2;
@@ -229,7 +242,7 @@ template <int BN, int STAGES, class Epi>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_a_lo,
                const __grid_constant__ CUtensorMap map_w, int M, int N, int K, int split, Epi epi, int* err,
-               int ksplit, int part_rows) {
+               int ksplit, int part_rows, const int2* bounds) {
   static_assert(SmemLayout<BN, STAGES>::TILE_BIAS_OFFSET + 1024 <= SmemLayout<BN, STAGES>::STAGE_OUT_OFFSET +
                 SmemLayout<BN, STAGES>::STAGE_OUT_BYTES, "bias tile must fit behind the store boxes");
   using SL = SmemLayout<BN, STAGES>;
@@ -255,9 +268,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // [W | W], i.e. both products accumulate into the same TMEM tile.
   const int kb_per_pass = (K + BK - 1) / BK;
   auto slab_begin = [&](int slice) { return (int)((long long)kb_per_pass * slice / ksplit); };
+  // k slabs of a tile: a slice of them all, or (never sliced) those inside the bounds of its columns
+  auto slabs_of = [&](int slice, int n0) -> SlabRange {
+    if (bounds != nullptr) return slab_range(bounds, n0, BN, N, kb_per_pass);
+    return {slab_begin(slice), slab_begin(slice + 1)};
+  };
   constexpr uint32_t TMEM_COLS = 2 * BN;  // two accumulator buffers (power of two >= 32)
 
   if (threadIdx.x == 0) {
+    prefetch_map(&map_a);
+    prefetch_map(&map_w);
+    if (split) prefetch_map(&map_a_lo);
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
@@ -276,9 +297,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   }
   tcgen05_fence_before();
   __syncthreads();
-    prefetch_map(&map_a);
-    prefetch_map(&map_w);
-    if (split) prefetch_map(&map_a_lo);
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   if constexpr (Epi::kTmaCols > 0) {
@@ -298,7 +316,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         const int mn = tile / ksplit, slice = tile - mn * ksplit;
         const int m0 = (mn / tiles_n) * BM, n0 = (mn % tiles_n) * BN;
-        const int kb0 = slab_begin(slice), nkb = slab_begin(slice + 1) - kb0;
+        const SlabRange sr = slabs_of(slice, n0);
+        const int kb0 = sr.begin, nkb = sr.end - kb0;
         const int kblocks = split ? 2 * nkb : nkb;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, err, TFERR_WAIT_EMPTY)) { ok = false; break; }
@@ -325,8 +344,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, err, TFERR_WAIT_TMEM_EMPTY)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN;
-        const int slice = tile % ksplit;
-        const int kblocks = (split ? 2 : 1) * (slab_begin(slice + 1) - slab_begin(slice));
+        const int mn = tile / ksplit, slice = tile - mn * ksplit;
+        const SlabRange sr = slabs_of(slice, (mn % tiles_n) * BN);
+        const int kblocks = (split ? 2 : 1) * (sr.end - sr.begin);
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(full_bar(stage), phase, err, TFERR_WAIT_FULL)) { ok = false; break; }
           tcgen05_fence_after();

@@ -87,7 +87,7 @@ template <class Epi>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_a_lo,
                 const __grid_constant__ CUtensorMap map_w, int M, int N, int K, int split, Epi epi, int* err, int ksplit,
-                int part_rows) {
+                int part_rows, const int2* bounds) {
   static_assert(Epi::kTmaCols > 0, "the pair kernel has the bulk-store epilogue only");
   using SL = Smem2;
   extern __shared__ uint8_t smem_raw2[];
@@ -113,12 +113,27 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   // (48 KB, four stages in the same 192 KB), so the weight slab is fetched once for both products.
   const int kblocks_all = (K + BK - 1) / BK;
   auto slab_begin = [&](int slice) { return (int)((long long)kblocks_all * slice / ksplit); };
+  // k slabs of a tile: a slice of them all, or (never sliced) those inside the bounds of its columns
+  auto slabs_of = [&](int slice, int n_tile) -> SlabRange {
+    if (bounds != nullptr) return slab_range(bounds, n_tile * BN2, BN2, N, kblocks_all);
+    return {slab_begin(slice), slab_begin(slice + 1)};
+  };
+  // Column tile of tile index mn.  With bounds the tiles of a row differ in length: every row starts with another one, so that
+  // the tiles a pair walks (every num_pairs-th) average out (100 000 rows, lengths 4 / 8 / 12 / 16: the longest pair has 1.10 times
+  // the mean instead of 1.25).
+  auto n_tile_of = [&](int mn) {
+    const int row = mn / tiles_n, j = mn - row * tiles_n;
+    return bounds != nullptr ? (j + row) % tiles_n : j;
+  };
   const uint32_t stage_bytes = split ? (uint32_t)(2 * SL::A_BYTES + SL::B_BYTES) : (uint32_t)SL::STAGE_BYTES;
   const int nstages = split ? 4 : STAGES2;
   const uint32_t w_off = split ? 2u * SL::A_BYTES : (uint32_t)SL::A_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BN2;
 
   if (threadIdx.x == 0) {
+    prefetch_map(&map_a);
+    prefetch_map(&map_w);
+    if (split) prefetch_map(&map_a_lo);
     for (int s = 0; s < STAGES2; ++s) {
       mbar_init(full_bar(s), 1);   // leader's: its own arrive.expect_tx; both CTAs' bytes complete on it
       mbar_init(empty_bar(s), 1);  // one multicast commit of the leader's MMA thread
@@ -131,9 +146,6 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   }
   if (warp == 1) {  // pair-wide allocation: the same warp in both CTAs, same destination
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
-    prefetch_map(&map_a);
-    prefetch_map(&map_w);
-    if (split) prefetch_map(&map_a_lo);
                  "r"(TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -158,8 +170,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
         const int mn = tile / ksplit, slice = tile - mn * ksplit;
-        const int m0 = (mn / tiles_n) * (2 * BM) + (int)rank * BM, n0 = (mn % tiles_n) * BN2 + (int)rank * (BN2 / 2);
-        const int kb0 = slab_begin(slice), kblocks = slab_begin(slice + 1) - kb0;
+        const int nt = n_tile_of(mn);
+        const int m0 = (mn / tiles_n) * (2 * BM) + (int)rank * BM, n0 = nt * BN2 + (int)rank * (BN2 / 2);
+        const SlabRange sr = slabs_of(slice, nt);
+        const int kb0 = sr.begin, kblocks = sr.end - kb0;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, err, TFERR_WAIT_EMPTY)) { ok = false; break; }
           if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * stage_bytes);
@@ -187,8 +201,9 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, err, TFERR_WAIT_TMEM_EMPTY)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN2;
-        const int slice = tile % ksplit;
-        const int kblocks = slab_begin(slice + 1) - slab_begin(slice);
+        const int mn = tile / ksplit, slice = tile - mn * ksplit;
+        const SlabRange sr = slabs_of(slice, n_tile_of(mn));
+        const int kblocks = sr.end - sr.begin;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(full_bar(stage), phase, err, TFERR_WAIT_FULL)) { ok = false; break; }
           tcgen05_fence_after();
@@ -222,19 +237,19 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     // this thread's bias of the next tile is fetched one tile ahead, so its latency is off the epilogue's path
     float next_bias = 0.f;
     if (pair < num_tiles && etid < BN2) {
-      const int nn = ((pair / ksplit) % tiles_n) * BN2 + etid;
+      const int nn = n_tile_of(pair / ksplit) * BN2 + etid;
       next_bias = epi.col_const(nn, nn < N);
     }
     for (int tile = pair; tile < num_tiles; tile += num_pairs, ++it) {
       const int mn = tile / ksplit, slice = tile - mn * ksplit;
-      const int m0 = (mn / tiles_n) * (2 * BM) + (int)rank * BM, n0 = (mn % tiles_n) * BN2;
+      const int m0 = (mn / tiles_n) * (2 * BM) + (int)rank * BM, n0 = n_tile_of(mn) * BN2;
       const int acc = it & 1;
       const uint32_t acc_phase = (it >> 1) & 1;
       named_bar_sync(1, 32 * NUM_EPI_WARPS);
       if (etid < BN2) tile_bias[etid] = next_bias;
       named_bar_sync(1, 32 * NUM_EPI_WARPS);
       if (tile + num_pairs < num_tiles && etid < BN2) {
-        const int nn = (((tile + num_pairs) / ksplit) % tiles_n) * BN2 + etid;
+        const int nn = n_tile_of((tile + num_pairs) / ksplit) * BN2 + etid;
         next_bias = epi.col_const(nn, nn < N);
       }
       if (ok && !mbar_wait(tfull_bar(acc), acc_phase, err, TFERR_WAIT_TMEM_FULL)) ok = false;

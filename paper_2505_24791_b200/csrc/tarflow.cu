@@ -8,6 +8,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cstdarg>
 #include <cstdio>
@@ -138,6 +139,7 @@ struct Matrix {       // a linear layer's weight [N, K]
   CUtensorMap map;    // bf16 engine: box 64 x bn
   int bn = 0;
   CUtensorMap map_seq;  // bf16 engine: box 64 x 128 for the sequential-step GEMM
+  const int2* bounds = nullptr;  // masked layers: per 128 columns the k slabs that hold weights (null: all)
 };
 struct LayerW {
   float *ln1_g, *ln1_b, *b_qkv, *b_o, *ln2_g, *ln2_b, *b_1, *b_2;
@@ -402,7 +404,7 @@ static int dev_alloc(tf_model* m, T** p, size_t count) {
 template <int BN, int STAGES, class Epi>
 static int launch_gemm_tc(tf_model* m, int cls, cudaStream_t stream, const CUtensorMap& ma, const CUtensorMap* ma_lo,
                           const CUtensorMap& mw, int M, int N, int K, const Epi& epi, int* err, int num_sms,
-                          int64_t* launches, int ksplit = 1, int part_rows = 0) {
+                          int64_t* launches, int ksplit = 1, int part_rows = 0, const int2* bounds = nullptr) {
   using SL = tc::SmemLayout<BN, STAGES>;
   if (ksplit < 1 || ksplit > (K + tc::BK - 1) / tc::BK || (ksplit > 1 && Epi::kTmaCols == 0))
     return fail(TF_EINVAL, "gemm_tc_kernel: bad K split %d", ksplit);
@@ -418,7 +420,7 @@ static int launch_gemm_tc(tf_model* m, int cls, cudaStream_t stream, const CUten
   int grid = tiles < num_sms ? tiles : num_sms;
   if (m) m->pre(cls);
   launch_pdl_raw(stream, kern, dim3(grid), dim3(tc::NUM_THREADS), (size_t)SL::TOTAL, ma, ma_lo ? *ma_lo : ma, mw, M, N, K,
-                 ma_lo ? 1 : 0, epi, err, ksplit, part_rows);
+                 ma_lo ? 1 : 0, epi, err, ksplit, part_rows, bounds);
   if (m) m->post(cls); else if (launches) ++*launches;
   return check_launch("gemm_tc_kernel");
 }
@@ -426,7 +428,7 @@ static int launch_gemm_tc(tf_model* m, int cls, cudaStream_t stream, const CUten
 // pair kernel: 256 x 256 tiles on clusters of two CTAs (N % 256 == 0, bulk-store epilogues)
 template <class Epi>
 static int launch_gemm_tc2(tf_model* m, int cls, const CUtensorMap& ma, const CUtensorMap* ma_lo, const CUtensorMap& mw, int M,
-                           int N, int K, const Epi& epi, int ksplit = 1, int part_rows = 0) {
+                           int N, int K, const Epi& epi, int ksplit = 1, int part_rows = 0, const int2* bounds = nullptr) {
   if (ksplit < 1 || ksplit > (K + tc::BK - 1) / tc::BK) return fail(TF_EINVAL, "gemm_tc2_kernel: bad K split %d", ksplit);
   auto kern = tc2::gemm_tc2_kernel<Epi>;
   static bool configured[kMaxDevices] = {false};  // per instantiation and device
@@ -454,7 +456,7 @@ static int launch_gemm_tc2(tf_model* m, int cls, const CUtensorMap& ma, const CU
   lc.attrs = at;
   lc.numAttrs = 2;
   m->pre(cls);
-  cudaError_t e = cudaLaunchKernelEx(&lc, kern, ma, ma_lo ? *ma_lo : ma, mw, M, N, K, ma_lo ? 1 : 0, epi, m->err, ksplit, part_rows);
+  cudaError_t e = cudaLaunchKernelEx(&lc, kern, ma, ma_lo ? *ma_lo : ma, mw, M, N, K, ma_lo ? 1 : 0, epi, m->err, ksplit, part_rows, bounds);
   m->post(cls);
   if (e != cudaSuccess) return fail(TF_ECUDA, "gemm_tc2_kernel launch failed: %s", cudaGetErrorString(e));
   return TF_OK;
@@ -504,16 +506,16 @@ static int gemm(tf_model* m, int cls, const T* A, const CUtensorMap* map_a, cons
       // and K slices (ksplit > 1: partial products, added by the consumer) fill the rest of the GPU
       if (M <= m->small_m_rows && W.N % 128 == 0)
         return launch_gemm_tc<128, 6, Epi>(m, cls, m->stream, *map_a, map_a_lo, W.map_seq, M, W.N, W.K, epi, m->err,
-                                           m->num_sms, nullptr, ksplit, part_rows);
+                                           m->num_sms, nullptr, ksplit, part_rows, W.bounds);
       if (m->use_pair_gemm && W.N % 256 == 0 && M >= 256)
-        return launch_gemm_tc2<Epi>(m, cls, *map_a, map_a_lo, W.map_seq, M, W.N, W.K, epi, ksplit, part_rows);
+        return launch_gemm_tc2<Epi>(m, cls, *map_a, map_a_lo, W.map_seq, M, W.N, W.K, epi, ksplit, part_rows, W.bounds);
     }
     if (ksplit > 1) return fail(TF_EINVAL, "no K-split kernel for this shape");
     if (W.bn == 256)
       return launch_gemm_tc<256, 4, Epi>(m, cls, m->stream, *map_a, map_a_lo, W.map, M, W.N, W.K, epi, m->err,
-                                         m->num_sms, nullptr);
+                                         m->num_sms, nullptr, 1, 0, W.bounds);
     return launch_gemm_tc<128, 6, Epi>(m, cls, m->stream, *map_a, map_a_lo, W.map, M, W.N, W.K, epi, m->err,
-                                       m->num_sms, nullptr);
+                                       m->num_sms, nullptr, 1, 0, W.bounds);
   } else {
     return launch_gemm_simt<T, Epi>(m, cls, A, W, M, epi);
   }
@@ -2145,6 +2147,32 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
   return TF_OK;
 }
 
+// Per 128 rows of the weight matrix (= columns of the product) the range of 64-wide k slabs outside which they are all zero.
+static int upload_slab_bounds(tf_model* m, Matrix* W, const float* w) {
+  if (m->cfg.dtype == 0) return TF_OK;
+  const int groups = (W->N + 127) / 128, slabs = (W->K + tc::BK - 1) / tc::BK;
+  std::vector<int2> bounds(groups);
+  for (int j = 0; j < groups; ++j) {
+    int first = W->K, last = -1;
+    for (int n = 128 * j; n < W->N && n < 128 * (j + 1); ++n) {
+      const float* row = w + (size_t)n * W->K;
+      int a = 0, b = W->K - 1;
+      while (a < first && row[a] == 0.f) ++a;
+      while (b > last && row[b] == 0.f) --b;
+      if (a < first) first = a;
+      if (b > last) last = b;
+    }
+    if (last < 0) first = last = 0;  // no weight at all: one slab of zeros
+    bounds[j] = make_int2(first / tc::BK, last / tc::BK + 1);
+    if (bounds[j].y > slabs) bounds[j].y = slabs;
+  }
+  int2* dev = nullptr;
+  TF_TRY(dev_alloc(m, &dev, groups));
+  CU_OK(cudaMemcpy(dev, bounds.data(), groups * sizeof(int2), cudaMemcpyHostToDevice));
+  W->bounds = dev;
+  return TF_OK;
+}
+
 // ---- loading an MLP-based flow: masks and the layer permutation are applied to the weights here ----------------
 // Degrees (MADE): input i has degree i + 1, hidden unit j of either hidden layer 1 + (j mod (D - 1)), output i degree
 // i + 1.  A hidden unit keeps the weights from inputs / hidden units of degree <= its own, an output those from
@@ -2168,7 +2196,18 @@ static int maf_load_impl(tf_model* m, const void* blob, size_t nbytes, int D, in
   if (c.dtype == 1) CU_OK(cudaMalloc(&staging, max_mat * sizeof(float)));
   struct Guard { float* p; ~Guard() { if (p) cudaFree(p); } } guard{staging};
 
-  auto deg_hidden = [&](int j) { return 1 + j % (D > 1 ? D - 1 : 1); };
+  // Hidden units are kept sorted by degree (rows of a matrix and columns of the next): the masked matrices become block
+  // triangular and the GEMMs leave out the k slabs in which a column group has no weight.  unit[j]: unit in place j.
+  auto degree = [&](int j) { return 1 + j % (D > 1 ? D - 1 : 1); };
+  std::vector<int> unit(H);
+  for (int j = 0; j < H; ++j) unit[j] = j;
+  std::stable_sort(unit.begin(), unit.end(), [&](int a, int b) { return degree(a) < degree(b); });
+  auto deg_hidden = [&](int j) { return degree(unit[j]); };
+  std::vector<float> vec(H);
+  auto upload_sorted = [&](float** dst, const float* src) -> int {
+    for (int j = 0; j < H; ++j) vec[j] = src[unit[j]];
+    return upload_f32(m, dst, vec.data(), H);
+  };
   BlobReader rd{reinterpret_cast<const float*>(reinterpret_cast<const char*>(blob) + 64), nullptr};
   m->maf_blocks.resize(c.n_blocks);
   std::vector<float> tmp, btmp(2 * D);
@@ -2179,16 +2218,18 @@ static int maf_load_impl(tf_model* m, const void* blob, size_t nbytes, int D, in
     tmp.assign((size_t)H * D, 0.f);
     for (int j = 0; j < H; ++j)
       for (int i = 0; i < D; ++i)
-        if (deg_hidden(j) >= i + 1) tmp[(size_t)j * D + (rev ? D - 1 - i : i)] = w1[(size_t)j * D + i];
+        if (deg_hidden(j) >= i + 1) tmp[(size_t)j * D + (rev ? D - 1 - i : i)] = w1[(size_t)unit[j] * D + i];
     TF_TRY(upload_matrix(m, &bw.w1, tmp.data(), H, D, staging));
-    TF_TRY(upload_f32(m, &bw.b1, rd.take(H), H));
+    TF_TRY(upload_slab_bounds(m, &bw.w1, tmp.data()));
+    TF_TRY(upload_sorted(&bw.b1, rd.take(H)));
     const float* w2 = rd.take((size_t)H * H);
     tmp.assign((size_t)H * H, 0.f);
     for (int j = 0; j < H; ++j)
       for (int i = 0; i < H; ++i)
-        if (deg_hidden(j) >= deg_hidden(i)) tmp[(size_t)j * H + i] = w2[(size_t)j * H + i];
+        if (deg_hidden(j) >= deg_hidden(i)) tmp[(size_t)j * H + i] = w2[(size_t)unit[j] * H + unit[i]];
     TF_TRY(upload_matrix(m, &bw.w2, tmp.data(), H, H, staging));
-    TF_TRY(upload_f32(m, &bw.b2, rd.take(H), H));
+    TF_TRY(upload_slab_bounds(m, &bw.w2, tmp.data()));
+    TF_TRY(upload_sorted(&bw.b2, rd.take(H)));
     // output layer [mu | alpha] -> interleaved rows (2 i, 2 i + 1) = (mu_i, alpha_i) in the sample's own order
     const float* w3 = rd.take((size_t)2 * D * H);
     const float* b3 = rd.take((size_t)2 * D);
@@ -2197,13 +2238,14 @@ static int maf_load_impl(tf_model* m, const void* blob, size_t nbytes, int D, in
       const int r = rev ? D - 1 - i : i;  // position of the layer's dimension i in the sample's order
       for (int j = 0; j < H; ++j)
         if (i + 1 > deg_hidden(j)) {
-          tmp[(size_t)(2 * r) * H + j] = w3[(size_t)i * H + j];
-          tmp[(size_t)(2 * r + 1) * H + j] = w3[(size_t)(D + i) * H + j];
+          tmp[(size_t)(2 * r) * H + j] = w3[(size_t)i * H + unit[j]];
+          tmp[(size_t)(2 * r + 1) * H + j] = w3[(size_t)(D + i) * H + unit[j]];
         }
       btmp[2 * r] = b3[i];
       btmp[2 * r + 1] = b3[D + i];
     }
     TF_TRY(upload_matrix(m, &bw.w3, tmp.data(), 2 * D, H, staging));
+    TF_TRY(upload_slab_bounds(m, &bw.w3, tmp.data()));
     TF_TRY(upload_f32(m, &bw.b3, btmp.data(), btmp.size()));
   }
 
