@@ -95,7 +95,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
   using C = Cfg<SPLIT>;
   constexpr int KV_STAGES = C::KV_STAGES, KV_RING = C::KV_RING;
   extern __shared__ uint8_t smem_attn_raw[];
-  pdl_launch_dependents();  // the next kernel of the stream may be scheduled; it waits for this one to complete
   uint8_t* smem = align1024(smem_attn_raw);
   const uint32_t sQ = smem_u32(smem), sK = sQ + C::Q_ALL, sV = sK + KV_STAGES * C::K_SLOT, sP = sV + KV_STAGES * C::V_SLOT;
   const uint32_t bar_base = sP + C::P_ALL;
@@ -133,6 +132,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_co
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // The next kernel of the stream may be scheduled (it waits for this one to complete).  Not before the tensor memory of this CTA
+  // is allocated: the next kernel's CTAs may fit beside this one's, and would hold columns that this kernel still has to get.
+  pdl_launch_dependents();
   if (threadIdx.x == 64) {
     prefetch_map(map_out);
     if constexpr (SPLIT) prefetch_map(map_out_lo);

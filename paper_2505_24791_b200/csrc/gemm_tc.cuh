@@ -115,6 +115,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+__device__ __forceinline__ void prefetch_tile(const CUtensorMap* map, int x, int y) {  // into L2
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
+}
+
 // Bulk tensor stores from shared memory (the TMA engine writes whole row segments; the SM issues one
 // instruction per box).  `tma_reduce_add_2d` adds the fp32 box into global memory instead of storing it.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, uint32_t src) {
@@ -264,8 +268,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // k slabs, and slice s stores its partial tile part_rows * s rows further down; the consumer adds the slices in
   // index order.  Tile index = (m tile, n tile, slice) with the slice fastest.
   const int num_tiles = tiles_m * tiles_n * ksplit;
-  // split != 0: A is an error-compensated pair (hi + lo); the K loop runs over [A_hi | A_lo] against
-  // [W | W], i.e. both products accumulate into the same TMEM tile.
+  // split != 0: A is an error-compensated pair (hi + lo).  A stage then holds [A_hi | A_lo | W] of one k slab, so the weight slab
+  // is fetched once for both products, which accumulate into the same TMEM tile.
+  const uint32_t w_off = split ? 2u * SL::A_BYTES : (uint32_t)SL::A_BYTES, stage_bytes = w_off + SL::B_BYTES;
+  const int nstages = split ? STAGES * SL::STAGE_BYTES / (2 * SL::A_BYTES + SL::B_BYTES) : STAGES;
   const int kb_per_pass = (K + BK - 1) / BK;
   auto slab_begin = [&](int slice) { return (int)((long long)kb_per_pass * slice / ksplit); };
   // k slabs of a tile: a slice of them all, or (never sliced) those inside the bounds of its columns
@@ -288,6 +294,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       mbar_init(tempty_bar(a), NUM_EPI_WARPS);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // few rows: the weights mostly come from memory and pace the tile (requested once per column tile)
+  if (gridDim.x >= num_tiles && blockIdx.x < tiles_n * ksplit && threadIdx.x == 96) {
+    const int n_tile = blockIdx.x / ksplit, n0 = n_tile * BN;
+    const SlabRange sr = slabs_of(blockIdx.x - n_tile * ksplit, n0);
+    for (int s = sr.begin; s < sr.end; ++s) prefetch_tile(&map_w, s * BK, n0);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
@@ -318,15 +330,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const int m0 = (mn / tiles_n) * BM, n0 = (mn % tiles_n) * BN;
         const SlabRange sr = slabs_of(slice, n0);
         const int kb0 = sr.begin, nkb = sr.end - kb0;
-        const int kblocks = split ? 2 * nkb : nkb;
-        for (int kb = 0; kb < kblocks; ++kb) {
+        for (int kb = 0; kb < nkb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, err, TFERR_WAIT_EMPTY)) { ok = false; break; }
-          mbar_arrive_expect_tx(full_bar(stage), SL::STAGE_BYTES);
-          const uint32_t sa = smem_base + stage * SL::STAGE_BYTES;
-          const int kk = (kb0 + (kb >= nkb ? kb - nkb : kb)) * BK;
-          tma_load_2d(sa, kb >= nkb ? &map_a_lo : &map_a, kk, m0, full_bar(stage));
-          tma_load_2d(sa + SL::A_BYTES, &map_w, kk, n0, full_bar(stage));
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          mbar_arrive_expect_tx(full_bar(stage), stage_bytes);
+          const uint32_t sa = smem_base + stage * stage_bytes;
+          const int kk = (kb0 + kb) * BK;
+          tma_load_2d(sa, &map_a, kk, m0, full_bar(stage));
+          if (split) tma_load_2d(sa + SL::A_BYTES, &map_a_lo, kk, m0, full_bar(stage));
+          tma_load_2d(sa + w_off, &map_w, kk, n0, full_bar(stage));
+          if (++stage == nstages) { stage = 0; phase ^= 1u; }
         }
       }
     }
@@ -346,19 +358,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const uint32_t d_tmem = tmem_base + acc * BN;
         const int mn = tile / ksplit, slice = tile - mn * ksplit;
         const SlabRange sr = slabs_of(slice, (mn % tiles_n) * BN);
-        const int kblocks = (split ? 2 : 1) * (sr.end - sr.begin);
+        const int kblocks = sr.end - sr.begin;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(full_bar(stage), phase, err, TFERR_WAIT_FULL)) { ok = false; break; }
           tcgen05_fence_after();
-          const uint32_t sa = smem_base + stage * SL::STAGE_BYTES;
-          const uint64_t adesc = make_smem_desc(sa), bdesc = make_smem_desc(sa + SL::A_BYTES);
+          const uint32_t sa = smem_base + stage * stage_bytes;
+          const uint64_t adesc = make_smem_desc(sa), bdesc = make_smem_desc(sa + w_off);
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             // advancing 16 bf16 = 32 bytes along K inside the swizzled row: +2 in 16-byte units
             umma_f16(d_tmem, adesc + 2u * k, bdesc + 2u * k, idesc, (kb | k) != 0);
           }
+          if (split) {  // the low halves against the same weight slab
+            const uint64_t ldesc = make_smem_desc(sa + SL::A_BYTES);
+#pragma unroll
+            for (int k = 0; k < BK / UMMA_K; ++k) umma_f16(d_tmem, ldesc + 2u * k, bdesc + 2u * k, idesc, 1u);
+          }
           umma_commit(empty_bar(stage));  // frees the stage once these MMAs have read it
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == nstages) { stage = 0; phase ^= 1u; }
         }
         if (ok) umma_commit(tfull_bar(acc));  // accumulator complete
       }

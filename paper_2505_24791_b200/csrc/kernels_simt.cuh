@@ -371,18 +371,18 @@ resid_sum_ln_kernel(float* x, const float* __restrict__ part, int ksplit, int pa
   const int row = blockIdx.x, k = threadIdx.x, dv = d >> 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   const float4 g = reinterpret_cast<const float4*>(gamma)[k], bb = reinterpret_cast<const float4*>(beta)[k];
-  const float4 rb = reinterpret_cast<const float4*>(rbias)[k];
+  const float4 rb = ksplit > 0 ? reinterpret_cast<const float4*>(rbias)[k] : make_float4(0.f, 0.f, 0.f, 0.f);
   pdl_wait();
   float4 a = reinterpret_cast<const float4*>(x)[(size_t)row * dv + k];
   float4 p[MAXS];
 #pragma unroll
   for (int s = 0; s < MAXS; ++s)
     if (s < ksplit) p[s] = reinterpret_cast<const float4*>(part)[((size_t)s * part_rows + row) * dv + k];
-  a.x += rb.x; a.y += rb.y; a.z += rb.z; a.w += rb.w;
+  if (ksplit > 0) { a.x += rb.x; a.y += rb.y; a.z += rb.z; a.w += rb.w; }
 #pragma unroll
   for (int s = 0; s < MAXS; ++s)
     if (s < ksplit) { a.x += p[s].x; a.y += p[s].y; a.z += p[s].z; a.w += p[s].w; }
-  reinterpret_cast<float4*>(x)[(size_t)row * dv + k] = a;
+  if (ksplit > 0) reinterpret_cast<float4*>(x)[(size_t)row * dv + k] = a;
   float v = warp_sum((a.x + a.y) + (a.z + a.w));
   if (lane == 0) s_red[0][warp] = v;
   __syncthreads();
@@ -596,45 +596,6 @@ __global__ void jacobi_update_kernel(const float* __restrict__ o, const float* _
     }
     atomic_max_nonneg(maxdiff + b, fabsf(nw - old));
   }
-}
-
-// Jacobi update of sweeps over few rows, where the head projection left its result as `ksplit` K-slice partial
-// products (slice s of row r at part[(s * part_rows + r) * npad], columns interleaved (mu~_c, alpha~_c), npad >= 2D):
-// head = bias + slice 0 + slice 1 + ... (this order), then Algorithm 1's update line as in the fused epilogue: row
-// (slot s, position l) updates token l + 1 of sample idx[s], the last position's row copies token 0.  One warp per
-// row; per-row max|du| merged with the order-independent atomic max (NaN propagates).
-__global__ void __launch_bounds__(256)
-jacobi_update_split_kernel(const float* __restrict__ part, int ksplit, int part_rows, int npad, const float* __restrict__ bias,
-                           const float* __restrict__ v, float* __restrict__ u, float* __restrict__ maxdiff,
-                           const int* __restrict__ idx, int n_rows, int L, int D, int reversed) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (row >= n_rows) return;
-  const int s = row / L, l = row - s * L;
-  const int b = idx ? idx[s] : s;
-  const bool upd = l < L - 1;
-  const size_t e0 = ((size_t)b * L + tok_index(upd ? l + 1 : 0, L, reversed)) * D;
-  float df = 0.f;
-  for (int c = lane; c < D; c += 32) {
-    float2 o = *reinterpret_cast<const float2*>(bias + 2 * c);
-    for (int k = 0; k < ksplit; ++k) {
-      const float2 p = __ldcg(reinterpret_cast<const float2*>(part + ((size_t)k * part_rows + row) * npad + 2 * c));
-      o.x += p.x;
-      o.y += p.y;
-    }
-    const float old = u[e0 + c], vv = v[e0 + c];
-    const float nw = upd ? fmaf(vv, expf(o.y), o.x) : vv;
-    u[e0 + c] = nw;
-    const float dd = fabsf(nw - old);
-    df = (dd > df || dd != dd) ? dd : df;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float other = __shfl_xor_sync(0xffffffffu, df, o);
-    df = (other > df || other != other) ? other : df;
-  }
-  if (lane == 0) atomic_max_nonneg(maxdiff + b, df);
 }
 
 // First sweep of a block whose samples all start from u^0 = 0 without class labels: every sample's causal pass sees the
@@ -1019,6 +980,8 @@ __global__ void __launch_bounds__(256) l2_distance_kernel(const float* __restric
 template <class T>
 __global__ void maf_cast_rows_kernel(const float* __restrict__ u, const int* __restrict__ idx, T* __restrict__ a,
                                      T* __restrict__ a_lo, int n_slots, int D) {
+  pdl_launch_dependents();
+  pdl_wait();
   if ((D & 3) == 0) {
     const int d4 = D >> 2;
     const size_t total = (size_t)n_slots * d4;
@@ -1059,6 +1022,8 @@ __global__ void maf_cast_rows_kernel(const float* __restrict__ u, const int* __r
 __global__ void __launch_bounds__(256) maf_update_kernel(const float* __restrict__ o, const float* __restrict__ v,
                                                          float* __restrict__ u, float* __restrict__ maxdiff,
                                                          const int* __restrict__ idx, int n_slots, int D, int only_col) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int s = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (s >= n_slots) return;

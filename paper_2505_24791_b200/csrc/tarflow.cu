@@ -28,6 +28,7 @@
 #include "f32_engine.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_tc2.cuh"
+#include "gemm_few.cuh"
 #include "kernels_simt.cuh"
 #include "seq_decode.cuh"
 #include "seq_persist.cuh"
@@ -139,6 +140,8 @@ struct Matrix {       // a linear layer's weight [N, K]
   CUtensorMap map;    // bf16 engine: box 64 x bn
   int bn = 0;
   CUtensorMap map_seq;  // bf16 engine: box 64 x 128 for the sequential-step GEMM
+  CUtensorMap map_few;  // bf16 engine: box 64 x few_bn for sweeps over few rows
+  int few_bn = 0;
   const int2* bounds = nullptr;  // masked layers: per 128 columns the k slabs that hold weights (null: all)
 };
 struct LayerW {
@@ -166,7 +169,7 @@ struct tf_model {
   void *xn = nullptr, *qkv = nullptr, *att = nullptr, *mlp = nullptr, *kcache = nullptr, *vcache = nullptr;
   void *xn_lo = nullptr, *qkv_lo = nullptr, *att_lo = nullptr, *mlp_lo = nullptr;  // second terms (bf16 engine)
   CUtensorMap map_xn, map_att, map_mlp, map_xn_lo, map_att_lo, map_mlp_lo;
-  enum { SM_QKV, SM_QKV_LO, SM_MLP, SM_MLP_LO, SM_H, SM_ATT3, SM_ATT3_LO, SM_PART, SM_PART_HEAD, SM_COUNT };
+  enum { SM_QKV, SM_QKV_LO, SM_MLP, SM_MLP_LO, SM_H, SM_ATT3, SM_ATT3_LO, SM_PART, SM_COUNT };
   CUtensorMap map_qkv3, map_kv3, map_qkv3_lo, map_kv3_lo;  // qkv as [slot][position][3d] for the tensor-core attention (query / key boxes)
   bool use_tc_attention = true;   // single-operand attention on tcgen05 (TARFLOW_ATTN_TC=0: the mma.sync kernel)
   bool use_tc_attention_split = true;  // two-term attention on tcgen05 too (TARFLOW_ATTN_TC_SPLIT=0: mma.sync)
@@ -233,7 +236,6 @@ struct tf_model {
   bool small_m_split = true;    // TARFLOW_SMALL_M_SPLIT=0: the residual projections of such sweeps keep whole-K tiles
   float* sweep_part = nullptr;  // K-slice partial products of the residual projections of such sweeps [part_cap_rows, d]
   int part_cap_rows = 0;
-  int part_head_npad = 0, part_head_rows = 0;  // the same buffer seen as [part_head_rows, part_head_npad] for the head's slices
   int64_t sweep_graph_rows = 4096;  // TARFLOW_SWEEP_GRAPH_ROWS: largest slots x tokens replayed from a graph (0 = never)
   // fp32 engine: blocks that fit a cluster's shared memory are decoded by one launch (f32_engine.cuh)
   f32::SeqPlan seq_plan;
@@ -462,6 +464,36 @@ static int launch_gemm_tc2(tf_model* m, int cls, const CUtensorMap& ma, const CU
   return TF_OK;
 }
 
+// few rows: one 128 x BN tile, or a K slice of one, per CTA (gemm_few.cuh); W.map_few has a box of BN rows
+template <int BN, class Epi>
+static int launch_few(tf_model* m, int cls, const CUtensorMap& ma, const CUtensorMap* ma_lo, const Matrix& W, int M, const Epi& epi,
+                      const float* bias, int ksplit = 1, int part_rows = 0) {
+  using C = few::Cfg<BN>;
+  if (ksplit < 1 || ksplit > (W.K + tc::BK - 1) / tc::BK || W.few_bn != BN) return fail(TF_EINVAL, "gemm_few_kernel: bad K split %d or tile %d", ksplit, BN);
+  auto kern = few::gemm_few_kernel<BN, Epi>;
+  static bool configured[kMaxDevices] = {false};  // per instantiation and device
+  const int dev = current_device();
+  if (dev < 0) return fail(TF_ECUDA, "no usable current device");
+  if (!configured[dev]) {
+    CU_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::MAX_RING + C::EXTRA));
+    configured[dev] = true;
+  }
+  const int per = ((W.K + tc::BK - 1) / tc::BK + ksplit - 1) / ksplit, want = ma_lo ? few::STAGES_SPLIT : few::STAGES;
+  int ring = (per < want ? per : want) * ((ma_lo ? 2 : 1) * C::A_BYTES + C::W_BYTES);
+  if (ring < 8 * few::BOX) ring = 8 * few::BOX;  // the epilogue's boxes
+  const int tiles = (M + tc::BM - 1) / tc::BM * ((W.N + BN - 1) / BN);
+  LAUNCH_PDL(m, cls, kern, tiles * ksplit, few::THREADS, ring + C::EXTRA, ma, ma_lo ? *ma_lo : ma, W.map_few, M, W.N, W.K, ma_lo ? 1 : 0, epi, bias,
+             m->err, ksplit, part_rows, ksplit == 1 ? W.bounds : (const int2*)nullptr, ring);
+  return check_launch("gemm_few_kernel");
+}
+
+// Whether the narrow tiles of a product fit the GPU at once: beyond one wave the wider tiles of the other kernels win (256-token
+// sweeps of width 1024, narrow / wide tiles everywhere: 1 sample 335 / 385 us and, with two-term operands, 414 / 522; 4 samples
+// 809 / 567).
+static bool few_fits(const tf_model* m, int M, const Matrix& W) {
+  return m->small_m_rows > 0 && W.few_bn > 0 && (M + tc::BM - 1) / tc::BM * ((W.N + W.few_bn - 1) / W.few_bn) <= m->num_sms;
+}
+
 template <int BM, int BN, int TM, class Epi>
 static int launch_gemm_f32(tf_model* m, int cls, const float* A, const Matrix& W, int M, const Epi& epi) {
   using C = f32::GemmCfg<BM, BN, TM>;
@@ -540,6 +572,11 @@ static int layernorm(tf_model* m, int cls, const float* x, const float* g, const
                g, b, y, y_lo, d);
     return check_launch("resid_sum_ln_kernel");
   }
+  if (sizeof(T) == 2 && rows <= m->small_m_rows && d % 128 == 0 && d <= 4096) {  // few rows: a CTA per row
+    LAUNCH_PDL(m, cls, resid_sum_ln_kernel<T>, rows, d / 4, 0, const_cast<float*>(x), (const float*)nullptr, 0, 0, (const float*)nullptr,
+               g, b, y, y_lo, d);
+    return check_launch("resid_sum_ln_kernel");
+  }
   int blocks = (rows * 32 + 255) / 256;
   if (d <= 128 * 1) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 1>), blocks, 256, 0, x, g, b, y, y_lo, rows, d);
   else if (d <= 128 * 4) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 4>), blocks, 256, 0, x, g, b, y, y_lo, rows, d);
@@ -573,7 +610,7 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   const bool fused_embed = d % 4 == 0 && d <= 1024 && (size_t)16 * D * sizeof(float) <= EMBED_TOKEN_BYTES;
   if (fused_embed) {
     const LayerW& l0 = bw.layers[0];
-    const bool few = M <= m->small_m_rows;  // few rows: four per CTA instead of sixteen, for four times the CTAs
+    const bool few = M <= 16 * m->num_sms;  // fewer CTAs of sixteen rows than SMs: four rows each instead (1053 rows: 19 -> 10 us)
     const int R = few ? 4 : 16, threads = ((d / 4 + 31) / 32) * 32;
     int cc = EMBED_WEIGHT_BYTES / (2 * d * (int)sizeof(float));  // token values per weight buffer
     cc = cc > D ? D : cc;
@@ -589,21 +626,31 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
                bw.w_in_t, bw.b_in, bw.pos, bw.cls, m->h, L, D, d, rev, M);
   }
   TF_TRY(check_launch("embed_kernel"));
-  // Few rows (bf16 engine): the two projections into the residual stream have d / 128 column tiles per 128 rows, too few
+  // Few rows (bf16 engine): the two projections into the residual stream have d / 64 or d / 128 column tiles per 128 rows, too few
   // CTAs to stream their weights, so they are cut into K slices that leave partial products; the LayerNorm that follows
   // (this layer's second, the next layer's first, or the block's last) adds them to the stream in slice order.
   const int m_pad = (M + 127) / 128 * 128;
-  auto slices_for = [&](int K) -> int {
-    if (sizeof(T) != 2 || m->sweep_part == nullptr || !m->small_m_split || d > 4096) return 1;
-    int ks;
-    if (M <= m->small_m_rows) ks = m->num_sms / ((m_pad / 128) * (d / 128));  // 128 x 128 tiles
-    else if (M <= m->split_m_rows && m->use_pair_gemm && d % 256 == 0 && M >= 256)
-      ks = (m->num_sms / 2) / (((M + 255) / 256) * (d / 256));                // pair tiles
-    else return 1;
-    if (ks > K / (2 * tc::BK)) ks = K / (2 * tc::BK);  // at least two k slabs per slice
-    if (ks > 8) ks = 8;
-    if (ks > m->part_cap_rows / m_pad) ks = m->part_cap_rows / m_pad;
-    return ks < 1 ? 1 : ks;
+  struct Slices { int n; bool narrow; };  // n == 1: no partial products
+  auto slices_for = [&](const Matrix& W) -> Slices {
+    if (sizeof(T) != 2 || m->sweep_part == nullptr || !m->small_m_split || d > 4096) return {1, false};
+    auto slices = [&](int tiles, int ctas) {
+      int ks = ctas / tiles;
+      if (ks > W.K / (2 * tc::BK)) ks = W.K / (2 * tc::BK);  // at least two k slabs per slice
+      if (ks > 8) ks = 8;
+      if (ks > m->part_cap_rows / m_pad) ks = m->part_cap_rows / m_pad;
+      return ks < 1 ? 1 : ks;
+    };
+    if (few_fits(m, M, W)) {
+      // A slab of a 128 x 64 tile takes about 0.25 us, one of a 128 x 128 tile 0.33 us; the wide tiles' epilogue and the LayerNorm
+      // over twice the slices cost 3 us more.  256-token sweeps of width 1024, down projection alone, narrow / wide: 7.4 / 7.4 us
+      // with the LayerNorms at 2.7 / 3.6 us each (1 sample), 26 / 14 us (4 samples).
+      const int n = slices((m_pad / 128) * (d / 64), m->num_sms), w = slices((m_pad / 128) * (d / 128), m->num_sms), slabs = W.K / tc::BK;
+      if (M > m->small_m_rows || slabs * 0.25f / n <= slabs * 0.33f / w + 3.f) return {n, true};
+    }
+    if (M <= m->small_m_rows) return {slices((m_pad / 128) * (d / 128), m->num_sms), false};  // 128 x 128 tiles
+    if (M <= m->split_m_rows && m->use_pair_gemm && d % 256 == 0 && M >= 256)
+      return {slices((M + 255) / 256 * (d / 256), m->num_sms / 2), false};                     // pair tiles
+    return {1, false};
   };
   SplitSum pend{nullptr, 0, 0, nullptr};
   bool has_pend = false;
@@ -614,7 +661,8 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
     first_layer = false;
     if constexpr (sizeof(T) == 2) {
       const CUtensorMap* sm = m->store_maps;
-      TF_TRY(gemm<T>(m, KC_GEMM_QKV, xn, &m->map_xn, mxl, lw.w_qkv, M,
+      if (few_fits(m, M, lw.w_qkv)) TF_TRY(launch_few<64>(m, KC_GEMM_QKV, m->map_xn, mxl, lw.w_qkv, M, few::Store<ACT_NONE>{sm + tf_model::SM_QKV, hp ? sm + tf_model::SM_QKV_LO : nullptr}, lw.b_qkv));
+      else TF_TRY(gemm<T>(m, KC_GEMM_QKV, xn, &m->map_xn, mxl, lw.w_qkv, M,
                      EpiStoreTma<false>{lw.b_qkv, sm + tf_model::SM_QKV, hp ? sm + tf_model::SM_QKV_LO : nullptr}));
     } else {
       TF_TRY(gemm<T>(m, KC_GEMM_QKV, xn, &m->map_xn, mxl, lw.w_qkv, M, EpiStore<T, false>{qkv, lw.b_qkv, 3 * d, qkv_lo}));
@@ -649,11 +697,12 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
     }
     TF_TRY(check_launch("attention kernel"));
     if constexpr (sizeof(T) == 2) {
-      const int ks = slices_for(d);
-      if (ks > 1) {
-        TF_TRY(gemm<T>(m, KC_GEMM_O, att, &m->map_att, mal, lw.w_o, M, EpiStoreF32Tma{nullptr, m->store_maps + tf_model::SM_PART},
-                       ks, m_pad));
-        pend = SplitSum{m->sweep_part, ks, m_pad, lw.b_o};
+      const Slices ks = slices_for(lw.w_o);
+      const CUtensorMap* part = m->store_maps + tf_model::SM_PART;
+      if (ks.n > 1 || ks.narrow) {
+        if (ks.narrow) TF_TRY(launch_few<64>(m, KC_GEMM_O, m->map_att, mal, lw.w_o, M, few::StoreF32{part}, nullptr, ks.n, m_pad));
+        else TF_TRY(gemm<T>(m, KC_GEMM_O, att, &m->map_att, mal, lw.w_o, M, EpiStoreF32Tma{nullptr, part}, ks.n, m_pad));
+        pend = SplitSum{m->sweep_part, ks.n, m_pad, lw.b_o};
         has_pend = true;
       } else {
         TF_TRY(gemm<T>(m, KC_GEMM_O, att, &m->map_att, mal, lw.w_o, M, EpiResidTma{lw.b_o, m->store_maps + tf_model::SM_H}));
@@ -665,12 +714,15 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
     has_pend = false;
     if constexpr (sizeof(T) == 2) {
       const CUtensorMap* sm = m->store_maps;
-      TF_TRY(gemm<T>(m, KC_GEMM_MLP1, xn, &m->map_xn, mxl, lw.w_1, M,
+      if (few_fits(m, M, lw.w_1)) TF_TRY(launch_few<64>(m, KC_GEMM_MLP1, m->map_xn, mxl, lw.w_1, M, few::Store<ACT_GELU>{sm + tf_model::SM_MLP, hp ? sm + tf_model::SM_MLP_LO : nullptr}, lw.b_1));
+      else TF_TRY(gemm<T>(m, KC_GEMM_MLP1, xn, &m->map_xn, mxl, lw.w_1, M,
                      EpiStoreTma<true>{lw.b_1, sm + tf_model::SM_MLP, hp ? sm + tf_model::SM_MLP_LO : nullptr}));
-      const int ks = slices_for(m->hid);
-      if (ks > 1) {
-        TF_TRY(gemm<T>(m, KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, M, EpiStoreF32Tma{nullptr, sm + tf_model::SM_PART}, ks, m_pad));
-        pend = SplitSum{m->sweep_part, ks, m_pad, lw.b_2};
+      const Slices ks = slices_for(lw.w_2);
+      const CUtensorMap* part = m->store_maps + tf_model::SM_PART;
+      if (ks.n > 1 || ks.narrow) {
+        if (ks.narrow) TF_TRY(launch_few<64>(m, KC_GEMM_MLP2, m->map_mlp, mml, lw.w_2, M, few::StoreF32{part}, nullptr, ks.n, m_pad));
+        else TF_TRY(gemm<T>(m, KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, M, EpiStoreF32Tma{nullptr, part}, ks.n, m_pad));
+        pend = SplitSum{m->sweep_part, ks.n, m_pad, lw.b_2};
         has_pend = true;
       } else {
         TF_TRY(gemm<T>(m, KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, M, EpiResidTma{lw.b_2, sm + tf_model::SM_H}));
@@ -682,27 +734,9 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   }
   TF_TRY(layernorm<T>(m, KC_LN, m->h, bw.lnf_g, bw.lnf_b, xn, xn_lo, M, has_pend ? &pend : nullptr));
   if (mode == PASS_JACOBI) {
-    // few rows: the head projection has one or two CTAs that walk K alone, so it is cut into K slices too and a small
-    // kernel adds them and applies the update (otherwise the update is the projection's epilogue)
-    int ks_head = 1;
-    if constexpr (sizeof(T) == 2) {
-      if (M <= m->small_m_rows && m->sweep_part != nullptr && m->small_m_split && bw.w_out.bn == 128 && D % 2 == 0 && d % 128 == 0) {
-        ks_head = m->num_sms / ((m_pad / 128) * ((2 * D + 127) / 128));
-        if (ks_head > d / (2 * tc::BK)) ks_head = d / (2 * tc::BK);
-        if (ks_head > 8) ks_head = 8;
-        if (ks_head > m->part_head_rows / m_pad) ks_head = m->part_head_rows / m_pad;
-        if (ks_head < 1) ks_head = 1;
-      }
-    }
-    if (ks_head > 1) {
-      if constexpr (sizeof(T) == 2) {
-        TF_TRY((launch_gemm_tc<128, 6, EpiStoreF32Tma>(m, KC_GEMM_HEAD_UPDATE, m->stream, m->map_xn, mxl, bw.w_out.map, M, 2 * D, d,
-                                                       EpiStoreF32Tma{nullptr, m->store_maps + tf_model::SM_PART_HEAD}, m->err,
-                                                       m->num_sms, nullptr, ks_head, m_pad)));
-        LAUNCH_PDL(m, KC_GEMM_HEAD_UPDATE, jacobi_update_split_kernel, (M * 32 + 255) / 256, 256, 0, m->sweep_part, ks_head, m_pad,
-                   m->part_head_npad, bw.b_out, v, u_upd, m->maxdiff, idx, M, L, D, rev);
-        TF_TRY(check_launch("jacobi_update_split_kernel"));
-      }
+    if (sizeof(T) == 2 && few_fits(m, M, bw.w_out) && D % 4 == 0) {
+      if constexpr (sizeof(T) == 2)
+        TF_TRY(launch_few<32>(m, KC_GEMM_HEAD_UPDATE, m->map_xn, mxl, bw.w_out, M, few::HeadUpdate{v, u_upd, m->maxdiff, idx, L, D, rev}, bw.b_out));
     } else {
       EpiHeadUpdate epi{v, u_upd, m->maxdiff, idx, bw.b_out, L, D, rev};
       TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, xn, &m->map_xn, mxl, bw.w_out, M, epi));
@@ -1679,14 +1713,20 @@ static int maf_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   m->cur_rows = M;
   int cb = (int)(((size_t)M * ((D & 3) == 0 ? D / 4 : D) + 255) / 256);
   if (cb > 148 * 16) cb = 148 * 16;
-  LAUNCH(m, KC_EMBED, (maf_cast_rows_kernel<T>), cb, 256, 0, u_src, idx, a0, a0_lo, M, D);
+  LAUNCH_PDL(m, KC_EMBED, (maf_cast_rows_kernel<T>), cb, 256, 0, u_src, idx, a0, a0_lo, M, D);
   TF_TRY(check_launch("maf_cast_rows_kernel"));
   if constexpr (sizeof(T) == 2) {
     const CUtensorMap* sm = m->maf_store_maps;
-    TF_TRY(gemm<T>(m, KC_GEMM_MLP1, a0, &m->maf_map[0][0], hp ? &m->maf_map[0][1] : nullptr, bw.w1, M,
-                   EpiStoreTma<ACT_RELU>{bw.b1, sm + 0, hp ? sm + 1 : nullptr}));
-    TF_TRY(gemm<T>(m, KC_GEMM_MLP2, h1, &m->maf_map[1][0], hp ? &m->maf_map[1][1] : nullptr, bw.w2, M,
-                   EpiStoreTma<ACT_RELU>{bw.b2, sm + 2, hp ? sm + 3 : nullptr}));
+    if (H % 64 == 0 && few_fits(m, M, bw.w1)) {
+      const CUtensorMap *l0 = hp ? &m->maf_map[0][1] : nullptr, *l1 = hp ? &m->maf_map[1][1] : nullptr;
+      TF_TRY(launch_few<64>(m, KC_GEMM_MLP1, m->maf_map[0][0], l0, bw.w1, M, few::Store<ACT_RELU>{sm + 0, hp ? sm + 1 : nullptr}, bw.b1));
+      TF_TRY(launch_few<64>(m, KC_GEMM_MLP2, m->maf_map[1][0], l1, bw.w2, M, few::Store<ACT_RELU>{sm + 2, hp ? sm + 3 : nullptr}, bw.b2));
+    } else {
+      TF_TRY(gemm<T>(m, KC_GEMM_MLP1, a0, &m->maf_map[0][0], hp ? &m->maf_map[0][1] : nullptr, bw.w1, M,
+                     EpiStoreTma<ACT_RELU>{bw.b1, sm + 0, hp ? sm + 1 : nullptr}));
+      TF_TRY(gemm<T>(m, KC_GEMM_MLP2, h1, &m->maf_map[1][0], hp ? &m->maf_map[1][1] : nullptr, bw.w2, M,
+                     EpiStoreTma<ACT_RELU>{bw.b2, sm + 2, hp ? sm + 3 : nullptr}));
+    }
   } else {
     TF_TRY(gemm<T>(m, KC_GEMM_MLP1, a0, nullptr, nullptr, bw.w1, M, EpiStore<T, ACT_RELU>{h1, bw.b1, H, h1_lo}));
     TF_TRY(gemm<T>(m, KC_GEMM_MLP2, h1, nullptr, nullptr, bw.w2, M, EpiStore<T, ACT_RELU>{h2, bw.b2, H, h2_lo}));
@@ -1697,8 +1737,9 @@ static int maf_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
     if constexpr (sizeof(T) == 2) {
       // tensor-core engine: the raw (mu, alpha) leave through bulk stores, a row-per-warp kernel applies the update
       // (measured: 381 us for the fused lane-per-column epilogue against 85 + 60 us for the pair on 69 k rows)
-      TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, h2, map2, map2_lo, bw.w3, M, EpiStoreF32Tma{bw.b3, m->maf_store_maps + 4}));
-      LAUNCH(m, KC_AFFINE, maf_update_kernel, (M + 7) / 8, 256, 0, m->o, v, u_upd, m->maxdiff, idx, M, D, only_col);
+      if (few_fits(m, M, bw.w3)) TF_TRY(launch_few<64>(m, KC_GEMM_HEAD_UPDATE, *map2, map2_lo, bw.w3, M, few::StoreF32{m->maf_store_maps + 4}, bw.b3));
+      else TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, h2, map2, map2_lo, bw.w3, M, EpiStoreF32Tma{bw.b3, m->maf_store_maps + 4}));
+      LAUNCH_PDL(m, KC_AFFINE, maf_update_kernel, (M + 7) / 8, 256, 0, m->o, v, u_upd, m->maxdiff, idx, M, D, only_col);
       return check_launch("maf_update_kernel");
     } else {
       EpiMafUpdate epi{v, u_upd, m->maxdiff, idx, bw.b3, D, only_col};
@@ -1787,7 +1828,7 @@ static int upload_f32(tf_model* m, float** dst, const float* src, size_t n) {
 }
 
 // matrix [N, K]: fp32 engine keeps fp32; bf16 engine converts on the device (round to nearest even)
-static int upload_matrix(tf_model* m, Matrix* W, const float* src, int N, int K, float* staging) {
+static int upload_matrix(tf_model* m, Matrix* W, const float* src, int N, int K, float* staging, int few_bn = 64) {
   W->N = N;
   W->K = K;
   size_t n = (size_t)N * K;
@@ -1805,6 +1846,8 @@ static int upload_matrix(tf_model* m, Matrix* W, const float* src, int N, int K,
   W->w = w;
   W->bn = (N % 256 == 0) ? 256 : 128;
   TF_TRY(make_map_bf16(&W->map_seq, w, (uint64_t)N, (uint64_t)K, 128u));
+  W->few_bn = few_bn;
+  TF_TRY(make_map_bf16(&W->map_few, w, (uint64_t)N, (uint64_t)K, (uint32_t)few_bn));
   return make_map_bf16(&W->map, w, (uint64_t)N, (uint64_t)K, (uint32_t)W->bn);
 }
 
@@ -1983,7 +2026,7 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
       btmp[2 * cc] = b_out[cc];
       btmp[2 * cc + 1] = b_out[D + cc];
     }
-    TF_TRY(upload_matrix(m, &bw.w_out, tmp.data(), 2 * D, d, staging));
+    TF_TRY(upload_matrix(m, &bw.w_out, tmp.data(), 2 * D, d, staging, 32));
     TF_TRY(upload_f32(m, &bw.b_out, btmp.data(), btmp.size()));
     if (m->seq_clusters > 0) TF_TRY(upload_seq_images(m, layers, lnf, b_in, w_in_t.data(), tmp.data(), btmp.data()));
   }
@@ -2070,12 +2113,8 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
         m->part_cap_rows = 8192;
         TF_TRY(dev_alloc(m, &m->sweep_part, (size_t)m->part_cap_rows * d));
         TF_TRY(make_map_store(&sm[tf_model::SM_PART], m->sweep_part, (uint64_t)m->part_cap_rows, d, 4));
-        m->part_head_npad = (2 * m->D + 31) / 32 * 32;
-        m->part_head_rows = (int)((size_t)m->part_cap_rows * d / m->part_head_npad);
-        TF_TRY(make_map_store(&sm[tf_model::SM_PART_HEAD], m->sweep_part, (uint64_t)m->part_head_rows, m->part_head_npad, 4));
       } else {
         sm[tf_model::SM_PART] = sm[tf_model::SM_H];
-        sm[tf_model::SM_PART_HEAD] = sm[tf_model::SM_H];
       }
       TF_TRY(make_map_3d(&sm[tf_model::SM_ATT3], m->att, B, L, d, 32));
       TF_TRY(make_map_3d(&m->map_qkv3, m->qkv, B, L, 3 * (uint64_t)d, attn_tc::BQ));

@@ -260,3 +260,31 @@ def test_few_row_sweeps_agree_with_the_one_shape_path_and_the_oracle(name, monke
                 zf, ld = m.forward(xo, None if lab is None else lab[pick])
                 zo, ldo = O.model_forward(m.blocks, xo, None if lab is None else lab[pick], cfg)
                 assert rel_l2(zf, zo) <= 2e-2 and np.abs(ld - ldo).max() <= 2e-2 * max(1.0, np.abs(ldo).max())
+
+
+# H x W patches of 4 x 4 x 3 values (2 x 2 x 3 with D = 12), width, batch: fewer rows than a tile; one row beyond whole tiles and slices of one k
+# slab; 65 x 13 rows in nine tiles; the largest row count whose head still fits one wave of 32-column tiles, narrow and wide
+# products mixed; a head of 24 columns in a tile of 32
+@pytest.mark.parametrize("rows,cols,patch,width,batch", [(5, 5, 4, 128, 1), (3, 43, 4, 128, 3), (9, 9, 4, 256, 13), (16, 16, 4, 512, 24),
+                                                         (16, 16, 2, 512, 4)])
+def test_narrow_tiles_at_their_edges(rows, cols, patch, width, batch, monkeypatch):
+    cfg = synth.config("cfg3", H=patch * rows, W=patch * cols, patch=patch, n_blocks=1, n_layers=2, width=width, n_heads=width // 64,
+                       n_classes=10)
+    L = synth.seq_len(cfg)
+    z = synth.make_latents(cfg, 5300 + rows, B=batch)
+    lab = synth.make_labels(cfg, B=batch)
+    with Model(cfg, max_batch=batch) as m:
+        x, ib, its, rc = m.inverse(z, lab, [1], 1e-3, L + 1)
+        x2, _, its2, _ = m.inverse(z, lab, [1], 1e-3, L + 1)
+        pick = [0, batch - 1]
+        zf, ld = m.forward(x.astype(np.float32), lab)
+    monkeypatch.setenv("TARFLOW_SMALL_M_ROWS", "0")
+    monkeypatch.setenv("TARFLOW_SPLIT_M_ROWS", "0")
+    with Model(cfg, max_batch=batch) as ref:
+        xr, _, itsr, rcr = ref.inverse(z, lab, [1], 1e-3, L + 1)
+    assert rc == 0 and rcr == 0 and np.array_equal(x, x2) and np.array_equal(its, its2)
+    assert np.abs(x - xr).max() <= 2e-3 and np.abs(its - itsr).max() <= 1      # both end within tau = 1e-3 of the fixed point
+    xo, ito = O.model_inverse(m.blocks, z[pick], lab[pick], cfg, [1], 1e-3, L + 1)
+    _close(x[pick], xo)
+    assert np.abs(its[:, pick] - ito).max() <= 1
+    assert rel_l2(zf, z.astype(np.float64)) <= 2e-2
