@@ -130,17 +130,21 @@ gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, int M, int
 }
 
 // ---------------------------------------------------------------------------------------------
-// Causal attention of a sweep.  One CTA (4 warps) per (slot, head, 4 QW queries); keys and values pass through shared
+// Causal attention of a sweep.  One CTA of 8 / QW warps per (slot, head, 8 queries); keys and values pass through shared
 // memory in tiles of 64, a warp handles its QW queries against a tile: a lane scores two keys (q comes with broadcast
 // reads), the running maximum and sum are warp shuffles, then a lane accumulates channels lane, lane + 32, ... with the
 // probabilities read back from shared memory.  qkv rows are [q | k | v], 3d wide; HD % 4 == 0, HD <= 128.
+// QW = 1 halves the chain of a CTA, QW = 2 has fewer idle warps per loaded tile (64 tokens of width 128: sweep of 4 samples 76.8 us with
+// two queries per warp, 70.9 with one; of 64 samples 251 and 258).
 // The warp-per-query kernel it replaces read every key row from global memory one float at a time (19 us at 4 x 64 tokens).
 // ---------------------------------------------------------------------------------------------
-constexpr int AT_KEYS = 64, AT_QW = 2, AT_Q = 4 * AT_QW;
+constexpr int AT_KEYS = 64, AT_Q = 8;
 __host__ __device__ constexpr int attention_smem_floats(int hd) { return 2 * AT_KEYS * (hd + 4) + AT_Q * hd + AT_Q * AT_KEYS; }
 
-__global__ void __launch_bounds__(128)
+template <int AT_QW>
+__global__ void __launch_bounds__(32 * AT_Q / AT_QW)
 attention_kernel(const float* __restrict__ qkv, float* __restrict__ out, int L, int d, int hd, float scale) {
+  constexpr int THREADS = 32 * AT_Q / AT_QW;
   extern __shared__ __align__(16) float s_at[];
   pdl_launch_dependents();
   pdl_wait();
@@ -153,7 +157,7 @@ attention_kernel(const float* __restrict__ qkv, float* __restrict__ out, int L, 
   const size_t ld = 3 * (size_t)d;
   const float* base = qkv + (size_t)slot * L * ld + (size_t)head * hd;
   const int last_q = q0 + AT_Q - 1 < L - 1 ? q0 + AT_Q - 1 : L - 1;
-  for (int i = threadIdx.x; i < AT_Q * hq; i += 128) {
+  for (int i = threadIdx.x; i < AT_Q * hq; i += THREADS) {
     const int r = i / hq, c = i % hq, pos = q0 + r < L ? q0 + r : L - 1;
     float4 x = __ldg(reinterpret_cast<const float4*>(base + (size_t)pos * ld) + c);
     x.x *= scale; x.y *= scale; x.z *= scale; x.w *= scale;
@@ -169,7 +173,7 @@ attention_kernel(const float* __restrict__ qkv, float* __restrict__ out, int L, 
   }
   for (int j0 = 0; j0 <= last_q; j0 += AT_KEYS) {
     __syncthreads();  // the previous tile has been consumed
-    for (int i = threadIdx.x; i < AT_KEYS * hq; i += 128) {
+    for (int i = threadIdx.x; i < AT_KEYS * hq; i += THREADS) {
       const int r = i / hq, c = i % hq;
       const bool ok = j0 + r <= last_q;
       const float* row = base + (size_t)(ok ? j0 + r : 0) * ld + 4 * c;

@@ -511,15 +511,19 @@ static int launch_gemm_f32(tf_model* m, int cls, const float* A, const Matrix& W
 }
 
 // fp32 product.  The tile shrinks until about every SM has one: the kernels are short and few, so spreading a product over
-// more SMs matters more than operand reuse.  K % 4 != 0 (an MLP flow of odd dimension) takes the scalar-load kernel.
+// more SMs matters more than operand reuse.  Rows per thread were chosen by the reads from shared memory that an output costs
+// (sweeps of 64 tokens, width 128: 16 x 32 tiles with 1 / 2 / 4 rows per thread 89.4 / 76.8 / 78.3 us at 4 samples, 32 x 32 tiles with
+// 2 / 4 116 / 104 us at 16; 16 x 16 tiles where 16 x 32 ones would reach half of the SMs at most: 71.6 -> 67.3 us at 4, 62 -> 54 at 1).
+// K % 4 != 0 (an MLP flow of odd dimension) takes the scalar-load kernel.
 template <class T, class Epi>
 static int launch_gemm_simt(tf_model* m, int cls, const T* A, const Matrix& W, int M, const Epi& epi) {
   if constexpr (sizeof(T) == 4) {
     if (W.K % 4 == 0) {
       auto tiles = [&](int bm, int bn) { return ((M + bm - 1) / bm) * ((W.N + bn - 1) / bn); };
       if (tiles(64, 64) >= 2 * m->num_sms) return launch_gemm_f32<64, 64, 8>(m, cls, A, W, M, epi);
-      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, 2>(m, cls, A, W, M, epi);
-      return launch_gemm_f32<16, 32, 1>(m, cls, A, W, M, epi);
+      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, 4>(m, cls, A, W, M, epi);
+      if (tiles(16, 32) * 2 <= m->num_sms) return launch_gemm_f32<16, 16, 1>(m, cls, A, W, M, epi);
+      return launch_gemm_f32<16, 32, 2>(m, cls, A, W, M, epi);
     }
   }
   dim3 grid((W.N + 63) / 64, (M + 63) / 64);
@@ -577,11 +581,12 @@ static int layernorm(tf_model* m, int cls, const float* x, const float* g, const
                g, b, y, y_lo, d);
     return check_launch("resid_sum_ln_kernel");
   }
-  int blocks = (rows * 32 + 255) / 256;
-  if (d <= 128 * 1) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 1>), blocks, 256, 0, x, g, b, y, y_lo, rows, d);
-  else if (d <= 128 * 4) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 4>), blocks, 256, 0, x, g, b, y, y_lo, rows, d);
-  else if (d <= 128 * 8) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 8>), blocks, 256, 0, x, g, b, y, y_lo, rows, d);
-  else LAUNCH_PDL(m, cls, (layernorm_kernel<T, 16>), blocks, 256, 0, x, g, b, y, y_lo, rows, d);
+  // a warp per row; CTAs of two warps while there are few (256 rows of width 128: sweep 71.6 -> 68 us), else of eight
+  const int threads = rows <= 16 * m->num_sms ? 64 : 256, blocks = (int)(((int64_t)rows * 32 + threads - 1) / threads);
+  if (d <= 128 * 1) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 1>), blocks, threads, 0, x, g, b, y, y_lo, rows, d);
+  else if (d <= 128 * 4) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 4>), blocks, threads, 0, x, g, b, y, y_lo, rows, d);
+  else if (d <= 128 * 8) LAUNCH_PDL(m, cls, (layernorm_kernel<T, 8>), blocks, threads, 0, x, g, b, y, y_lo, rows, d);
+  else LAUNCH_PDL(m, cls, (layernorm_kernel<T, 16>), blocks, threads, 0, x, g, b, y, y_lo, rows, d);
   return check_launch("layernorm_kernel");
 }
 
@@ -686,8 +691,13 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
         LAUNCH(m, KC_ATTN, attn::attention_mma_kernel<false>, grid, 128, attn::smem_bytes<false>(), qkv, qkv_lo, att,
                att_lo, L, d, sl2);
     } else if (m->hd % 4 == 0 && m->hd <= 128) {
-      LAUNCH_PDL(m, KC_ATTN, f32::attention_kernel, dim3((L + f32::AT_Q - 1) / f32::AT_Q, m->cfg.n_heads, n_slots), 128,
-                 f32::attention_smem_floats(m->hd) * sizeof(float), qkv, att, L, d, m->hd, 1.0f / sqrtf((float)m->hd));
+      const dim3 grid((L + f32::AT_Q - 1) / f32::AT_Q, m->cfg.n_heads, n_slots);
+      const size_t smem = f32::attention_smem_floats(m->hd) * sizeof(float);
+      const float scale = 1.0f / sqrtf((float)m->hd);
+      if ((int64_t)grid.x * grid.y * grid.z <= 4 * m->num_sms)
+        LAUNCH_PDL(m, KC_ATTN, f32::attention_kernel<1>, grid, 32 * f32::AT_Q, smem, qkv, att, L, d, m->hd, scale);
+      else
+        LAUNCH_PDL(m, KC_ATTN, f32::attention_kernel<2>, grid, 16 * f32::AT_Q, smem, qkv, att, L, d, m->hd, scale);
     } else {
       const int warps = 4;
       dim3 grid((L + warps - 1) / warps, m->cfg.n_heads, n_slots);
@@ -2177,7 +2187,8 @@ static int load_impl(tf_model* m, const void* blob, size_t nbytes) {
     if (const char* e = getenv("TARFLOW_SEQ_PERSIST")) m->seq_use_persist = atoi(e) != 0;
   }
   if (c.dtype == 0) {
-    CU_OK(cudaFuncSetAttribute(f32::attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, f32::attention_smem_floats(128) * (int)sizeof(float)));
+    for (const auto kern : {f32::attention_kernel<1>, f32::attention_kernel<2>})
+      CU_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, f32::attention_smem_floats(128) * (int)sizeof(float)));
     if (const char* e = getenv("TARFLOW_SWEEP_GRAPH_ROWS")) m->sweep_graph_rows = atoll(e);
     if (const char* e = getenv("TARFLOW_GRAPHS")) m->use_graphs = atoi(e) != 0;
     CU_OK(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
