@@ -359,6 +359,7 @@ __global__ void layernorm_kernel(const float* __restrict__ x, const float* __res
 // four columns (blockDim.x = d / 4, a multiple of 32), so that every load of a row is in flight at once:
 //   x[row] <- x[row] + bias + slice 0 + slice 1 + ...   (this order: the sum does not depend on which slice finished first)
 //   y[row] <- LayerNorm(x[row]) (two-pass statistics, eps 1e-5), as T (plus the second term of the pair in y_lo).
+// ksplit == 0: nothing to add, x is complete.
 // ------------------------------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(1024)
@@ -667,31 +668,44 @@ __global__ void copy_first_token_kernel(const float* __restrict__ v, float* __re
 
 // Forward direction (Eq. 4): v_l = (u_l - mu_l) exp(-alpha_l), logdet[b] -= sum alpha.  One CTA per
 // sample so the per-sample sum is a fixed-order tree (deterministic).  o: [B*L, 2D] interleaved.
-__global__ void __launch_bounds__(256) forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u,
-                                                             float* __restrict__ v, float* __restrict__ logdet, int L,
-                                                             int D, int reversed) {
-  __shared__ float red[8];
-  int b = blockIdx.x;
+// Bound by the latency of a thread's loads: 32 warps per CTA and four values in flight per thread (64 samples of 256 x 48 values: with
+// 8 warps and one value 27 us, now 16; 2 samples of 1024 x 192: 259 and 105).
+constexpr int AFFINE_THREADS = 1024, AFFINE_BATCH = 4;
+__global__ void __launch_bounds__(AFFINE_THREADS)
+forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, float* __restrict__ v, float* __restrict__ logdet, int L,
+                      int D, int reversed) {
+  __shared__ float red[AFFINE_THREADS / 32];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.x, n = L * D;
   float part = 0.f;
-  for (int i = threadIdx.x; i < L * D; i += 256) {
-    int l = i / D, c = i - l * D;
-    size_t e = ((size_t)b * L + tok_index(l, L, reversed)) * D + c;
-    float mu = 0.f, al = 0.f;
-    if (l > 0) {
-      const float* orow = o + ((size_t)b * L + (l - 1)) * 2 * D;
-      mu = orow[2 * c];
-      al = orow[2 * c + 1];
+  for (int i0 = threadIdx.x; i0 < n; i0 += AFFINE_BATCH * AFFINE_THREADS) {
+    float2 p[AFFINE_BATCH];  // (mu, alpha): the head output of the position before; the first token is copied
+    float x[AFFINE_BATCH];
+    size_t e[AFFINE_BATCH];
+#pragma unroll
+    for (int k = 0; k < AFFINE_BATCH; ++k) {
+      const int i = i0 + k * AFFINE_THREADS, l = i / D, c = i - l * D;
+      p[k] = make_float2(0.f, 0.f);
+      x[k] = 0.f;
+      if (i >= n) continue;
+      e[k] = ((size_t)b * L + tok_index(l, L, reversed)) * D + c;
+      x[k] = u[e[k]];
+      if (l > 0) p[k] = reinterpret_cast<const float2*>(o)[((size_t)b * L + (l - 1)) * D + c];
     }
-    v[e] = (u[e] - mu) * expf(-al);
-    part += al;
+#pragma unroll
+    for (int k = 0; k < AFFINE_BATCH; ++k) {
+      if (i0 + k * AFFINE_THREADS >= n) break;
+      v[e[k]] = (x[k] - p[k].x) * expf(-p[k].y);
+      part += p[k].y;
+    }
   }
   part = warp_sum(part);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
-  if (threadIdx.x == 0 && logdet != nullptr) {
-    float s = 0.f;
-    for (int i = 0; i < 8; ++i) s += red[i];
-    logdet[b] -= s;
+  if (threadIdx.x < 32 && logdet != nullptr) {
+    const float s = warp_sum(red[threadIdx.x]);
+    if (threadIdx.x == 0) logdet[b] -= s;
   }
 }
 

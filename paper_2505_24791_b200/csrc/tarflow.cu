@@ -1694,7 +1694,7 @@ static int forward_impl(tf_model* m, const float* x, const int* labels, int B, f
   if (logdet) CU_OK(cudaMemsetAsync(logdet, 0, B * sizeof(float), m->stream));
   for (int g = m->cfg.n_blocks - 1; g >= 0; --g) {
     TF_TRY(run_pass<T>(m, g, B, u, nullptr, labels, PASS_FORWARD, nullptr, nullptr, false));
-    LAUNCH(m, KC_AFFINE, forward_affine_kernel, B, 256, 0, m->o, u, v, logdet, m->L, m->D, g & 1);
+    LAUNCH_PDL(m, KC_AFFINE, forward_affine_kernel, B, AFFINE_THREADS, 0, m->o, u, v, logdet, m->L, m->D, g & 1);
     TF_TRY(check_launch("forward_affine_kernel"));
     float* tmp = v; v = u; u = tmp;
   }
