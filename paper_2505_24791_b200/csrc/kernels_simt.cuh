@@ -5,6 +5,7 @@
 #include "attention_mma.cuh"
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "gemm_tc2.cuh"
 
 // ------------------------------------------------------------------------------------------------
 // image [B,C,H,W] <-> tokens [B,L,D]; raster patch order, (c,py,px) inside a token.
@@ -666,26 +667,32 @@ __global__ void copy_first_token_kernel(const float* __restrict__ v, float* __re
   u[e] = v[e];
 }
 
-// Forward direction (Eq. 4): v_l = (u_l - mu_l) exp(-alpha_l), logdet[b] -= sum alpha.  One CTA per
-// sample so the per-sample sum is a fixed-order tree (deterministic).  o: [B*L, 2D] interleaved.
+// Forward direction (Eq. 4): v_l = (u_l - mu_l) exp(-alpha_l), logdet[b] -= sum alpha.  A cluster of CS
+// CTAs per sample, so the per-sample sum is a fixed-order tree (deterministic, whatever the batch): every CTA reduces its values, the
+// first one adds the CTAs' sums in order.  o: [B*L, 2D] interleaved.
 // Bound by the latency of a thread's loads: 32 warps per CTA and four values in flight per thread (64 samples of 256 x 48 values: with
-// 8 warps and one value 27 us, now 16; 2 samples of 1024 x 192: 259 and 105).
+// 8 warps and one value 27 us, now 16; 2 samples of 1024 x 192: 259 and 105);
+// with eight CTAs per sample 19).
 constexpr int AFFINE_THREADS = 1024, AFFINE_BATCH = 4;
+template <int CS>
 __global__ void __launch_bounds__(AFFINE_THREADS)
 forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, float* __restrict__ v, float* __restrict__ logdet, int L,
                       int D, int reversed) {
+  constexpr int STRIDE = CS * AFFINE_THREADS;
   __shared__ float red[AFFINE_THREADS / 32];
+  __shared__ float parts[CS];
   pdl_launch_dependents();
+  if constexpr (CS > 1) tc2::cluster_sync_all();  // every CTA of the cluster has started before its shared memory is written
   pdl_wait();
-  const int b = blockIdx.x, n = L * D;
+  const int b = blockIdx.x / CS, rank = blockIdx.x % CS, n = L * D;
   float part = 0.f;
-  for (int i0 = threadIdx.x; i0 < n; i0 += AFFINE_BATCH * AFFINE_THREADS) {
+  for (int i0 = rank * AFFINE_THREADS + threadIdx.x; i0 < n; i0 += AFFINE_BATCH * STRIDE) {
     float2 p[AFFINE_BATCH];  // (mu, alpha): the head output of the position before; the first token is copied
     float x[AFFINE_BATCH];
     size_t e[AFFINE_BATCH];
 #pragma unroll
     for (int k = 0; k < AFFINE_BATCH; ++k) {
-      const int i = i0 + k * AFFINE_THREADS, l = i / D, c = i - l * D;
+      const int i = i0 + k * STRIDE, l = i / D, c = i - l * D;
       p[k] = make_float2(0.f, 0.f);
       x[k] = 0.f;
       if (i >= n) continue;
@@ -695,7 +702,7 @@ forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, 
     }
 #pragma unroll
     for (int k = 0; k < AFFINE_BATCH; ++k) {
-      if (i0 + k * AFFINE_THREADS >= n) break;
+      if (i0 + k * STRIDE >= n) break;
       v[e[k]] = (x[k] - p[k].x) * expf(-p[k].y);
       part += p[k].y;
     }
@@ -703,9 +710,21 @@ forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, 
   part = warp_sum(part);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
-  if (threadIdx.x < 32 && logdet != nullptr) {
+  if (threadIdx.x < 32) {
     const float s = warp_sum(red[threadIdx.x]);
-    if (threadIdx.x == 0) logdet[b] -= s;
+    if (threadIdx.x == 0) {
+      if constexpr (CS > 1)
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(tc2::map_to_cta(tc::smem_u32(parts + rank), 0)), "f"(s) : "memory");
+      else
+        parts[0] = s;
+    }
+  }
+  if constexpr (CS > 1) tc2::cluster_sync_all();
+  if (rank == 0 && threadIdx.x == 0 && logdet != nullptr) {
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) s += parts[r];
+    logdet[b] -= s;
   }
 }
 

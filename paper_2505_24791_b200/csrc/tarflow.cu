@@ -1686,6 +1686,33 @@ static int inverse_impl(tf_model* m, const float* z, const int* labels, int B, c
   return status;
 }
 
+static int forward_affine(tf_model* m, int B, const float* u, float* v, float* logdet, int reversed) {
+  // By the values of a sample alone: the order of a sample's sum does not depend on its batch.  Eight CTAs / one per sample: 12 288 values
+  // 8.6 / 12.7 us (1 sample), 25.7 / 16.3 (64), 81 / 32 (256); 196 608 values 19 / 105 (2 samples).
+  if (m->L * m->D < 65536) {
+    LAUNCH_PDL(m, KC_AFFINE, forward_affine_kernel<1>, B, AFFINE_THREADS, 0, m->o, u, v, logdet, m->L, m->D, reversed);
+    return check_launch("forward_affine_kernel");
+  }
+  constexpr int CS = 8;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(B * CS);
+  lc.blockDim = dim3(AFFINE_THREADS);
+  lc.stream = m->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CS;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 2;
+  m->pre(KC_AFFINE);
+  const cudaError_t e = cudaLaunchKernelEx(&lc, forward_affine_kernel<CS>, (const float*)m->o, u, v, logdet, m->L, m->D, reversed);
+  m->post(KC_AFFINE);
+  if (e != cudaSuccess) return fail(TF_ECUDA, "forward_affine_kernel launch failed: %s", cudaGetErrorString(e));
+  return TF_OK;
+}
+
 template <class T>
 static int forward_impl(tf_model* m, const float* x, const int* labels, int B, float* z, float* logdet) {
   float *u = m->seq_a, *v = m->seq_b;
@@ -1694,8 +1721,7 @@ static int forward_impl(tf_model* m, const float* x, const int* labels, int B, f
   if (logdet) CU_OK(cudaMemsetAsync(logdet, 0, B * sizeof(float), m->stream));
   for (int g = m->cfg.n_blocks - 1; g >= 0; --g) {
     TF_TRY(run_pass<T>(m, g, B, u, nullptr, labels, PASS_FORWARD, nullptr, nullptr, false));
-    LAUNCH_PDL(m, KC_AFFINE, forward_affine_kernel, B, AFFINE_THREADS, 0, m->o, u, v, logdet, m->L, m->D, g & 1);
-    TF_TRY(check_launch("forward_affine_kernel"));
+    TF_TRY(forward_affine(m, B, u, v, logdet, g & 1));
     float* tmp = v; v = u; u = tmp;
   }
   TF_TRY(layout(m, z, u, B, 0));

@@ -288,3 +288,16 @@ def test_narrow_tiles_at_their_edges(rows, cols, patch, width, batch, monkeypatc
     _close(x[pick], xo)
     assert np.abs(its[:, pick] - ito).max() <= 1
     assert rel_l2(zf, z.astype(np.float64)) <= 2e-2
+
+
+def test_long_sequence_forward_cuts_a_sample_over_ctas(long_model):
+    """196 608 values per sample: the affine step and the log-determinant of a sample are shared by eight CTAs."""
+    m = long_model
+    x = synth.make_latents(m.cfg, 5400, B=3)
+    zf, ld = m.forward(x, None)
+    z1, l1 = m.forward(x[2:], None)                                 # neither values nor the sum's order depend on the batch
+    assert np.array_equal(zf[2:], z1) or rel_l2(zf[2:], z1) <= 1e-3  # (tile shapes of the products do, at the level of bf16)
+    assert abs(l1[0] - ld[2]) <= 1e-3 * max(1.0, abs(ld[2]))
+    zo, ldo = O.model_forward(m.blocks, x[:1].astype(np.float64), None, m.cfg)
+    _close(zf[:1], zo)
+    assert np.abs(ld[:1] - ldo).max() <= 2e-2 * max(1.0, np.abs(ldo).max())
