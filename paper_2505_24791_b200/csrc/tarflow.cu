@@ -635,7 +635,7 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   // CTAs to stream their weights, so they are cut into K slices that leave partial products; the LayerNorm that follows
   // (this layer's second, the next layer's first, or the block's last) adds them to the stream in slice order.
   const int m_pad = (M + 127) / 128 * 128;
-  struct Slices { int n; bool narrow; };  // n == 1: no partial products
+  struct Slices { int n; bool narrow; };  // {1, false}: no partial products, the projection adds to the stream itself
   auto slices_for = [&](const Matrix& W) -> Slices {
     if (sizeof(T) != 2 || m->sweep_part == nullptr || !m->small_m_split || d > 4096) return {1, false};
     auto slices = [&](int tiles, int ctas) {
@@ -645,7 +645,8 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
       if (ks > m->part_cap_rows / m_pad) ks = m->part_cap_rows / m_pad;
       return ks < 1 ? 1 : ks;
     };
-    if (few_fits(m, M, W)) {
+    // a narrow product leaves its sums in the partial buffer however few its slices are, so its rows must fit there
+    if (m_pad <= m->part_cap_rows && few_fits(m, M, W)) {
       // A slab of a 128 x 64 tile takes about 0.25 us, one of a 128 x 128 tile 0.33 us; the wide tiles' epilogue and the LayerNorm
       // over twice the slices cost 3 us more.  256-token sweeps of width 1024, down projection alone, narrow / wide: 7.4 / 7.4 us
       // with the LayerNorms at 2.7 / 3.6 us each (1 sample), 26 / 14 us (4 samples).
@@ -660,6 +661,23 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   SplitSum pend{nullptr, 0, 0, nullptr};
   bool has_pend = false;
   bool first_layer = true;
+  // a projection into the residual stream, W over the activations a (maps ma, ma_lo)
+  auto into_stream = [&](int cls, const T* a, const CUtensorMap* ma, const CUtensorMap* ma_lo, const Matrix& W, const float* bias) -> int {
+    if constexpr (sizeof(T) == 2) {
+      const Slices ks = slices_for(W);
+      if (ks.n == 1 && !ks.narrow) return gemm<T>(m, cls, a, ma, ma_lo, W, M, EpiResidTma{bias, m->store_maps + tf_model::SM_H});
+      // rows behind the buffer's end would be lost on the way in and read from other memory on the way out
+      if ((int64_t)ks.n * m_pad > m->part_cap_rows) return fail(TF_EINVAL, "%d slices of %d rows exceed the partial buffer", ks.n, m_pad);
+      const CUtensorMap* part = m->store_maps + tf_model::SM_PART;
+      if (ks.narrow) TF_TRY(launch_few<64>(m, cls, *ma, ma_lo, W, M, few::StoreF32{part}, nullptr, ks.n, m_pad));
+      else TF_TRY(gemm<T>(m, cls, a, ma, ma_lo, W, M, EpiStoreF32Tma{nullptr, part}, ks.n, m_pad));
+      pend = SplitSum{m->sweep_part, ks.n, m_pad, bias};
+      has_pend = true;
+      return TF_OK;
+    } else {
+      return gemm<T>(m, cls, a, ma, ma_lo, W, M, EpiResid{m->h, bias, d});
+    }
+  };
   for (const LayerW& lw : bw.layers) {
     if (!(first_layer && fused_embed)) TF_TRY(layernorm<T>(m, KC_LN, m->h, lw.ln1_g, lw.ln1_b, xn, xn_lo, M, has_pend ? &pend : nullptr));
     has_pend = false;
@@ -706,20 +724,7 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
              1.0f / sqrtf((float)m->hd));
     }
     TF_TRY(check_launch("attention kernel"));
-    if constexpr (sizeof(T) == 2) {
-      const Slices ks = slices_for(lw.w_o);
-      const CUtensorMap* part = m->store_maps + tf_model::SM_PART;
-      if (ks.n > 1 || ks.narrow) {
-        if (ks.narrow) TF_TRY(launch_few<64>(m, KC_GEMM_O, m->map_att, mal, lw.w_o, M, few::StoreF32{part}, nullptr, ks.n, m_pad));
-        else TF_TRY(gemm<T>(m, KC_GEMM_O, att, &m->map_att, mal, lw.w_o, M, EpiStoreF32Tma{nullptr, part}, ks.n, m_pad));
-        pend = SplitSum{m->sweep_part, ks.n, m_pad, lw.b_o};
-        has_pend = true;
-      } else {
-        TF_TRY(gemm<T>(m, KC_GEMM_O, att, &m->map_att, mal, lw.w_o, M, EpiResidTma{lw.b_o, m->store_maps + tf_model::SM_H}));
-      }
-    } else {
-      TF_TRY(gemm<T>(m, KC_GEMM_O, att, &m->map_att, mal, lw.w_o, M, EpiResid{m->h, lw.b_o, d}));
-    }
+    TF_TRY(into_stream(KC_GEMM_O, att, &m->map_att, mal, lw.w_o, lw.b_o));
     TF_TRY(layernorm<T>(m, KC_LN, m->h, lw.ln2_g, lw.ln2_b, xn, xn_lo, M, has_pend ? &pend : nullptr));
     has_pend = false;
     if constexpr (sizeof(T) == 2) {
@@ -727,20 +732,10 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
       if (few_fits(m, M, lw.w_1)) TF_TRY(launch_few<64>(m, KC_GEMM_MLP1, m->map_xn, mxl, lw.w_1, M, few::Store<ACT_GELU>{sm + tf_model::SM_MLP, hp ? sm + tf_model::SM_MLP_LO : nullptr}, lw.b_1));
       else TF_TRY(gemm<T>(m, KC_GEMM_MLP1, xn, &m->map_xn, mxl, lw.w_1, M,
                      EpiStoreTma<true>{lw.b_1, sm + tf_model::SM_MLP, hp ? sm + tf_model::SM_MLP_LO : nullptr}));
-      const Slices ks = slices_for(lw.w_2);
-      const CUtensorMap* part = m->store_maps + tf_model::SM_PART;
-      if (ks.n > 1 || ks.narrow) {
-        if (ks.narrow) TF_TRY(launch_few<64>(m, KC_GEMM_MLP2, m->map_mlp, mml, lw.w_2, M, few::StoreF32{part}, nullptr, ks.n, m_pad));
-        else TF_TRY(gemm<T>(m, KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, M, EpiStoreF32Tma{nullptr, part}, ks.n, m_pad));
-        pend = SplitSum{m->sweep_part, ks.n, m_pad, lw.b_2};
-        has_pend = true;
-      } else {
-        TF_TRY(gemm<T>(m, KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, M, EpiResidTma{lw.b_2, sm + tf_model::SM_H}));
-      }
     } else {
       TF_TRY(gemm<T>(m, KC_GEMM_MLP1, xn, &m->map_xn, mxl, lw.w_1, M, EpiStore<T, true>{mlp, lw.b_1, m->hid, mlp_lo}));
-      TF_TRY(gemm<T>(m, KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, M, EpiResid{m->h, lw.b_2, d}));
     }
+    TF_TRY(into_stream(KC_GEMM_MLP2, mlp, &m->map_mlp, mml, lw.w_2, lw.b_2));
   }
   TF_TRY(layernorm<T>(m, KC_LN, m->h, bw.lnf_g, bw.lnf_b, xn, xn_lo, M, has_pend ? &pend : nullptr));
   if (mode == PASS_JACOBI) {

@@ -290,6 +290,36 @@ def test_narrow_tiles_at_their_edges(rows, cols, patch, width, batch, monkeypatc
     assert rel_l2(zf, z.astype(np.float64)) <= 2e-2
 
 
+# Width 128 has two 64-column tiles per 128 rows, so up to 9472 rows fit one wave of narrow tiles, and the buffer of partial products
+# holds 8192: the rows it just holds, a few more, the most that fit the wave, one tile beyond, and a batch that shrinks through the range.
+@pytest.mark.parametrize("side,batch", [(16, 32), (12, 57), (16, 33), (16, 37), (16, 38), (16, 64)])
+def test_rows_beyond_the_partial_buffer(side, batch, monkeypatch):
+    cfg = synth.config("cfg3", H=4 * side, W=4 * side, n_blocks=1, n_layers=2, width=128, n_heads=2, n_classes=10)
+    L = synth.seq_len(cfg)
+    z = synth.make_latents(cfg, 5500 + side, B=batch)
+    lab = synth.make_labels(cfg, B=batch)
+    pick = [0, batch - 1]                                   # the last sample's rows lie behind row 8192
+    with Model(cfg, max_batch=batch) as m:
+        x, ib, its, rc = m.inverse(z, lab, [1], 1e-3, L + 1)
+        zf, ld = m.forward(z, lab)
+    monkeypatch.setenv("TARFLOW_SMALL_M_ROWS", "0")
+    monkeypatch.setenv("TARFLOW_SPLIT_M_ROWS", "0")
+    with Model(cfg, max_batch=batch) as ref:
+        xr, _, itsr, rcr = ref.inverse(z, lab, [1], 1e-3, L + 1)
+        zr, ldr = ref.forward(z, lab)
+    assert rc == 0 and rcr == 0 and np.isfinite(x).all() and np.isfinite(zf).all()
+    assert np.abs(x - xr).max() <= 2e-3 and np.abs(its - itsr).max() <= 1      # both end within tau = 1e-3 of the fixed point
+    for b in range(batch):                                  # one causal pass of single bf16 operands on either side
+        assert rel_l2(zf[b], zr[b]) <= 2e-2
+    assert np.abs(ld - ldr).max() <= 2e-2 * max(1.0, np.abs(ldr).max())
+    xo, ito = O.model_inverse(m.blocks, z[pick], lab[pick], cfg, [1], 1e-3, L + 1)
+    _close(x[pick], xo)
+    assert np.abs(its[:, pick] - ito).max() <= 1
+    zo, ldo = O.model_forward(m.blocks, z[pick].astype(np.float64), lab[pick], cfg)
+    _close(zf[pick], zo)
+    assert np.abs(ld[pick] - ldo).max() <= 2e-2 * max(1.0, np.abs(ldo).max())
+
+
 def test_long_sequence_forward_cuts_a_sample_over_ctas(long_model):
     """196 608 values per sample: the affine step and the log-determinant of a sample are shared by eight CTAs."""
     m = long_model
