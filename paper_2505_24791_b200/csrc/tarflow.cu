@@ -645,18 +645,22 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
       if (ks > m->part_cap_rows / m_pad) ks = m->part_cap_rows / m_pad;
       return ks < 1 ? 1 : ks;
     };
-    // a narrow product leaves its sums in the partial buffer however few its slices are, so its rows must fit there
-    if (m_pad <= m->part_cap_rows && few_fits(m, M, W)) {
-      // A slab of a 128 x 64 tile takes about 0.25 us, one of a 128 x 128 tile 0.33 us; the wide tiles' epilogue and the LayerNorm
-      // over twice the slices cost 3 us more.  256-token sweeps of width 1024, down projection alone, narrow / wide: 7.4 / 7.4 us
-      // with the LayerNorms at 2.7 / 3.6 us each (1 sample), 26 / 14 us (4 samples).
-      const int n = slices((m_pad / 128) * (d / 64), m->num_sms), w = slices((m_pad / 128) * (d / 128), m->num_sms), slabs = W.K / tc::BK;
-      if (M > m->small_m_rows || slabs * 0.25f / n <= slabs * 0.33f / w + 3.f) return {n, true};
-    }
-    if (M <= m->small_m_rows) return {slices((m_pad / 128) * (d / 128), m->num_sms), false};  // 128 x 128 tiles
-    if (M <= m->split_m_rows && m->use_pair_gemm && d % 256 == 0 && M >= 256)
-      return {slices((M + 255) / 256 * (d / 256), m->num_sms / 2), false};                     // pair tiles
-    return {1, false};
+    Slices wide = {1, false};
+    const bool single = M <= m->small_m_rows, pairs = !single && m->use_pair_gemm && d % 256 == 0 && M >= 256;
+    if (single) wide.n = slices((m_pad / 128) * (d / 128), m->num_sms);                                       // 128 x 128 tiles
+    else if (pairs && M <= m->split_m_rows) wide.n = slices((M + 255) / 256 * (d / 256), m->num_sms / 2);     // pair tiles
+    // A narrow product leaves its sums in the partial buffer however few its slices are: its rows must fit there, and the LayerNorm
+    // reads them beside the stream.  Against 128 x 128 tiles that reduce into the stream this pays up to 4096 rows (width 128, narrow /
+    // wide: sweep 180 / 178 us, two-term 212 / 223 at 4096 rows, 205 / 199 and 242 / 236 at 5120, 241 / 208 and 290 / 256 at 8192).
+    if (m_pad > m->part_cap_rows || !few_fits(m, M, W) || (!single && !pairs && M > 4096)) return wide;
+    // Microseconds of a tile's k slabs, plus what the other form costs on top: a further slice for the LayerNorm, a longer epilogue.
+    // Per layer at four layers, narrow / wide: down projection, 512 rows of width 1024 8.0 / 6.6 (measured: wide 2.2 faster), 256 rows
+    // 4.0 / 4.9 (narrow 0.9 faster), 1280 rows of width 768 12 / 8.1 (wide 5.2 faster), of width 256 1.3 / 4.6 (narrow 4.6 faster);
+    // out-projection, 1024 rows of width 1024 4.0 / 3.5 (wide 0.5 faster), 1280 rows of width 512 2.0 / 4.3 (narrow 2.2 faster).
+    const int n = slices((m_pad / 128) * (d / 64), m->num_sms);
+    const float slabs = (float)(W.K / tc::BK), more = 0.45f * (wide.n - n);
+    if (slabs * 0.25f / n > slabs * (pairs ? 0.38f : 0.33f) / wide.n + (pairs ? 2.2f : 0.45f) + more) return wide;
+    return {n, true};
   };
   SplitSum pend{nullptr, 0, 0, nullptr};
   bool has_pend = false;

@@ -264,9 +264,11 @@ def test_few_row_sweeps_agree_with_the_one_shape_path_and_the_oracle(name, monke
 
 # H x W patches of 4 x 4 x 3 values (2 x 2 x 3 with D = 12), width, batch: fewer rows than a tile; one row beyond whole tiles and slices of one k
 # slab; 65 x 13 rows in nine tiles; the largest row count whose head still fits one wave of 32-column tiles, narrow and wide
-# products mixed; a head of 24 columns in a tile of 32
+# products mixed; a head of 24 columns in a tile of 32; the most rows of width 128 with narrow residual projections and a few more;
+# narrow ones beside pair tiles that are no longer cut in K; the down projection wide, the out-projection narrow (pair and single tiles)
 @pytest.mark.parametrize("rows,cols,patch,width,batch", [(5, 5, 4, 128, 1), (3, 43, 4, 128, 3), (9, 9, 4, 256, 13), (16, 16, 4, 512, 24),
-                                                         (16, 16, 2, 512, 4)])
+                                                         (16, 16, 2, 512, 4), (16, 16, 4, 128, 16), (17, 16, 4, 128, 16),
+                                                         (16, 16, 4, 256, 18), (16, 16, 4, 512, 5), (16, 16, 4, 1024, 2)])
 def test_narrow_tiles_at_their_edges(rows, cols, patch, width, batch, monkeypatch):
     cfg = synth.config("cfg3", H=patch * rows, W=patch * cols, patch=patch, n_blocks=1, n_layers=2, width=width, n_heads=width // 64,
                        n_classes=10)
