@@ -15,6 +15,8 @@
 // take 1.8 us for the exchange and save 1.2 us of loads, eight take 2.7 us.
 // Every wait is bounded as in gemm_tc.cuh.
 #pragma once
+#include <type_traits>
+
 #include "gemm_tc.cuh"
 
 namespace few {
@@ -127,8 +129,10 @@ struct StoreF32 {  // fp32 sums (a K slice's go part_rows rows further down per 
   }
 };
 
-// Algorithm 1's update line, as EpiHeadUpdate does it: columns (2c, 2c + 1) = (mu~_c, alpha~_c); D % 4 == 0.
+// Algorithm 1's update line, as EpiHeadUpdate does it: columns (2c, 2c + 1) = (mu~_c, alpha~_c).  V values per access (4 or 2), D % V == 0.
+template <int V>
 struct HeadUpdate {
+  using Vec = std::conditional_t<V == 4, float4, float2>;
   static constexpr int kOld = 16;  // eight values of the iterate, eight of the block's input
   const float* v;
   float *u, *maxdiff;
@@ -148,12 +152,15 @@ struct HeadUpdate {
     bool upd;
     const size_t e = element(row, sample(row), upd);
 #pragma unroll
-    for (int j = 0; j < 8; j += 4) {
+    for (int j = 0; j < 8; j += V) {
       const int c = col0 / 2 + j;
       if (c < D) {
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(u + e + c)), y = __ldcg(reinterpret_cast<const float4*>(v + e + c));
-        old[j] = x.x; old[j + 1] = x.y; old[j + 2] = x.z; old[j + 3] = x.w;
-        old[8 + j] = y.x; old[8 + j + 1] = y.y; old[8 + j + 2] = y.z; old[8 + j + 3] = y.w;
+        const Vec x = __ldcg(reinterpret_cast<const Vec*>(u + e + c)), y = __ldcg(reinterpret_cast<const Vec*>(v + e + c));
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+          old[j + i] = reinterpret_cast<const float*>(&x)[i];
+          old[8 + j + i] = reinterpret_cast<const float*>(&y)[i];
+        }
       }
     }
   }
@@ -166,19 +173,19 @@ struct HeadUpdate {
       b = sample(row0 + w.lane);
       const size_t e = element(row0 + w.lane, b, upd);
 #pragma unroll
-      for (int j = 0; j < 8; j += 4) {
+      for (int j = 0; j < 8; j += V) {
         const int c = col0 / 2 + j;
         if (c < D) {
-          float nw[4];
+          Vec nw;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
+          for (int i = 0; i < V; ++i) {
             const int k = j + i;
             const float mu = x[2 * k] + bias[2 * k], al = x[2 * k + 1] + bias[2 * k + 1], vv = old[8 + k];
-            nw[i] = upd ? fmaf(vv, expf(al), mu) : vv;
-            const float df = fabsf(nw[i] - old[k]);
+            const float now = upd ? fmaf(vv, expf(al), mu) : vv, df = fabsf(now - old[k]);
+            reinterpret_cast<float*>(&nw)[i] = now;
             m = (df > m || df != df) ? df : m;
           }
-          *reinterpret_cast<float4*>(u + e + c) = make_float4(nw[0], nw[1], nw[2], nw[3]);
+          *reinterpret_cast<Vec*>(u + e + c) = nw;
         }
       }
     }

@@ -743,9 +743,11 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   }
   TF_TRY(layernorm<T>(m, KC_LN, m->h, bw.lnf_g, bw.lnf_b, xn, xn_lo, M, has_pend ? &pend : nullptr));
   if (mode == PASS_JACOBI) {
-    if (sizeof(T) == 2 && few_fits(m, M, bw.w_out) && D % 4 == 0) {
-      if constexpr (sizeof(T) == 2)
-        TF_TRY(launch_few<32>(m, KC_GEMM_HEAD_UPDATE, m->map_xn, mxl, bw.w_out, M, few::HeadUpdate{v, u_upd, m->maxdiff, idx, L, D, rev}, bw.b_out));
+    if (sizeof(T) == 2 && few_fits(m, M, bw.w_out) && D % 2 == 0) {
+      if constexpr (sizeof(T) == 2) {
+        if (D % 4 == 0) TF_TRY(launch_few<32>(m, KC_GEMM_HEAD_UPDATE, m->map_xn, mxl, bw.w_out, M, few::HeadUpdate<4>{v, u_upd, m->maxdiff, idx, L, D, rev}, bw.b_out));
+        else TF_TRY(launch_few<32>(m, KC_GEMM_HEAD_UPDATE, m->map_xn, mxl, bw.w_out, M, few::HeadUpdate<2>{v, u_upd, m->maxdiff, idx, L, D, rev}, bw.b_out));
+      }
     } else {
       EpiHeadUpdate epi{v, u_upd, m->maxdiff, idx, bw.b_out, L, D, rev};
       TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, xn, &m->map_xn, mxl, bw.w_out, M, epi));

@@ -262,16 +262,18 @@ def test_few_row_sweeps_agree_with_the_one_shape_path_and_the_oracle(name, monke
                 assert rel_l2(zf, zo) <= 2e-2 and np.abs(ld - ldo).max() <= 2e-2 * max(1.0, np.abs(ldo).max())
 
 
-# H x W patches of 4 x 4 x 3 values (2 x 2 x 3 with D = 12), width, batch: fewer rows than a tile; one row beyond whole tiles and slices of one k
+# Channels, H x W patches of P x P of them, width, batch: fewer rows than a tile; one row beyond whole tiles and slices of one k
 # slab; 65 x 13 rows in nine tiles; the largest row count whose head still fits one wave of 32-column tiles, narrow and wide
 # products mixed; a head of 24 columns in a tile of 32; the most rows of width 128 with narrow residual projections and a few more;
-# narrow ones beside pair tiles that are no longer cut in K; the down projection wide, the out-projection narrow (pair and single tiles)
-@pytest.mark.parametrize("rows,cols,patch,width,batch", [(5, 5, 4, 128, 1), (3, 43, 4, 128, 3), (9, 9, 4, 256, 13), (16, 16, 4, 512, 24),
-                                                         (16, 16, 2, 512, 4), (16, 16, 4, 128, 16), (17, 16, 4, 128, 16),
-                                                         (16, 16, 4, 256, 18), (16, 16, 4, 512, 5), (16, 16, 4, 1024, 2)])
-def test_narrow_tiles_at_their_edges(rows, cols, patch, width, batch, monkeypatch):
-    cfg = synth.config("cfg3", H=patch * rows, W=patch * cols, patch=patch, n_blocks=1, n_layers=2, width=width, n_heads=width // 64,
-                       n_classes=10)
+# narrow ones beside pair tiles that are no longer cut in K; the down projection wide, the out-projection narrow (pair and single tiles);
+# tokens of 2, 6 and 18 values (two per access; a tile of four columns, one cut short, two tiles), a head of 14 columns (odd: general epilogue)
+@pytest.mark.parametrize("channels,rows,cols,patch,width,batch", [
+    (3, 5, 5, 4, 128, 1), (3, 3, 43, 4, 128, 3), (3, 9, 9, 4, 256, 13), (3, 16, 16, 4, 512, 24), (3, 16, 16, 2, 512, 4), (3, 16, 16, 4, 128, 16),
+    (3, 17, 16, 4, 128, 16), (3, 16, 16, 4, 256, 18), (3, 16, 16, 4, 512, 5), (3, 16, 16, 4, 1024, 2), (2, 16, 16, 1, 128, 1),
+    (6, 9, 13, 1, 256, 3), (18, 16, 16, 1, 128, 5), (7, 9, 9, 1, 128, 2)])
+def test_narrow_tiles_at_their_edges(channels, rows, cols, patch, width, batch, monkeypatch):
+    cfg = synth.config("cfg3", C=channels, H=patch * rows, W=patch * cols, patch=patch, n_blocks=1, n_layers=2, width=width,
+                       n_heads=width // 64, n_classes=10)
     L = synth.seq_len(cfg)
     z = synth.make_latents(cfg, 5300 + rows, B=batch)
     lab = synth.make_labels(cfg, B=batch)
