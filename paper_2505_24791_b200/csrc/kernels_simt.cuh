@@ -670,15 +670,19 @@ __global__ void copy_first_token_kernel(const float* __restrict__ v, float* __re
 // Forward direction (Eq. 4): v_l = (u_l - mu_l) exp(-alpha_l), logdet[b] -= sum alpha.  A cluster of CS
 // CTAs per sample, so the per-sample sum is a fixed-order tree (deterministic, whatever the batch): every CTA reduces its values, the
 // first one adds the CTAs' sums in order.  o: [B*L, 2D] interleaved.
-// Bound by the latency of a thread's loads: 32 warps per CTA and four values in flight per thread (64 samples of 256 x 48 values: with
-// 8 warps and one value 27 us, now 16; 2 samples of 1024 x 192: 259 and 105);
-// with eight CTAs per sample 19).
+// Bound by the latency of a thread's loads: four values in flight per thread and up to 32 warps per CTA (64 samples of 256 x 48 values:
+// 27 us with 8 warps and one value, 16 with 32 and four; 2 samples of 1024 x 192: 259 us with one CTA of 8 warps, 105 with one
+// of 32, 19 with eight CTAs).  Small samples get no more threads than values / 4 (affine_threads), so that more of them are resident.
 constexpr int AFFINE_THREADS = 1024, AFFINE_BATCH = 4;
+__host__ inline int affine_threads(int values) {  // of the single CTA of a sample
+  const int t = (values + 32 * AFFINE_BATCH - 1) / (32 * AFFINE_BATCH) * 32;
+  return t < AFFINE_THREADS ? t : AFFINE_THREADS;
+}
 template <int CS>
 __global__ void __launch_bounds__(AFFINE_THREADS)
 forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, float* __restrict__ v, float* __restrict__ logdet, int L,
                       int D, int reversed) {
-  constexpr int STRIDE = CS * AFFINE_THREADS;
+  const int stride = CS * blockDim.x;
   __shared__ float red[AFFINE_THREADS / 32];
   __shared__ float parts[CS];
   pdl_launch_dependents();
@@ -686,13 +690,13 @@ forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, 
   pdl_wait();
   const int b = blockIdx.x / CS, rank = blockIdx.x % CS, n = L * D;
   float part = 0.f;
-  for (int i0 = rank * AFFINE_THREADS + threadIdx.x; i0 < n; i0 += AFFINE_BATCH * STRIDE) {
+  for (int i0 = rank * blockDim.x + threadIdx.x; i0 < n; i0 += AFFINE_BATCH * stride) {
     float2 p[AFFINE_BATCH];  // (mu, alpha): the head output of the position before; the first token is copied
     float x[AFFINE_BATCH];
     size_t e[AFFINE_BATCH];
 #pragma unroll
     for (int k = 0; k < AFFINE_BATCH; ++k) {
-      const int i = i0 + k * STRIDE, l = i / D, c = i - l * D;
+      const int i = i0 + k * stride, l = i / D, c = i - l * D;
       p[k] = make_float2(0.f, 0.f);
       x[k] = 0.f;
       if (i >= n) continue;
@@ -702,7 +706,7 @@ forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, 
     }
 #pragma unroll
     for (int k = 0; k < AFFINE_BATCH; ++k) {
-      if (i0 + k * STRIDE >= n) break;
+      if (i0 + k * stride >= n) break;
       v[e[k]] = (x[k] - p[k].x) * expf(-p[k].y);
       part += p[k].y;
     }
@@ -711,7 +715,7 @@ forward_affine_kernel(const float* __restrict__ o, const float* __restrict__ u, 
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
   if (threadIdx.x < 32) {
-    const float s = warp_sum(red[threadIdx.x]);
+    const float s = warp_sum(threadIdx.x < blockDim.x >> 5 ? red[threadIdx.x] : 0.f);
     if (threadIdx.x == 0) {
       if constexpr (CS > 1)
         asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(tc2::map_to_cta(tc::smem_u32(parts + rank), 0)), "f"(s) : "memory");

@@ -1696,7 +1696,7 @@ static int forward_affine(tf_model* m, int B, const float* u, float* v, float* l
   // By the values of a sample alone: the order of a sample's sum does not depend on its batch.  Eight CTAs / one per sample: 12 288 values
   // 8.6 / 12.7 us (1 sample), 25.7 / 16.3 (64), 81 / 32 (256); 196 608 values 19 / 105 (2 samples).
   if (m->L * m->D < 65536) {
-    LAUNCH_PDL(m, KC_AFFINE, forward_affine_kernel<1>, B, AFFINE_THREADS, 0, m->o, u, v, logdet, m->L, m->D, reversed);
+    LAUNCH_PDL(m, KC_AFFINE, forward_affine_kernel<1>, B, affine_threads(m->L * m->D), 0, m->o, u, v, logdet, m->L, m->D, reversed);
     return check_launch("forward_affine_kernel");
   }
   constexpr int CS = 8;

@@ -335,3 +335,24 @@ def test_long_sequence_forward_cuts_a_sample_over_ctas(long_model):
     zo, ldo = O.model_forward(m.blocks, x[:1].astype(np.float64), None, m.cfg)
     _close(zf[:1], zo)
     assert np.abs(ld[:1] - ldo).max() <= 2e-2 * max(1.0, np.abs(ldo).max())
+
+
+# Values per sample: fewer than a warp, fewer than a warp's four per thread, not a multiple of the threads, exactly four for each of 1024
+# threads and a few more, the largest with one CTA per sample, eight CTAs with uneven shares.
+@pytest.mark.parametrize("rows,cols,channels,patch", [(4, 4, 1, 1), (5, 5, 1, 2), (7, 9, 3, 2), (16, 16, 1, 4), (17, 16, 1, 4), (21, 65, 3, 4),
+                                                      (23, 23, 3, 8)])
+def test_forward_affine_step_does_not_depend_on_the_batch(rows, cols, channels, patch):
+    """The order of a sample's log-determinant sum follows from its own size: bit-identical alone and in a batch (fp32
+    engine, whose products sum in an order of their own that no shape changes)."""
+    cfg = synth.micro_config(C=channels, H=patch * rows, W=patch * cols, patch=patch, n_blocks=2, n_layers=1, width=32, n_heads=1, mlp_ratio=2)
+    B = 5
+    with Model(cfg, max_batch=B) as m:
+        x = synth.make_latents(cfg, 5600 + rows, B=B)
+        zf, ld = m.forward(x, None)
+        for b in (0, B - 1):
+            z1, l1 = m.forward(x[b:b + 1], None)
+            assert np.array_equal(zf[b:b + 1], z1) and np.array_equal(ld[b:b + 1], l1)
+        zo, ldo = O.model_forward(m.blocks, x[:1].astype(np.float64), None, cfg)
+        assert rel_l2(zf[:1], zo) <= 1e-5
+        # n terms with rounding errors of their own (std about 1e-6 each: fp32 sums of 32 to 64 products)
+        assert np.abs(ld[:1] - ldo).max() <= 1e-5 * max(1.0, np.sqrt(zo.size))
