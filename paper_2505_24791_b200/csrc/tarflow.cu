@@ -618,8 +618,9 @@ static int run_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
     // Fewer CTAs of sixteen rows than SMs: four rows each instead, as long as fetching the weights four times as often costs less than
     // it saves.  Sweep of four layers, four / sixteen rows: width 256 154 / 164 us (1280 rows), 180 / 178 (2304), width 128 144 / 153 (2304),
     // width 512 213 / 216 (1280) and 251 / 245 (2304); width 1024 with 48 values per token 323 / 324 (1280) and 411 / 400 (2304), with
-    // 192 values 361 / 349 (1280) and 486 / 443 (2304).
-    const int few_rows = d <= 256 ? 16 * m->num_sms : (int64_t)D * d <= 48 * 1024 ? 10 * m->num_sms : 1024;
+    // 192 values 361 / 349 (1280) and 486 / 443 (2304), with 12 values 321 / 326 (1536) and 359 / 361 (1792); width 384 183 / 187 (1536).
+    const int64_t weights = (int64_t)D * d;
+    const int few_rows = d <= 256 ? 16 * m->num_sms : weights <= 24 * 1024 ? 12 * m->num_sms : weights <= 48 * 1024 ? 10 * m->num_sms : 1024;
     const bool few = M <= few_rows;
     const int R = few ? 4 : 16, threads = ((d / 4 + 31) / 32) * 32;
     int cc = EMBED_WEIGHT_BYTES / (2 * d * (int)sizeof(float));  // token values per weight buffer
