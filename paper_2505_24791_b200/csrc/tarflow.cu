@@ -18,6 +18,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/tarflow.h"
@@ -514,6 +515,8 @@ static int launch_gemm_f32(tf_model* m, int cls, const float* A, const Matrix& W
 // more SMs matters more than operand reuse.  Rows per thread were chosen by the reads from shared memory that an output costs
 // (sweeps of 64 tokens, width 128: 16 x 32 tiles with 1 / 2 / 4 rows per thread 89.4 / 76.8 / 78.3 us at 4 samples, 32 x 32 tiles with
 // 2 / 4 116 / 104 us at 16; 16 x 16 tiles where 16 x 32 ones would reach half of the SMs at most: 71.6 -> 67.3 us at 4, 62 -> 54 at 1).
+// The head with the update in its epilogue keeps two rows per thread in 32 x 32 tiles (width 32, 256 samples 199.2 us with four, 195.7 with
+// two; width 64 325.2 and 321.6).
 // K % 4 != 0 (an MLP flow of odd dimension) takes the scalar-load kernel.
 template <class T, class Epi>
 static int launch_gemm_simt(tf_model* m, int cls, const T* A, const Matrix& W, int M, const Epi& epi) {
@@ -521,7 +524,8 @@ static int launch_gemm_simt(tf_model* m, int cls, const T* A, const Matrix& W, i
     if (W.K % 4 == 0) {
       auto tiles = [&](int bm, int bn) { return ((M + bm - 1) / bm) * ((W.N + bn - 1) / bn); };
       if (tiles(64, 64) >= 2 * m->num_sms) return launch_gemm_f32<64, 64, 8>(m, cls, A, W, M, epi);
-      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, 4>(m, cls, A, W, M, epi);
+      constexpr int TM32 = std::is_same<Epi, EpiHeadUpdate>::value ? 2 : 4;
+      if (tiles(32, 32) >= m->num_sms) return launch_gemm_f32<32, 32, TM32>(m, cls, A, W, M, epi);
       if (tiles(16, 32) * 2 <= m->num_sms) return launch_gemm_f32<16, 16, 1>(m, cls, A, W, M, epi);
       return launch_gemm_f32<16, 32, 2>(m, cls, A, W, M, epi);
     }
