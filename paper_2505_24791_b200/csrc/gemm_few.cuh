@@ -85,7 +85,6 @@ struct Store {  // bf16(act(x)), and the second term of the pair where map_lo is
         const int j = 8 * k + 2 * i;
         float2 x = fadd2(make_float2(v[j], v[j + 1]), *reinterpret_cast<const float2*>(bias + j));
         if (ACT == ACT_GELU) x = gelu_erf_fast2(x);
-        if (ACT == ACT_RELU) x = make_float2(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f));
         h[i] = pack_bf16(x.x, x.y);
         const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[i]));
         l[i] = pack_bf16(x.x - f.x, x.y - f.y);
@@ -104,22 +103,20 @@ struct Store {  // bf16(act(x)), and the second term of the pair where map_lo is
   }
 };
 
-struct StoreF32 {  // fp32 sums (a K slice's go part_rows rows further down per slice); bias may be absent
+struct StoreF32 {  // fp32 sums, without bias (a K slice's go part_rows rows further down per slice)
   static constexpr int kOld = 1;
   const CUtensorMap* map;
   __device__ __forceinline__ void prefetch() const { prefetch_map(map); }
   template <int CH>
   __device__ __forceinline__ void load(int, int, bool, float (&)[kOld]) const {}
   template <int CH>
-  __device__ __forceinline__ void finish(int row0, int col0, bool, float (&v)[CH], float (&)[kOld], const float* bias, uint8_t* ring, int N, Warp w) const {
+  __device__ __forceinline__ void finish(int row0, int col0, bool, float (&v)[CH], float (&)[kOld], const float*, uint8_t* ring, int N, Warp w) const {
     static_assert(CH == 32, "a box is 32 columns");
     if (col0 >= N) return;
     uint8_t* box = ring + (w.quad * 2 + w.half) * BOX;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float4 b = *reinterpret_cast<const float4*>(bias + 4 * k);
-      *reinterpret_cast<float4*>(box + swz128(w.lane, k)) = make_float4(v[4 * k] + b.x, v[4 * k + 1] + b.y, v[4 * k + 2] + b.z, v[4 * k + 3] + b.w);
-    }
+    for (int k = 0; k < 8; ++k)
+      *reinterpret_cast<float4*>(box + swz128(w.lane, k)) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
     fence_proxy_async_smem();
     __syncwarp();
     if (w.lane == 0) {
@@ -204,12 +201,12 @@ struct HeadUpdate {
   }
 };
 
-// grid: tiles * ksplit; map_w has a box of BN rows; `bounds` (ksplit == 1 only) as in gemm_tc.cuh; `bias` may be null
+// grid: tiles * ksplit; map_w has a box of BN rows; `bias` may be null
 template <int BN, class Epi>
 __global__ void __launch_bounds__(THREADS, 2)
 gemm_few_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_a_lo,
                 const __grid_constant__ CUtensorMap map_w, int M, int N, int K, int split, Epi epi, const float* bias, int* err,
-                int ksplit, int part_rows, const int2* bounds, int ring_bytes) {
+                int ksplit, int part_rows, int ring_bytes) {
   using C = Cfg<BN>;
   constexpr int CH = C::CH;
   extern __shared__ uint8_t smem_few[];
@@ -224,8 +221,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   const int slice = blockIdx.x % ksplit, tile = blockIdx.x / ksplit, tiles_n = (N + BN - 1) / BN;
   const int m0 = tile / tiles_n * BM, n0 = tile % tiles_n * BN;
   const int slabs = (K + BK - 1) / BK;
-  SlabRange sr = {slabs * slice / ksplit, slabs * (slice + 1) / ksplit};
-  if (bounds != nullptr) sr = slab_range(bounds, n0, BN, N, slabs);
+  const SlabRange sr = {slabs * slice / ksplit, slabs * (slice + 1) / ksplit};
   const int n = sr.end - sr.begin;
   const uint32_t w_off = split ? 2u * C::A_BYTES : (uint32_t)C::A_BYTES, stage_bytes = w_off + C::W_BYTES;
   const int nst = ring_bytes / (int)stage_bytes, pre = n < nst ? n : nst;

@@ -484,7 +484,7 @@ static int launch_few(tf_model* m, int cls, const CUtensorMap& ma, const CUtenso
   if (ring < 8 * few::BOX) ring = 8 * few::BOX;  // the epilogue's boxes
   const int tiles = (M + tc::BM - 1) / tc::BM * ((W.N + BN - 1) / BN);
   LAUNCH_PDL(m, cls, kern, tiles * ksplit, few::THREADS, ring + C::EXTRA, ma, ma_lo ? *ma_lo : ma, W.map_few, M, W.N, W.K, ma_lo ? 1 : 0, epi, bias,
-             m->err, ksplit, part_rows, ksplit == 1 ? W.bounds : (const int2*)nullptr, ring);
+             m->err, ksplit, part_rows, ring);
   return check_launch("gemm_few_kernel");
 }
 
@@ -1764,16 +1764,10 @@ static int maf_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
   TF_TRY(check_launch("maf_cast_rows_kernel"));
   if constexpr (sizeof(T) == 2) {
     const CUtensorMap* sm = m->maf_store_maps;
-    if (H % 64 == 0 && few_fits(m, M, bw.w1)) {
-      const CUtensorMap *l0 = hp ? &m->maf_map[0][1] : nullptr, *l1 = hp ? &m->maf_map[1][1] : nullptr;
-      TF_TRY(launch_few<64>(m, KC_GEMM_MLP1, m->maf_map[0][0], l0, bw.w1, M, few::Store<ACT_RELU>{sm + 0, hp ? sm + 1 : nullptr}, bw.b1));
-      TF_TRY(launch_few<64>(m, KC_GEMM_MLP2, m->maf_map[1][0], l1, bw.w2, M, few::Store<ACT_RELU>{sm + 2, hp ? sm + 3 : nullptr}, bw.b2));
-    } else {
-      TF_TRY(gemm<T>(m, KC_GEMM_MLP1, a0, &m->maf_map[0][0], hp ? &m->maf_map[0][1] : nullptr, bw.w1, M,
-                     EpiStoreTma<ACT_RELU>{bw.b1, sm + 0, hp ? sm + 1 : nullptr}));
-      TF_TRY(gemm<T>(m, KC_GEMM_MLP2, h1, &m->maf_map[1][0], hp ? &m->maf_map[1][1] : nullptr, bw.w2, M,
-                     EpiStoreTma<ACT_RELU>{bw.b2, sm + 2, hp ? sm + 3 : nullptr}));
-    }
+    TF_TRY(gemm<T>(m, KC_GEMM_MLP1, a0, &m->maf_map[0][0], hp ? &m->maf_map[0][1] : nullptr, bw.w1, M,
+                   EpiStoreTma<ACT_RELU>{bw.b1, sm + 0, hp ? sm + 1 : nullptr}));
+    TF_TRY(gemm<T>(m, KC_GEMM_MLP2, h1, &m->maf_map[1][0], hp ? &m->maf_map[1][1] : nullptr, bw.w2, M,
+                   EpiStoreTma<ACT_RELU>{bw.b2, sm + 2, hp ? sm + 3 : nullptr}));
   } else {
     TF_TRY(gemm<T>(m, KC_GEMM_MLP1, a0, nullptr, nullptr, bw.w1, M, EpiStore<T, ACT_RELU>{h1, bw.b1, H, h1_lo}));
     TF_TRY(gemm<T>(m, KC_GEMM_MLP2, h1, nullptr, nullptr, bw.w2, M, EpiStore<T, ACT_RELU>{h2, bw.b2, H, h2_lo}));
@@ -1784,8 +1778,7 @@ static int maf_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
     if constexpr (sizeof(T) == 2) {
       // tensor-core engine: the raw (mu, alpha) leave through bulk stores, a row-per-warp kernel applies the update
       // (measured: 381 us for the fused lane-per-column epilogue against 85 + 60 us for the pair on 69 k rows)
-      if (few_fits(m, M, bw.w3)) TF_TRY(launch_few<64>(m, KC_GEMM_HEAD_UPDATE, *map2, map2_lo, bw.w3, M, few::StoreF32{m->maf_store_maps + 4}, bw.b3));
-      else TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, h2, map2, map2_lo, bw.w3, M, EpiStoreF32Tma{bw.b3, m->maf_store_maps + 4}));
+      TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, h2, map2, map2_lo, bw.w3, M, EpiStoreF32Tma{bw.b3, m->maf_store_maps + 4}));
       // Launched early, the update's CTAs crowd onto the SMs that the output layer leaves idle and stay there, which costs more than the
       // kernel boundary once there is something to move (early / not: 1000 rows of 784 values 53.5 / 47.1 us per sweep, 3000 of 2048
       // 125 / 97.5, 100 000 of 256 377 / 362; but 500 rows of 784 43.2 / 43.6, 300 of 2048 51.0 / 51.3, 100 of 256 34.3 / 34.8).
@@ -1881,6 +1874,7 @@ static int upload_f32(tf_model* m, float** dst, const float* src, size_t n) {
 }
 
 // matrix [N, K]: fp32 engine keeps fp32; bf16 engine converts on the device (round to nearest even)
+// few_bn: columns of the narrow tiles (0: the matrix has none)
 static int upload_matrix(tf_model* m, Matrix* W, const float* src, int N, int K, float* staging, int few_bn = 64) {
   W->N = N;
   W->K = K;
@@ -1900,7 +1894,7 @@ static int upload_matrix(tf_model* m, Matrix* W, const float* src, int N, int K,
   W->bn = (N % 256 == 0) ? 256 : 128;
   TF_TRY(make_map_bf16(&W->map_seq, w, (uint64_t)N, (uint64_t)K, 128u));
   W->few_bn = few_bn;
-  TF_TRY(make_map_bf16(&W->map_few, w, (uint64_t)N, (uint64_t)K, (uint32_t)few_bn));
+  if (few_bn > 0) TF_TRY(make_map_bf16(&W->map_few, w, (uint64_t)N, (uint64_t)K, (uint32_t)few_bn));
   return make_map_bf16(&W->map, w, (uint64_t)N, (uint64_t)K, (uint32_t)W->bn);
 }
 
@@ -2312,7 +2306,7 @@ static int maf_load_impl(tf_model* m, const void* blob, size_t nbytes, int D, in
     for (int j = 0; j < H; ++j)
       for (int i = 0; i < D; ++i)
         if (deg_hidden(j) >= i + 1) tmp[(size_t)j * D + (rev ? D - 1 - i : i)] = w1[(size_t)unit[j] * D + i];
-    TF_TRY(upload_matrix(m, &bw.w1, tmp.data(), H, D, staging));
+    TF_TRY(upload_matrix(m, &bw.w1, tmp.data(), H, D, staging, 0));
     TF_TRY(upload_slab_bounds(m, &bw.w1, tmp.data()));
     TF_TRY(upload_sorted(&bw.b1, rd.take(H)));
     const float* w2 = rd.take((size_t)H * H);
@@ -2320,7 +2314,7 @@ static int maf_load_impl(tf_model* m, const void* blob, size_t nbytes, int D, in
     for (int j = 0; j < H; ++j)
       for (int i = 0; i < H; ++i)
         if (deg_hidden(j) >= deg_hidden(i)) tmp[(size_t)j * H + i] = w2[(size_t)unit[j] * H + unit[i]];
-    TF_TRY(upload_matrix(m, &bw.w2, tmp.data(), H, H, staging));
+    TF_TRY(upload_matrix(m, &bw.w2, tmp.data(), H, H, staging, 0));
     TF_TRY(upload_slab_bounds(m, &bw.w2, tmp.data()));
     TF_TRY(upload_sorted(&bw.b2, rd.take(H)));
     // output layer [mu | alpha] -> interleaved rows (2 i, 2 i + 1) = (mu_i, alpha_i) in the sample's own order
@@ -2337,7 +2331,7 @@ static int maf_load_impl(tf_model* m, const void* blob, size_t nbytes, int D, in
       btmp[2 * r] = b3[i];
       btmp[2 * r + 1] = b3[D + i];
     }
-    TF_TRY(upload_matrix(m, &bw.w3, tmp.data(), 2 * D, H, staging));
+    TF_TRY(upload_matrix(m, &bw.w3, tmp.data(), 2 * D, H, staging, 0));
     TF_TRY(upload_slab_bounds(m, &bw.w3, tmp.data()));
     TF_TRY(upload_f32(m, &bw.b3, btmp.data(), btmp.size()));
   }
