@@ -266,7 +266,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       tmem_ld_wait();
       tcgen05_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));  // release on the leader's barrier
+      if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));  // relaxed: the tensor-memory reads above are complete and fenced
       if (row0 < M) {
 #pragma unroll
         for (int g = 0; g < NCH / CPG; ++g) {

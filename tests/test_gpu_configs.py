@@ -232,11 +232,11 @@ def test_long_sequence_full_size_properties():
 # ---------------------------------------------------------------- sweeps over few rows (K-split residual projections)
 @pytest.mark.parametrize("name", ["cfg2", "cfg3"])
 def test_few_row_sweeps_agree_with_the_one_shape_path_and_the_oracle(name, monkeypatch):
-    """Sweeps of up to 1024 rows run on 128 x 128 tiles with the residual projections cut into K slices that the next
-    LayerNorm adds; up to 4096 rows the pair tiles are cut.  Batches 1 (256 rows, 8 slices at width 1024 / 4 at 512),
-    3 (768 rows), 5 (1280 rows: pair tiles, 3 to 6 slices) and 8 (2048 rows) against the oracle, and against
-    the same library with both paths switched off (every sweep on one tile shape, reduce-add epilogue).  The forward
-    direction takes the same path."""
+    """Sweeps over few rows run on 128 x 64 tiles where those fit the GPU at once, else (up to 1024 rows) on 128 x 128 tiles; the
+    residual projections are cut into K slices that the next LayerNorm adds, up to 4096 rows on pair tiles too.  Batches 1 (256
+    rows: narrow tiles, 4 slices at width 1024), 3 (768 rows: narrow and 128 x 128 tiles), 5 (1280 rows: narrow and pair tiles) and
+    8 (2048 rows) against the oracle, and against the same library with both paths switched off (every sweep on one tile
+    shape, reduce-add epilogue).  The forward direction takes the same path."""
     cfg = synth.config(name, n_blocks=2, n_layers=2)
     L = synth.seq_len(cfg)
     lab_of = (lambda B: synth.make_labels(cfg, B=B)) if cfg.get("n_classes", 0) else (lambda B: None)
@@ -329,8 +329,8 @@ def test_long_sequence_forward_cuts_a_sample_over_ctas(long_model):
     m = long_model
     x = synth.make_latents(m.cfg, 5400, B=3)
     zf, ld = m.forward(x, None)
-    z1, l1 = m.forward(x[2:], None)                                 # neither values nor the sum's order depend on the batch
-    assert np.array_equal(zf[2:], z1) or rel_l2(zf[2:], z1) <= 1e-3  # (tile shapes of the products do, at the level of bf16)
+    z1, l1 = m.forward(x[2:], None)                                 # tile shapes of the products depend on the batch, at the level of bf16
+    assert rel_l2(zf[2:], z1) <= 1e-3
     assert abs(l1[0] - ld[2]) <= 1e-3 * max(1.0, abs(ld[2]))
     zo, ldo = O.model_forward(m.blocks, x[:1].astype(np.float64), None, m.cfg)
     _close(zf[:1], zo)

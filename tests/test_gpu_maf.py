@@ -206,3 +206,27 @@ def test_fp32_sample_does_not_depend_on_the_batch():
             zp, lp = m.forward(z[pick])
             assert np.array_equal(xp, x[pick]) and np.array_equal(itp, its[:, pick]), pick
             assert np.array_equal(zp, zf[pick]) and np.array_equal(lp, ld[pick]), pick
+
+
+def test_non_finite_sample_stays_its_own_and_reaches_no_earlier_slab():
+    """Units are sorted by degree and the products leave out the k slabs a column group has no weight in, so a value that is
+    not finite spoils its own sample only, and there nothing of the positions whose slabs all lie before it.  Which
+    slabs a column group takes depends on the matrix alone: one-CTA tiles (10 rows) and pair tiles (600 rows) agree bit for bit."""
+    cfg = synth.maf_config("maf_ising", n_blocks=1)                   # 256 dimensions, 1024 units, about four per degree
+    with Maf(cfg, 600) as m:
+        x = synth.make_maf_latents(cfg, 26, B=600)
+        clean, ld_clean = m.forward(x)
+        x[3, 200], x[5, 255] = np.nan, np.inf                         # 200: a hidden slab of degrees above 192, outputs from 128 on
+        z, ld = m.forward(x)
+        others = [b for b in range(600) if b not in (3, 5)]
+        assert np.array_equal(z[others], clean[others]) and np.array_equal(ld[others], ld_clean[others])
+        assert np.array_equal(z[3, :128], clean[3, :128]) and np.isnan(z[3, 200])
+        assert np.array_equal(z[5, :128], clean[5, :128]) and not np.isfinite(z[5, 255])
+        zs, lds = m.forward(x[:10])
+        assert np.array_equal(zs, z[:10], equal_nan=True) and np.array_equal(lds, ld[:10], equal_nan=True)
+        for bad in (x[3:4], x[5:6]):
+            with pytest.raises(binding.TarflowError) as e:            # Jacobi decoding reports it
+                m.jacobi(bad, cfg["tau"], m.D + 1)
+            assert e.value.code == binding.TF_ENONFINITE
+        y, _, _, rc = m.jacobi(clean[:4].astype(np.float32), cfg["tau"], m.D + 1)
+        assert rc == 0 and np.isfinite(y).all()
