@@ -1781,8 +1781,9 @@ static int maf_pass(tf_model* m, int g, int n_slots, const float* u_src, const i
       TF_TRY(gemm<T>(m, KC_GEMM_HEAD_UPDATE, h2, map2, map2_lo, bw.w3, M, EpiStoreF32Tma{bw.b3, m->maf_store_maps + 4}));
       // Launched early, the update's CTAs crowd onto the SMs that the output layer leaves idle and stay there, which costs more than the
       // kernel boundary once there is something to move (early / not: 1000 rows of 784 values 53.5 / 47.1 us per sweep, 3000 of 2048
-      // 125 / 97.5, 100 000 of 256 377 / 362; but 500 rows of 784 43.2 / 43.6, 300 of 2048 51.0 / 51.3, 100 of 256 34.3 / 34.8).
-      if (only_col < 0 && (int64_t)M * D >= 512 * 1024)
+      // 125 / 97.5, 100 000 of 256 378 / 362; but 500 rows of 784 43.2 / 43.6, 300 of 2048 51.0 / 51.3, 100 of 256 34.3 / 34.8).  Short rows
+      // are done before it matters (20 000 rows of 64: 45.0 / 47.2, 100 000: 107 / 107).
+      if (only_col < 0 && (int64_t)M * D >= (D >= 256 ? 512 * 1024 : 4 * 1024 * 1024))
         LAUNCH(m, KC_AFFINE, maf_update_kernel, (M + 7) / 8, 256, 0, m->o, v, u_upd, m->maxdiff, idx, M, D, only_col);
       else
         LAUNCH_PDL(m, KC_AFFINE, maf_update_kernel, (M + 7) / 8, 256, 0, m->o, v, u_upd, m->maxdiff, idx, M, D, only_col);
