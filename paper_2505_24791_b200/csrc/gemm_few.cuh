@@ -9,8 +9,8 @@
 //     do not cover the latency: two-term sweep of 256 rows, width 1024: 525 us with 2 slabs, 414 with 3, 418 with 4);
 //   * a weight slab is fetched once for both terms of a pair;
 //   * eight warps share the epilogue (bulk stores, as in epilogue.cuh).
-// 256 rows, width 1024, eight layers (128 x 128 tiles of gemm_tc.cuh -> these): single-term sweep 385 -> 335 us, two-term 522 -> 414;
-// 1053 rows, width 256, two layers: 155 -> 85 and 167 -> 88 us.
+// 256 rows, width 1024, eight layers (128 x 128 tiles of gemm_tc.cuh -> these): single-term sweep 387 -> 333 us, two-term 523 -> 413;
+// 1053 rows, width 256, two layers: 144 -> 76 and 164 -> 84 us.
 // A split of K over the CTAs of a cluster with an exchange through distributed shared memory was slower (429 and 555 us): two CTAs
 // take 1.8 us for the exchange and save 1.2 us of loads, eight take 2.7 us.
 // Every wait is bounded as in gemm_tc.cuh.
